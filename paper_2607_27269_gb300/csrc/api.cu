@@ -434,10 +434,12 @@ mla_status gqa_as_mla(const mla_gqa_dims *g, mla_dims *d)
     return MLA_OK;
 }
 
-int gqa_splits(const mla_gqa_dims *g, int batch, int max_kv_len, int requested, int sms)
+int gqa_splits(const mla_gqa_dims *g, int batch, int q_len, int max_kv_len, int requested, int sms)
 {
     if (requested > 0) return requested;
-    int64_t s = sms;  // one CTA per SM
+    // as many partitions (warps) as the SMs hold at a time, each shared by the row groups
+    int64_t s = static_cast<int64_t>(sms) * kGqaPartsPerSm /
+                gqa_row_groups(q_len * (g->num_heads / g->num_kv_groups), g->head_dim);
     const int64_t tiles = static_cast<int64_t>(batch) * g->num_kv_groups * ((max_kv_len + MLA_SPLIT_TILE - 1) / MLA_SPLIT_TILE);
     if (s > tiles) s = tiles;
     if (s < 1) s = 1;
@@ -476,7 +478,7 @@ mla_status mla_gqa_workspace_size(const mla_gqa_dims *dims, int32_t batch, int32
     if (q_len * (dims->num_heads / dims->num_kv_groups) > 128) return MLA_ERR_UNSUPPORTED;
     int sms = 0;
     if ((s = device_info(nullptr, &sms)) != MLA_OK) return s;
-    const int S = gqa_splits(dims, batch, max_kv_len, num_splits, sms);
+    const int S = gqa_splits(dims, batch, q_len, max_kv_len, num_splits, sms);
     const size_t units = static_cast<size_t>(batch) * dims->num_kv_groups;
     const size_t slots = units > 0 ? units + S - 1 : 0;
     const size_t rows = static_cast<size_t>(q_len) * (dims->num_heads / dims->num_kv_groups);
@@ -513,7 +515,7 @@ mla_status mla_gqa_decode_attn(const mla_gqa_dims *dims, const mla_cache *cache,
     g.hpg = hpg;
     g.head_dim = dims->head_dim;
     g.max_kv = max_kv_len;
-    g.num_splits = gqa_splits(dims, batch, max_kv_len, num_splits, sms);
+    g.num_splits = gqa_splits(dims, batch, q_len, max_kv_len, num_splits, sms);
     g.sm_scale = dims->sm_scale;
     g.rope_style = dims->rope_style;
     g.rope_base = dims->rope_base;
@@ -523,6 +525,7 @@ mla_status mla_gqa_decode_attn(const mla_gqa_dims *dims, const mla_cache *cache,
     g.lse_part = lse_part;
     g.status = status;
     g.cache = v;
+    g.sms = sms;
     const cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e = launch_gqa_attn(g, st);
     if (e != cudaSuccess) return from_cuda(e);

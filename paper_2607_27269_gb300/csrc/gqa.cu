@@ -5,19 +5,26 @@
 // position) and value cache V; unit u = b * G + g is one such (sequence,
 // group), with kv_len[b] tokens.
 //
-// One CTA = one split-KV partition of the units' 128-token tiles (the same
-// partition as the MLA path, over units instead of sequences), 256 threads:
-//   warp 0      TMA producer: the K tile of every tile into the K ring, the V
-//               tile into the V ring (each read once from HBM);
-//   warp 1      MMA issuer: S[rows, 128 tok] = Q K^T into one of two TMEM
-//               buffers, O[rows, d] += P V into TMEM;
-//   warps 4..7  one thread per query row (row r = position i * hpg + head hh
-//               of the group): stages the rotated queries of each unit,
-//               runs the online softmax of its row (lazy rescaling), writes
-//               its row of P, and at the end of a unit writes its partial.
-// The rows of a unit (q_len * hpg <= 128) fill the MMA's M = 128; rows past
-// them are padding.  Every wait is bounded; a timeout is recorded in the
-// status word and the CTA winds down.
+// The kernel is bound by the cache bytes: a unit has only q_len * H/G query
+// rows (3 .. 56 in the draft shapes), so the tensor work is a few percent of
+// the pipe, and what has to be hidden is the chain load -> scores -> softmax ->
+// values.  One warp is one split-KV partition (the MLA path's partition, over
+// the units' 128-token tiles): it keeps its own ring of TMA stages, issues its
+// own loads and never waits on another warp, so that the SM's seven warps hide
+// each other's chains and the ring keeps 224 KB per SM in flight or in use.
+// Within a warp everything between the cache stage and the partial stays in
+// registers (mma.m16n8k16, tokens on M, query rows on N in steps of 8):
+//   S^T[16 tok, N]  = K (ldmatrix) x Q^T (fragments loaded and rotated once a unit)
+//   P^T             = 2^(S^T scale - m) rounded to bf16, transposed 8 x 8 by movmatrix
+//   O^T[D, N]      += V^T (ldmatrix.trans) x P^T
+// A column's running maximum, sum and accumulators sit in the same lanes, so
+// a rescale (only when a score passes the base by 2^8) needs no exchange.
+// More than 32 rows run as row groups (grid y) that each read the cache.
+//
+// The first form of this kernel (one CTA per partition, tcgen05 with M = 128
+// query rows of which 20 are real, one softmax warp) took 727 us on the
+// 128-sequence paged batch (20 rows of 64) and 231 us on eight long sequences
+// (3 rows of 128): the serial TMEM round trips per tile set the pace.
 #include <cudaTypedefs.h>
 
 #include "common.cuh"
@@ -27,14 +34,15 @@
 namespace gbmla {
 namespace {
 
-constexpr int kGqaThreads = 256;
-constexpr int kTokTile = MLA_SPLIT_TILE;  // 128 tokens per tile
-constexpr int kSmBase = 128;              // first softmax thread (warp 4)
-constexpr int kMaxRing = 8;
+constexpr int kTokTile = MLA_SPLIT_TILE;  // 128 tokens per tile of the partition
+constexpr int kPage = 64;
+constexpr int kStageBytes = 16384;        // K and V of one stage: 64 tokens of width 64, 32 of width 128
+constexpr int kStages = 2;                // per warp
+constexpr int kWarps = kGqaPartsPerSm;    // 7 warps x 2 stages x 16 KB of shared memory
 
 struct GqaArgs {
     int batch, q_len, groups, hpg, rows, max_kv, num_splits;
-    int paged, bt_stride, num_pages, nk, nv;  // nk / nv: K / V ring slots
+    int paged, bt_stride, num_pages;
     float scale_log2;
     int style;
     const int32_t *kv_len;
@@ -45,63 +53,6 @@ struct GqaArgs {
     RopeTurns turns;
 };
 
-struct __align__(8) GqaBars {
-    uint64_t k_full[kMaxRing], k_empty[kMaxRing], v_full[kMaxRing], v_empty[kMaxRing];
-    uint64_t s_full[2], s_free[2], p_full, pv_done, q_full;
-};
-
-// Units [u0, ..) and their tiles, walked in the partition's order.
-struct UnitWalk {
-    const int32_t *kv;
-    int groups, q_len, max_kv, batch;
-    int u;             // current unit
-    int64_t start, nb; // first flat tile of the unit, its tile count
-    int64_t t, t_end;
-    __device__ void init(const int32_t *kv_len, int groups_, int q_len_, int max_kv_, int units, int64_t tb,
-                         int64_t te)
-    {
-        kv = kv_len;
-        groups = groups_;
-        q_len = q_len_;
-        max_kv = max_kv_;
-        batch = units;
-        t = tb;
-        t_end = te;
-        start = 0;
-        nb = 0;
-        for (u = 0; u < units; ++u) {
-            nb = seq_tiles(kv[u / groups], q_len, max_kv);
-            if (start + nb > t) break;
-            start += nb;
-        }
-    }
-    __device__ int tile() const { return static_cast<int>(t - start); }
-    __device__ bool first(int64_t tb) const { return t == tb || t == start; }
-    __device__ bool last() const { return t + 1 == t_end || t + 1 == start + nb; }
-    __device__ void next()
-    {
-        ++t;
-        if (t < t_end && t >= start + nb) {
-            start += nb;
-            for (++u; u < batch; ++u) {
-                nb = seq_tiles(kv[u / groups], q_len, max_kv);
-                if (nb > 0) break;
-            }
-        }
-    }
-};
-
-__device__ __forceinline__ bool wait_all(uint64_t *bar, uint32_t parity)
-{
-    return __all_sync(0xffffffffu, mbar_wait(smem_u32(bar), parity, kWaitLimitNs));
-}
-
-// byte offset of 16-byte chunk j of row r in a 128-row SW128 K-major atom
-__device__ __forceinline__ uint32_t sw128(int r, int j)
-{
-    return static_cast<uint32_t>((r >> 3) * 1024 + (r & 7) * 128 + ((j ^ (r & 7)) << 4));
-}
-
 __device__ __forceinline__ float ex2(float x)
 {
     float y;
@@ -109,387 +60,404 @@ __device__ __forceinline__ float ex2(float x)
     return y;
 }
 
-// Query row r of the unit, rotated to position pos (RoPE over the whole head,
-// fp32), into the SW128 K-major Q tile; a null src writes a zero row (padding).
-template <int D>
-__device__ __forceinline__ void stage_query(unsigned char *q_buf, int r, const uint16_t *src, int64_t pos, int style,
-                                            const RopeTurns &turns)
+__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4])
 {
-    float x[D];
-    if (src) {
-#pragma unroll
-        for (int v = 0; v < D / 8; ++v) {
-            const uint4 raw = reinterpret_cast<const uint4 *>(src)[v];
-            const uint32_t wd[4] = {raw.x, raw.y, raw.z, raw.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                x[8 * v + 2 * e] = __uint_as_float(wd[e] << 16);
-                x[8 * v + 2 * e + 1] = __uint_as_float(wd[e] & 0xffff0000u);
-            }
-        }
-        if (style == 0) {
-#pragma unroll
-            for (int k = 0; k < D / 2; ++k) {
-                float cs, sn;
-                rope_cos_sin(pos, turns.f[k], &cs, &sn);
-                const float a0 = x[k], a1 = x[k + D / 2];
-                x[k] = a0 * cs - a1 * sn;
-                x[k + D / 2] = a1 * cs + a0 * sn;
-            }
-        } else {
-#pragma unroll
-            for (int k = 0; k < D / 2; ++k) {
-                float cs, sn;
-                rope_cos_sin(pos, turns.f[k], &cs, &sn);
-                const float a0 = x[2 * k], a1 = x[2 * k + 1];
-                x[2 * k] = a0 * cs - a1 * sn;
-                x[2 * k + 1] = a1 * cs + a0 * sn;
-            }
-        }
-    } else {
-#pragma unroll
-        for (int e = 0; e < D; ++e) x[e] = 0.f;
-    }
-#pragma unroll
-    for (int at = 0; at < D / 64; ++at)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            uint32_t wd[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const __nv_bfloat162 h2 = __floats2bfloat162_rn(x[64 * at + 8 * j + 2 * e], x[64 * at + 8 * j + 2 * e + 1]);
-                wd[e] = *reinterpret_cast<const uint32_t *>(&h2);
-            }
-            *reinterpret_cast<uint4 *>(q_buf + at * 128 * 128 + sw128(r, j)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-        }
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
 }
 
-template <int D>
-__global__ void __launch_bounds__(kGqaThreads) gqa_attn_kernel(const __grid_constant__ GqaArgs a,
-                                                              const __grid_constant__ CUtensorMap map_k,
-                                                              const __grid_constant__ CUtensorMap map_v)
+__device__ __forceinline__ void ldsm4_trans(uint32_t addr, uint32_t (&r)[4])
 {
-    constexpr int KA = D / 64;                  // 64-column atoms of a K or V tile
-    constexpr uint32_t kTileBytes = kTokTile * D * 2;
-    constexpr uint32_t kAtom = 128 * 128;       // 128 rows x 64 columns bf16
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+
+__device__ __forceinline__ uint32_t mov_trans(uint32_t x)
+{
+    uint32_t y;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
+    return y;
+}
+
+__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2])
+{
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
+{
+    const __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
+    return *reinterpret_cast<const uint32_t *>(&h2);
+}
+
+// The warp's place in its partition: a segment is the partition's run of
+// tokens [tok, tok_end) of unit u; stages cut it into TOK tokens each.  All
+// members are the same in every lane.
+struct Segments {
+    int b, g, kv, tok, tok_end;
+    int64_t left;  // tiles of the partition not yet in a segment
+
+    // Tile t (of the flat list of all units' tiles) and n tiles from it on.
+    __device__ void init(const GqaArgs &a, int64_t t, int64_t n, int lane)
+    {
+        left = n;
+        int64_t before = 0;  // tiles of the sequences before the 32 looked at
+        for (int b0 = 0;; b0 += 32) {
+            const int bb = b0 + lane;
+            const int64_t nb = bb < a.batch ? seq_tiles(a.kv_len[bb], a.q_len, a.max_kv) * a.groups : 0;
+            int64_t incl = nb;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const unsigned hit = __ballot_sync(0xffffffffu, before + incl > t);
+            if (hit || b0 + 32 >= a.batch) {
+                const int src = hit ? __ffs(hit) - 1 : 31;
+                b = b0 + src;
+                const int64_t at = t - before - __shfl_sync(0xffffffffu, incl - nb, src);  // tile within the sequence
+                kv = a.kv_len[b];
+                const int nt = static_cast<int>(seq_tiles(kv, a.q_len, a.max_kv));
+                g = static_cast<int>(at / nt);
+                open(static_cast<int>(at - static_cast<int64_t>(g) * nt), nt);
+                return;
+            }
+            before += __shfl_sync(0xffffffffu, incl, 31);
+        }
+    }
+    // The segment from tile j of the current unit, which has nt tiles.
+    __device__ void open(int j, int nt)
+    {
+        const int n = static_cast<int>(min(static_cast<int64_t>(nt - j), left));
+        left -= n;
+        tok = j * kTokTile;
+        tok_end = min((j + n) * kTokTile, kv);
+    }
+    __device__ bool more() const { return tok < tok_end; }
+    // The next stage's tokens; at a segment's end the next unit's segment
+    // (none is left when more() is false then).
+    __device__ void next(const GqaArgs &a, int step)
+    {
+        tok += step;
+        if (tok >= tok_end && left > 0) {
+            if (++g == a.groups) {
+                g = 0;
+                do {  // (a length that cannot be served holds no tiles)
+                    ++b;
+                    kv = a.kv_len[b];
+                } while (seq_tiles(kv, a.q_len, a.max_kv) == 0);
+            }
+            open(0, static_cast<int>(seq_tiles(kv, a.q_len, a.max_kv)));
+        }
+    }
+};
+
+// D: head width.  N: query rows of a row group, rounded up to 8.
+template <int D, int N>
+__global__ void __launch_bounds__(32 * kWarps, 1)
+    gqa_attn_kernel(const __grid_constant__ GqaArgs a, const __grid_constant__ CUtensorMap map_k,
+                    const __grid_constant__ CUtensorMap map_v)
+{
+    constexpr int KA = D / 64;                       // 64-column atoms of a row
+    constexpr int TOK = kStageBytes / (4 * D);       // tokens per stage
+    constexpr int NJ = N / 8;                        // 8-row column blocks
+    constexpr int TB = D == 64 || N <= 16 ? 32 : 16; // tokens scored together (by registers)
+    constexpr uint32_t kAtom = TOK * 128;            // TOK rows x 64 columns, 128-byte swizzle
     extern __shared__ __align__(1024) unsigned char smem_raw[];
-    __shared__ GqaBars bars;
-    __shared__ uint32_t tmem_base;
-    __shared__ int64_t red64[64];
-    __shared__ int abort_flag;
-    unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
-                                                            ~static_cast<uintptr_t>(1023));
-    unsigned char *q_buf = smem;                       // KA atoms: Q [128 rows, D]
-    unsigned char *p_buf = q_buf + KA * kAtom;         // 2 atoms: P [128 rows, 128 tokens]
-    unsigned char *k_ring = p_buf + 2 * kAtom;         // nk tiles
-    unsigned char *v_ring = k_ring + a.nk * kTileBytes; // nv tiles
+    __shared__ __align__(8) uint64_t bars[kWarps][kStages];
+    __shared__ int64_t red64[32];
+    __shared__ uint64_t turns[64];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int part = blockIdx.y;
-    const int units = a.batch * a.groups;
-    const int nw = (a.rows + 31) / 32;  // softmax warps holding real rows
-
     if (tid == 0) {
-        for (int s = 0; s < kMaxRing; ++s) {
-            mbar_init(&bars.k_full[s], 1);
-            mbar_init(&bars.k_empty[s], 1);
-            mbar_init(&bars.v_full[s], 1);
-            mbar_init(&bars.v_empty[s], 1);
-        }
-        for (int j = 0; j < 2; ++j) {
-            mbar_init(&bars.s_full[j], 1);
-            mbar_init(&bars.s_free[j], nw);
-        }
-        mbar_init(&bars.p_full, nw);
-        mbar_init(&bars.pv_done, 1);
-        mbar_init(&bars.q_full, nw);
-        abort_flag = 0;
+        for (int w = 0; w < kWarps; ++w)
+            for (int s = 0; s < kStages; ++s) mbar_init(&bars[w][s], 1);
         tc::fence_barrier_init();
+        tc::prefetch_tensormap(&map_k);
+        tc::prefetch_tensormap(&map_v);
     }
-    if (warp == 1) {
-        tc::tmem_alloc(smem_u32(&tmem_base), 512);
-        tc::tmem_relinquish();
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-    tc::fence_after_sync();
+    for (int k = tid; k < D / 2; k += 32 * kWarps) turns[k] = a.turns.f[k];
     // the cache is final when this kernel runs (a cache writer releases its
-    // dependents only on completion); the queries come from the previous
-    // launch: the softmax warps wait before they read them
+    // dependents only on completion); the queries and the partial buffers
+    // belong to the previous launches: a warp waits before it reads queries
     griddep_launch_dependents();
-    const int64_t T = block_tile_sum(a.kv_len, units, a.q_len, a.max_kv, red64, a.groups);
-    const int64_t t_begin = T ? part_begin(part, T, a.num_splits) : 0;
-    const int64_t t_end = T ? part_begin(part + 1, T, a.num_splits) : 0;
-    const int n_items = static_cast<int>(t_end - t_begin);
-    const uint32_t tmem = tmem_base;
-    auto fail = [&]() {
-        record_status(a.status, kStatusTimeout);
-        abort_flag = 1;
-    };
-
-    if (warp == 0 && n_items > 0) {
-        // ================================================================ TMA producer
-        if (lane == 0) {
-            tc::prefetch_tensormap(&map_k);
-            tc::prefetch_tensormap(&map_v);
-        }
-        UnitWalk w;
-        w.init(a.kv_len, a.groups, a.q_len, a.max_kv, units, t_begin, t_end);
-        for (int it = 0; it < n_items; ++it, w.next()) {
-            // where the tile lives: one 128-row box (contiguous) or a 64-row box per page
-            const int u = w.u, j = w.tile();
-            int nh = 1;
-            int32_t blk[2] = {u, 0}, tok0[2] = {j * kTokTile, 0};
-            if (a.paged) {
-                const int kv = a.kv_len[u / a.groups];
-                nh = kv - j * kTokTile > 64 ? 2 : 1;
-                for (int h = 0; h < nh; ++h) {
-                    const int32_t pg = a.block_table[static_cast<int64_t>(u) * a.bt_stride + 2 * j + h];
-                    if (pg < 0 || pg >= a.num_pages) {
-                        if (lane == 0) record_status(a.status, kStatusBounds);
-                        nh = h;
-                        break;
-                    }
-                    blk[h] = pg;
-                    tok0[h] = 0;
-                }
-            }
-            const uint32_t bytes = static_cast<uint32_t>(nh) * (a.paged ? 64u : 128u) * D * 2;
-            for (int kind = 0; kind < 2; ++kind) {  // K, then V
-                const int ring = kind == 0 ? a.nk : a.nv;
-                const int s = it % ring, round = it / ring;
-                uint64_t *empty = kind == 0 ? &bars.k_empty[s] : &bars.v_empty[s];
-                uint64_t *full = kind == 0 ? &bars.k_full[s] : &bars.v_full[s];
-                if (round > 0 && !wait_all(empty, (round - 1) & 1)) {
-                    if (lane == 0) fail();
-                    it = n_items;
-                    break;
-                }
-                if (lane == 0) {
-                    const uint32_t dst = smem_u32((kind == 0 ? k_ring : v_ring) + s * kTileBytes);
-                    const CUtensorMap *map = kind == 0 ? &map_k : &map_v;
-                    // (the arrive completes the phase at once when a bad page left nothing to load)
-                    tc::mbar_arrive_expect_tx(smem_u32(full), bytes);
-                    for (int at = 0; at < KA; ++at)
-                        for (int h = 0; h < nh; ++h)
-                            tc::tma_load_3d(dst + at * kAtom + h * 64 * 128, map, 64 * at, tok0[h], blk[h],
-                                            smem_u32(full));
-                }
-                __syncwarp();
-            }
-        }
-    } else if (warp == 1 && n_items > 0) {
-        // ================================================================ MMA issuer
-        const uint32_t idesc_qk = tc::idesc_bf16_f32(128, 128, false, false);
-        const uint32_t idesc_pv = tc::idesc_bf16_f32(128, D, false, true);
-        const uint64_t d_k = tc::smem_desc(0, 16, 1024, tc::kSwizzle128B);           // K-major operands
-        const uint64_t d_v = tc::smem_desc(0, kAtom, 1024, tc::kSwizzle128B);        // V: N-major
-        auto with_addr = [](uint64_t tmpl, uint32_t saddr) {
-            return tmpl | static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
-        };
-        const uint32_t q_base = smem_u32(q_buf), p_base = smem_u32(p_buf);
-        const uint32_t o_tmem = tmem + 256;  // S buffers at columns [0, 128) and [128, 256)
-        UnitWalk w;
-        w.init(a.kv_len, a.groups, a.q_len, a.max_kv, units, t_begin, t_end);
-        bool ok = true;
-        int seq = 0;  // units begun (q_full phases)
-        auto qk = [&](int it) {
-            const int s = it % a.nk;
-            if (it >= 2) ok = ok && wait_all(&bars.s_free[it & 1], ((it - 2) >> 1) & 1);
-            ok = ok && wait_all(&bars.k_full[s], (it / a.nk) & 1);
-            if (!ok) return;
-            tc::fence_after_sync();
-            const uint32_t kb = smem_u32(k_ring + s * kTileBytes);
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-                const uint32_t off = (kk >> 2) * kAtom + (kk & 3) * 32;
-                tc::mma_bf16_elect(tmem + (it & 1) * 128, with_addr(d_k, q_base + off), with_addr(d_k, kb + off),
-                                   idesc_qk, kk > 0);
-            }
-            tc::commit_elect(smem_u32(&bars.k_empty[s]));
-            tc::commit_elect(smem_u32(&bars.s_full[it & 1]));
-        };
-        auto pv = [&](int it, bool first, int u, int j) {
-            const int s = it % a.nv;
-            ok = ok && wait_all(&bars.p_full, it & 1);
-            ok = ok && wait_all(&bars.v_full[s], (it / a.nv) & 1);
-            if (!ok) return;
-            tc::fence_after_sync();
-            // value rows at or past the unit's end (never loaded, or past kv_len)
-            // may hold anything; their weights are 0, and 0 x NaN is NaN: zero them
-            const int valid = min(a.kv_len[u / a.groups] - j * kTokTile, kTokTile);
-            if (valid < kTokTile) {
-                unsigned char *vt = v_ring + s * kTileBytes;
-                for (int at = 0; at < KA; ++at)
-                    for (int rr = valid + lane; rr < kTokTile; rr += 32)
-#pragma unroll
-                        for (int ch = 0; ch < 8; ++ch)
-                            *reinterpret_cast<uint4 *>(vt + at * kAtom + (rr >> 3) * 1024 + (rr & 7) * 128 + ch * 16) =
-                                make_uint4(0u, 0u, 0u, 0u);
-                tc::fence_proxy_async_smem();
-                __syncwarp();
-            }
-            const uint32_t vb = smem_u32(v_ring + s * kTileBytes);
-#pragma unroll
-            for (int kk = 0; kk < kTokTile / 16; ++kk) {
-                const uint32_t pa = p_base + (kk >> 2) * kAtom + (kk & 3) * 32;
-                tc::mma_bf16_elect(o_tmem, with_addr(d_k, pa), with_addr(d_v, vb + kk * 16 * 128), idesc_pv,
-                                   !(first && kk == 0));
-            }
-            tc::commit_elect(smem_u32(&bars.v_empty[s]));
-            tc::commit_elect(smem_u32(&bars.pv_done));
-        };
-        // QK(t + 1) goes ahead of PV(t) within a unit; at a unit boundary PV(t)
-        // goes first (the next unit's queries are staged after this unit's end)
-        ok = wait_all(&bars.q_full, 0);
-        seq = 1;
-        if (ok) qk(0);
-        for (int it = 0; it < n_items && ok; ++it) {
-            const bool first = w.first(t_begin), last = w.last();
-            const int u = w.u, j = w.tile();
-            if (!last && it + 1 < n_items) qk(it + 1);
-            pv(it, first, u, j);
-            w.next();
-            if (last && it + 1 < n_items && ok) {
-                ok = wait_all(&bars.q_full, seq & 1);
-                ++seq;
-                if (ok) qk(it + 1);
-            }
-        }
-        if (!ok && lane == 0) fail();
-    } else if (warp >= 4 && warp < 4 + nw) {
-        // ================================================================ softmax / epilogue
-        // (only the warps holding real rows: nw = ceil(rows / 32))
-        griddep_wait();  // the queries come from the previous launch
-        const int r = tid - kSmBase;                 // query row = TMEM lane
-        const int qq = warp & 3;                     // lane quarter
-        const uint32_t lane_addr = tmem + (static_cast<uint32_t>(qq * 32) << 16);
-        const bool row_ok = r < a.rows;
-        const int i = r / a.hpg, hh = r % a.hpg;     // query position and head in the group
-        UnitWalk w;
-        w.init(a.kv_len, a.groups, a.q_len, a.max_kv, units, t_begin, t_end);
-        float m_used = -INFINITY, l = 0.f;
-        bool ok = true;
-        int64_t pos = 0;  // this row's query position in the current unit
-        for (int it = 0; it < n_items && ok; ++it, w.next()) {
-            const int u = w.u, b = u / a.groups, g = u % a.groups;
-            const int kv = a.kv_len[b];
-            if (w.first(t_begin)) {
-                // ---- stage the unit's rotated queries: row r = (i, hh), head g * hpg + hh
-                pos = static_cast<int64_t>(kv) - a.q_len + i;
-                const uint16_t *src =
-                    a.q + ((static_cast<int64_t>(b) * a.q_len + i) * (a.groups * a.hpg) + g * a.hpg + hh) * D;
-                stage_query<D>(q_buf, r, row_ok ? src : nullptr, pos, a.style, a.turns);
-                tc::fence_proxy_async_smem();
-                __syncwarp();
-                tc::mbar_arrive_elect(smem_u32(&bars.q_full));
-                m_used = -INFINITY;
-                l = 0.f;
-            }
-            // ---- scores of tile it: pass 1 the row maximum, pass 2 the weights
-            ok = wait_all(&bars.s_full[it & 1], (it >> 1) & 1);
-            if (!ok) break;
-            tc::fence_after_sync();
-            const uint32_t s_addr = lane_addr + (it & 1) * 128;
-            // causal mask and the tile's tail: token t0 + c is visible iff <= pos and < kv
-            const int64_t t0 = static_cast<int64_t>(w.tile()) * kTokTile;
-            const int vis = row_ok ? static_cast<int>(min(pos + 1, static_cast<int64_t>(kv)) - t0) : 0;
-            float mx = -INFINITY;
-#pragma unroll 1
-            for (int c = 0; c < kTokTile; c += 16) {
-                uint32_t v[16];
-                tc::ld_32x32b_x16(s_addr + c, v);
-                tc::wait_ld();
-#pragma unroll
-                for (int e = 0; e < 16; ++e)
-                    if (c + e < vis) mx = fmaxf(mx, __uint_as_float(v[e]));
-            }
-            mx = mx == -INFINITY ? mx : mx * a.scale_log2;
-            const bool over = row_ok && mx != -INFINITY && (m_used == -INFINITY || mx > m_used + 8.f);
-            float alpha = 1.f;
-            if (over) {
-                alpha = m_used == -INFINITY ? 0.f : ex2(m_used - mx);
-                m_used = mx;
-                l *= alpha;
-            }
-            // P(it) overwrites P(it - 1) and O may be rescaled: PV(it - 1) must be done
-            if (it > 0) {
-                ok = wait_all(&bars.pv_done, (it - 1) & 1);
-                if (!ok) break;
-                tc::fence_after_sync();
-            }
-            if (__any_sync(0xffffffffu, over) && !w.first(t_begin)) {
-                // rescale this row of O (earlier tiles of the unit)
-#pragma unroll 1
-                for (int c = 0; c < D; c += 16) {
-                    uint32_t v[16];
-                    tc::ld_32x32b_x16(lane_addr + 256 + c, v);
-                    tc::wait_ld();
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * alpha);
-                    tc::st_32x32b_x16(lane_addr + 256 + c, v);
-                }
-                tc::wait_st();
-            }
-            const float mu = m_used == -INFINITY ? 0.f : m_used;
-#pragma unroll 1
-            for (int c = 0; c < kTokTile; c += 16) {
-                uint32_t v[16];
-                tc::ld_32x32b_x16(s_addr + c, v);
-                tc::wait_ld();
-                uint32_t wd[8];
-#pragma unroll
-                for (int e = 0; e < 16; e += 2) {
-                    const float p0 = c + e < vis ? ex2(fmaf(__uint_as_float(v[e]), a.scale_log2, -mu)) : 0.f;
-                    const float p1 = c + e + 1 < vis ? ex2(fmaf(__uint_as_float(v[e + 1]), a.scale_log2, -mu)) : 0.f;
-                    const __nv_bfloat162 h2 = __floats2bfloat162_rn(p0, p1);
-                    l += __low2float(h2) + __high2float(h2);  // the weights P V uses
-                    wd[e / 2] = *reinterpret_cast<const uint32_t *>(&h2);
-                }
-                // columns c .. c + 15 are 16-byte chunks 2 (c % 64) / 16, +1 of atom c / 64
-                const int at = c >> 6, j0 = (c & 63) >> 3;
-                *reinterpret_cast<uint4 *>(p_buf + at * kAtom + sw128(r, j0)) = make_uint4(wd[0], wd[1], wd[2], wd[3]);
-                *reinterpret_cast<uint4 *>(p_buf + at * kAtom + sw128(r, j0 + 1)) = make_uint4(wd[4], wd[5], wd[6], wd[7]);
-            }
-            tc::fence_before_sync();
-            __syncwarp();
-            tc::mbar_arrive_elect(smem_u32(&bars.s_free[it & 1]));  // S(it) read
-            tc::fence_proxy_async_smem();
-            __syncwarp();
-            tc::mbar_arrive_elect(smem_u32(&bars.p_full));
-            if (w.last()) {
-                // ---- the unit's partial: O / l and its log-sum-exp, slot u + part
-                ok = wait_all(&bars.pv_done, it & 1);
-                if (!ok) break;
-                tc::fence_after_sync();
-                const float inv = l > 0.f ? 1.f / l : 0.f;
-                const int64_t slot = static_cast<int64_t>(u) + part;
-                float *out = a.o_part + (slot * a.rows + r) * D;
-#pragma unroll 1
-                for (int c = 0; c < D; c += 16) {
-                    uint32_t v[16];
-                    tc::ld_32x32b_x16(lane_addr + 256 + c, v);
-                    tc::wait_ld();
-                    if (row_ok) {
-#pragma unroll
-                        for (int e = 0; e < 16; e += 4)
-                            *reinterpret_cast<float4 *>(out + c + e) =
-                                make_float4(__uint_as_float(v[e]) * inv, __uint_as_float(v[e + 1]) * inv,
-                                            __uint_as_float(v[e + 2]) * inv, __uint_as_float(v[e + 3]) * inv);
-                    }
-                }
-                if (row_ok)
-                    a.lse_part[slot * a.rows + r] = l > 0.f ? (m_used + log2f(l)) * 0.69314718055994531f : -INFINITY;
-                tc::fence_before_sync();
-                __syncwarp();
-            }
-        }
-        if (!ok && lane == 0) fail();
+    // (the block-wide sums also order the barriers' set-up before their use)
+    const int64_t T = block_tile_sum(a.kv_len, a.batch, a.q_len, a.max_kv, red64) * a.groups;
+    const int part = warp * gridDim.x + blockIdx.x;  // spread over the SMs first
+    const bool mine = T > 0 && part < a.num_splits;
+    const int64_t t_begin = mine ? part_begin(part, T, a.num_splits) : 0;
+    const int64_t n_tiles = mine ? part_begin(part + 1, T, a.num_splits) - t_begin : 0;
+    if (n_tiles == 0) {
+        griddep_wait();
+        return;
     }
-    tc::fence_before_sync();
-    __syncthreads();
-    if (warp == 1) {
-        tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, 512);
+    const int row0 = blockIdx.y * N;                 // first query row of this row group
+
+    const uint32_t ring =
+        ((smem_u32(smem_raw) + 1023u) & ~1023u) + static_cast<uint32_t>(warp) * (kStages * kStageBytes);
+    const uint64_t policy = gridDim.y == 1 ? tc::policy_evict_first() : tc::policy_evict_last();
+    Segments ld;  // where the next load goes
+    ld.init(a, t_begin, n_tiles, lane);
+    Segments sg = ld;
+    // page ids of 32 consecutive pages of the load's unit, one per lane
+    int page_u = -1, page_0 = 0, page_id = 0;
+    unsigned bad = 0;  // stages whose page id is out of range: not loaded, not used
+
+    // Load the stage at `ld` into slot s, and step on.
+    auto load = [&](int s) {
+        const int u = ld.b * a.groups + ld.g;
+        int blk = u, tok0 = ld.tok;
+        bool good = true;
+        if (a.paged) {
+            const int pg = ld.tok / kPage;
+            if (u != page_u || pg >= page_0 + 32) {
+                page_u = u;
+                page_0 = pg;
+                const int n = min(32, (ld.tok_end + kPage - 1) / kPage - pg);
+                page_id = lane < n ? a.block_table[static_cast<int64_t>(u) * a.bt_stride + pg + lane] : 0;
+            }
+            blk = __shfl_sync(0xffffffffu, page_id, pg - page_0);
+            tok0 = ld.tok % kPage;
+            good = blk >= 0 && blk < a.num_pages;
+            if (!good && lane == 0) record_status(a.status, kStatusBounds);
+        }
+        bad = good ? bad & ~(1u << s) : bad | (1u << s);
+        const uint32_t bar = smem_u32(&bars[warp][s]);
+        if (lane == 0) tc::mbar_arrive_expect_tx(bar, good ? kStageBytes : 0);
+        __syncwarp();
+        if (good && lane < 2 * KA)  // K atoms, then V atoms
+            tc::tma_load_3d_hint(ring + s * kStageBytes + lane * kAtom, lane < KA ? &map_k : &map_v,
+                                 64 * (lane % KA), tok0, blk, bar, policy);
+        ld.next(a, TOK);
+    };
+    for (int s = 0; s < kStages; ++s)
+        if (ld.more()) load(s);
+    griddep_wait();
+
+    uint32_t qf[D / 16][NJ][2];  // Q^T fragments: rows lane / 4 + 8 j, columns 16 k + 2 (lane % 4) (+ 8)
+    float o[D / 16][NJ][4];      // O^T: d = 16 i + lane / 4 (+ 8), rows 8 j + 2 (lane % 4) (+ 1)
+    float m[NJ][2], l[NJ][2];    // exponent base and sum of this lane's columns (the sum over its own tokens)
+    int lim[NJ][2];              // last visible token of this lane's columns
+    int slot = 0;
+    uint32_t phase = 0;          // bit s: parity slot s waits for next
+    bool ok = true;
+    const int r4 = lane >> 2, c4 = (lane & 3) * 2;
+    // ldmatrix row and 16-byte column of this lane
+    const int k_row = (lane & 7) + ((lane >> 3) & 1) * 8, k_hi = lane >> 4;
+    const int v_row = (lane & 7) + (lane >> 4) * 8, v_hi = (lane >> 3) & 1;
+
+    while (sg.more()) {  // one segment (unit) per round
+        const int u = sg.b * a.groups + sg.g, kv = sg.kv, tok_end = sg.tok_end;
+        // ---- the unit's rotated queries, straight into fragments: a rotation
+        // pair (k, k + D/2) or (2k, 2k + 1) lies in one lane's columns
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) {
+            const int r = row0 + 8 * j + r4;
+            const bool real = r < a.rows;
+            const int i = r / a.hpg, hh = r - i * a.hpg;
+            const int64_t pos = static_cast<int64_t>(kv) - a.q_len + i;
+            const uint32_t *src = reinterpret_cast<const uint32_t *>(
+                a.q + ((static_cast<int64_t>(sg.b) * a.q_len + (real ? i : 0)) * (a.groups * a.hpg) +
+                       sg.g * a.hpg + (real ? hh : 0)) * D + c4);
+            uint32_t w[D / 8];
+#pragma unroll
+            for (int k = 0; k < D / 8; ++k) w[k] = real ? src[4 * k] : 0u;
+            if (a.style == 0) {
+#pragma unroll
+                for (int k = 0; k < D / 16; ++k) {
+                    float x[2], y[2], cs, sn;
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const float p = e ? __uint_as_float(w[k] & 0xffff0000u) : __uint_as_float(w[k] << 16);
+                        const float q = e ? __uint_as_float(w[k + D / 16] & 0xffff0000u)
+                                          : __uint_as_float(w[k + D / 16] << 16);
+                        rope_cos_sin(pos, turns[8 * k + c4 + e], &cs, &sn);
+                        x[e] = p * cs - q * sn;
+                        y[e] = q * cs + p * sn;
+                    }
+                    w[k] = pack_bf16(x[0], x[1]);
+                    w[k + D / 16] = pack_bf16(y[0], y[1]);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < D / 8; ++k) {
+                    float cs, sn;
+                    rope_cos_sin(pos, turns[4 * k + c4 / 2], &cs, &sn);
+                    const float p = __uint_as_float(w[k] << 16), q = __uint_as_float(w[k] & 0xffff0000u);
+                    w[k] = pack_bf16(p * cs - q * sn, q * cs + p * sn);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < D / 8; ++k) qf[k / 2][j][k % 2] = w[k];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const int rc = row0 + 8 * j + c4 + e;
+                lim[j][e] = rc < a.rows ? kv - a.q_len + rc / a.hpg : kv - 1;  // (padding columns are never written)
+                m[j][e] = -INFINITY;
+                l[j][e] = 0.f;
+            }
+#pragma unroll
+            for (int i2 = 0; i2 < D / 16; ++i2)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) o[i2][j][e] = 0.f;
+        }
+
+        for (int tok = sg.tok; tok < tok_end; tok += TOK) {
+            const uint32_t kb = ring + slot * kStageBytes, vb = kb + KA * kAtom;
+            if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars[warp][slot]), (phase >> slot) & 1u, kWaitLimitNs))) {
+                ok = false;
+                break;
+            }
+            phase ^= 1u << slot;
+            const int valid = min(kv - tok, TOK);  // cached rows of the stage
+            if (valid < TOK) {
+                // value rows past the unit's end may hold anything; their weights
+                // are 0, and 0 x NaN is NaN: clear them
+                for (int x = lane; x < (TOK - valid) * 8 * KA; x += 32) {
+                    const int at = x / ((TOK - valid) * 8), y = x - at * (TOK - valid) * 8;
+                    asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(vb + at * kAtom + (valid + y / 8) * 128 +
+                                                                                  (y % 8) * 16),
+                                 "r"(0)
+                                 : "memory");
+                }
+                tc::fence_proxy_async_smem();  // before a later load overwrites them
+                __syncwarp();
+            }
+            const bool need_mask = tok + TOK - 1 > kv - a.q_len;
+#pragma unroll 1
+            for (int t0 = 0; t0 < ((bad >> slot) & 1u ? 0 : valid); t0 += TB) {
+                // ---- scores of TB tokens (this lane's: t0 + 16 x + lane / 4 (+ 8)), log2 domain before the base
+                float s[TB / 16][NJ][4];
+#pragma unroll
+                for (int x = 0; x < TB / 16; ++x)
+#pragma unroll
+                    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) s[x][j][e] = 0.f;
+#pragma unroll
+                for (int k = 0; k < D / 16; ++k) {
+#pragma unroll
+                    for (int x = 0; x < TB / 16; ++x) {
+                        const int row = t0 + 16 * x + k_row;
+                        uint32_t ka[4];
+                        ldsm4(kb + (k / 4) * kAtom + row * 128 + ((((k % 4) * 2 + k_hi) ^ (lane & 7)) << 4), ka);
+#pragma unroll
+                        for (int j = 0; j < NJ; ++j) mma16816(s[x][j], ka, qf[k][j]);
+                    }
+                }
+                if (need_mask) {
+#pragma unroll
+                    for (int x = 0; x < TB / 16; ++x)
+#pragma unroll
+                        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                if (tok + t0 + 16 * x + r4 + (e >> 1) * 8 > lim[j][e & 1]) s[x][j][e] = -INFINITY;
+                }
+                // ---- exponent bases: raised only when a score passes one by 2^8
+                float mx[NJ][2];
+                bool over = false;
+#pragma unroll
+                for (int j = 0; j < NJ; ++j)
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        float v = fmaxf(s[0][j][e], s[0][j][e + 2]);
+#pragma unroll
+                        for (int x = 1; x < TB / 16; ++x) v = fmaxf(v, fmaxf(s[x][j][e], s[x][j][e + 2]));
+                        mx[j][e] = v * a.scale_log2;
+                        over |= mx[j][e] > m[j][e] + 8.f;
+                    }
+                if (__any_sync(0xffffffffu, over)) {
+#pragma unroll
+                    for (int j = 0; j < NJ; ++j)
+#pragma unroll
+                        for (int e = 0; e < 2; ++e) {
+                            float v = mx[j][e];  // the column's maximum over the eight lanes that hold its tokens
+#pragma unroll
+                            for (int d = 4; d < 32; d <<= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, d));
+                            if (v > m[j][e] + 8.f) {
+                                const float alpha = ex2(m[j][e] - v);  // (0 from a base of -inf)
+                                m[j][e] = v;
+                                l[j][e] *= alpha;
+#pragma unroll
+                                for (int i = 0; i < D / 16; ++i) {
+                                    o[i][j][e] *= alpha;
+                                    o[i][j][e + 2] *= alpha;
+                                }
+                            }
+                        }
+                }
+                // ---- weights, their sums, and P^T as fragments
+                uint32_t pf[TB / 16][NJ][2];
+#pragma unroll
+                for (int j = 0; j < NJ; ++j) {
+                    const float m0 = m[j][0] == -INFINITY ? 0.f : m[j][0], m1 = m[j][1] == -INFINITY ? 0.f : m[j][1];
+#pragma unroll
+                    for (int x = 0; x < TB / 16; ++x)
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const uint32_t w = pack_bf16(ex2(fmaf(s[x][j][2 * h], a.scale_log2, -m0)),
+                                                         ex2(fmaf(s[x][j][2 * h + 1], a.scale_log2, -m1)));
+                            l[j][0] += __uint_as_float(w << 16);  // the weights the products use
+                            l[j][1] += __uint_as_float(w & 0xffff0000u);
+                            pf[x][j][h] = mov_trans(w);
+                        }
+                }
+#pragma unroll
+                for (int x = 0; x < TB / 16; ++x) {
+                    const int row = t0 + 16 * x + v_row;
+#pragma unroll
+                    for (int i = 0; i < D / 16; ++i) {
+                        uint32_t va[4];
+                        ldsm4_trans(vb + (i / 4) * kAtom + row * 128 + ((((i % 4) * 2 + v_hi) ^ (lane & 7)) << 4), va);
+#pragma unroll
+                        for (int j = 0; j < NJ; ++j) mma16816(o[i][j], va, pf[x][j]);
+                    }
+                }
+            }
+            __syncwarp();  // every lane has read the slot
+            if (ld.more()) load(slot);
+            if (++slot == kStages) slot = 0;
+        }
+        if (!ok) break;
+
+        // ---- the unit's partial: O / l and its log-sum-exp, slot u + part
+        const int64_t at = (static_cast<int64_t>(u) + part) * a.rows;
+#pragma unroll
+        for (int j = 0; j < NJ; ++j)
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                float sum = l[j][e];
+#pragma unroll
+                for (int d = 4; d < 32; d <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, d);
+                const int r = row0 + 8 * j + c4 + e;
+                if (r < a.rows) {
+                    const float inv = sum > 0.f ? 1.f / sum : 0.f;
+                    float *out = a.o_part + (at + r) * D + r4;
+#pragma unroll
+                    for (int i = 0; i < D / 16; ++i) {
+                        out[16 * i] = o[i][j][e] * inv;
+                        out[16 * i + 8] = o[i][j][e + 2] * inv;
+                    }
+                    if (r4 == 0)
+                        a.lse_part[at + r] = sum > 0.f ? (m[j][e] + log2f(sum)) * 0.69314718055994531f : -INFINITY;
+                }
+            }
+        // on to the next unit's segment (every token of this one was used)
+        sg.tok = tok_end;
+        sg.next(a, 0);
+    }
+    if (!ok) {
+        // a load did not arrive in time: record it, and give the warp's loads
+        // in flight (bounded) time to land before its shared memory goes
+        if (lane == 0) record_status(a.status, kStatusTimeout);
+        for (int s = 0; s < kStages; ++s) mbar_wait(smem_u32(&bars[warp][s]), (phase >> s) & 1u, kWaitLimitNs);
     }
 }
 
@@ -515,27 +483,19 @@ cudaError_t encode_tile_map(CUtensorMap *m, const void *base, int cols, int64_t 
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-template <int D>
-cudaError_t launch_d(const GqaLaunch &g, cudaStream_t st)
+template <int D, int N>
+cudaError_t launch_dn(const GqaLaunch &g, int row_groups, cudaStream_t st)
 {
     const CacheView &c = g.cache;
     const bool paged = c.block_table != nullptr;
     const int tpb = paged ? c.page_size : c.capacity;
     const int blocks = paged ? c.num_pages : g.batch * g.groups;
-    const int box_rows = paged ? 64 : kTokTile;
+    constexpr int box_rows = kStageBytes / (4 * D);  // a stage's tokens (never across a page)
+    static_assert(kPage % box_rows == 0, "a stage lies in one page");
     CUtensorMap mk, mv;
     cudaError_t e;
     if ((e = encode_tile_map(&mk, c.k_rope, D, c.r_tok, c.r_blk, tpb, blocks, box_rows)) != cudaSuccess) return e;
     if ((e = encode_tile_map(&mv, c.c_kv, D, c.c_tok, c.c_blk, tpb, blocks, box_rows)) != cudaSuccess) return e;
-    constexpr int tile = kTokTile * D * 2, atom = 128 * 128;
-    int dev = 0, optin = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const int fixed = 1024 + (D / 64) * atom + 2 * atom;
-    const int static_bytes = static_cast<int>(sizeof(GqaBars)) + 64 * 8 + 64;
-    int slots = (optin - static_bytes - fixed) / tile;
-    if (slots > 2 * kMaxRing) slots = 2 * kMaxRing;
-    if (slots < 2) return cudaErrorInvalidConfiguration;
     GqaArgs a;
     a.batch = g.batch;
     a.q_len = g.q_len;
@@ -547,8 +507,6 @@ cudaError_t launch_d(const GqaLaunch &g, cudaStream_t st)
     a.paged = paged;
     a.bt_stride = c.bt_stride;
     a.num_pages = c.num_pages;
-    a.nk = (slots + 1) / 2;
-    a.nv = slots - a.nk;
     a.scale_log2 = g.sm_scale * 1.4426950408889634f;
     a.style = g.rope_style;
     a.kv_len = g.kv_len;
@@ -558,21 +516,52 @@ cudaError_t launch_d(const GqaLaunch &g, cudaStream_t st)
     a.lse_part = g.lse_part;
     a.status = g.status;
     a.turns = rope_turns(D, g.rope_base);
-    const size_t smem = static_cast<size_t>(fixed) + static_cast<size_t>(slots) * tile;
-    if ((e = cudaFuncSetAttribute(gqa_attn_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    constexpr size_t smem = 1024 + static_cast<size_t>(kWarps) * kStages * kStageBytes;
+    if ((e = cudaFuncSetAttribute(gqa_attn_kernel<D, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   static_cast<int>(smem))) != cudaSuccess)
         return e;
-    return launch_dependent(gqa_attn_kernel<D>, dim3(1, g.num_splits, 1), dim3(kGqaThreads), smem, st, 1, a, mk, mv);
+    // the partitions over the SMs' blocks first, then over each block's warps
+    const int per_group = (g.sms + row_groups - 1) / row_groups;
+    int grid = g.num_splits < per_group ? g.num_splits : per_group;
+    if (g.num_splits > grid * kWarps) grid = (g.num_splits + kWarps - 1) / kWarps;
+    return launch_dependent(gqa_attn_kernel<D, N>, dim3(grid, row_groups, 1), dim3(32 * kWarps), smem, st, 1, a, mk,
+                            mv);
+}
+
+template <int D>
+cudaError_t launch_d(const GqaLaunch &g, int row_groups, int n, cudaStream_t st)
+{
+    switch (n) {
+    case 8: return launch_dn<D, 8>(g, row_groups, st);
+    case 16: return launch_dn<D, 16>(g, row_groups, st);
+    case 24: return launch_dn<D, 24>(g, row_groups, st);
+    case 32:
+        if constexpr (D == 64) return launch_dn<D, 32>(g, row_groups, st);
+        return cudaErrorInvalidConfiguration;
+    default: return cudaErrorInvalidConfiguration;
+    }
 }
 
 }  // namespace
 
+int gqa_row_groups(int rows, int head_dim)
+{
+    // The accumulators (D x N fp32 over 32 lanes) and query fragments have to
+    // fit a warp's registers: 32 rows of width 64 take 248, 24 of width 128
+    // 255 without spills, 32 of width 128 spill 100 words.
+    const int most = head_dim == 64 ? 32 : 24;
+    return (rows + most - 1) / most;
+}
+
 cudaError_t launch_gqa_attn(const GqaLaunch &g, cudaStream_t st)
 {
     if (g.batch <= 0) return cudaSuccess;
-    if (g.q_len * g.hpg > 128) return cudaErrorInvalidConfiguration;
-    if (g.head_dim == 64) return launch_d<64>(g, st);
-    if (g.head_dim == 128) return launch_d<128>(g, st);
+    const int rows = g.q_len * g.hpg;
+    if (rows > 128) return cudaErrorInvalidConfiguration;
+    const int groups = gqa_row_groups(rows, g.head_dim);
+    const int n = ((rows + groups - 1) / groups + 7) / 8 * 8;
+    if (g.head_dim == 64) return launch_d<64>(g, groups, n, st);
+    if (g.head_dim == 128) return launch_d<128>(g, groups, n, st);
     return cudaErrorInvalidConfiguration;
 }
 

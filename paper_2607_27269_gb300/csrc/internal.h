@@ -136,7 +136,12 @@ struct GqaLaunch {
     float *o_part, *lse_part;
     unsigned *status;
     CacheView cache;
+    int sms;
 };
+// A partition is one warp; query rows past what a warp's registers hold run
+// as row groups that each walk every partition.
+constexpr int kGqaPartsPerSm = 7;
+int gqa_row_groups(int rows, int head_dim);
 cudaError_t launch_gqa_attn(const GqaLaunch &g, cudaStream_t st);
 
 // E2E loss forward (mla_e2e_loss): a_mla, a_orig bf16 [rows, hidden], mask [rows] or null.

@@ -101,3 +101,30 @@ def test_gqa_split_counts_and_paged(splits):
                              block_table=None, num_pages=0, capacity=cap)
     _, step_c = run(gc, splits)
     assert torch.equal(step_p.o.cpu(), step_c.o.cpu())
+
+
+@pytest.mark.parametrize("hpg,q_len,d,paged,style", [
+    (1, 1, 64, False, 0), (3, 1, 128, True, 1), (8, 1, 128, False, 0), (3, 3, 64, True, 0), (5, 5, 64, False, 1),
+    (6, 4, 128, True, 0), (5, 5, 128, False, 0), (8, 4, 64, True, 1), (11, 3, 64, False, 0), (8, 6, 128, False, 1),
+    (7, 8, 64, True, 0), (8, 16, 64, False, 0), (8, 16, 128, True, 0)])
+def test_gqa_row_counts_and_stage_tails(hpg, q_len, d, paged, style):
+    """Query rows from 1 to 128 (every width of the kernel's row blocks, one
+    to six row groups) against units that end around every load stage and tile
+    boundary; rows past a unit's end hold NaN and must not reach an output."""
+    lens = [1, 31, 32, 33, 63, 64, 65, 96, 127, 128, 129, 192, 300]
+    G, B = 2, len(lens)
+    shape = wl.Shape("rows", B, hpg * G, G, d, 64, d, 128, 0, q_len, 300, 300, paged=paged, rope_style=style)
+    w = wl.make(shape, seed=63)
+    w.kv_len = torch.tensor([max(t, q_len) for t in lens], dtype=torch.int32)
+    w.start_pos = w.kv_len - q_len
+    gw = wl.gqa(w, seed=63)
+    for u in range(B * G):
+        kv = int(gw.kv_len[u // G])
+        for t in range(kv, -(-kv // 64) * 64 if paged else gw.capacity):
+            at = (int(gw.block_table[u, t // 64]), t % 64) if paged else (u, t)
+            gw.k_cache[at] = float("nan")
+            gw.v_cache[at] = float("nan")
+    _, step = run(gw)
+    _, ref = oracle_run(gw)
+    assert_close(step.o.cpu().numpy(), ref["o"], "o")
+    assert_close(step.lse.cpu().numpy(), ref["lse"], "lse")
