@@ -3,28 +3,26 @@
 // of the two softmax distributions (Eq. 9) and greedy agreement of their
 // argmaxes (Eq. 10), one vocabulary row per context.
 //
-// Many rows (at least kRowKernelRows): one CTA per row, rows strided over a
-// grid of two CTAs per SM.  Pass 1 streams both logit rows from HBM and marks
-// their lines evict-last, so that pass 2 reads them again from L2; a CTA moves
-// on to its next row as soon as it has written this one, so the SM's loads
-// never wait on another CTA's reductions.  Block-wide reductions run in a
-// fixed order (bit-reproducible).
-//
-// Few rows: a row is split over a cluster of kCluster CTAs, each owning a
-// contiguous slice of the vocabulary.  When both rows' slices fit in shared memory
-// (every vocabulary of the workloads, in bf16), one thread copies them in with
-// bulk copies at the start, so the whole slice is in flight at once and HBM is
-// read exactly once; both passes then read shared memory.  Otherwise the
-// passes stream the slice from global memory (the second from L2).
-// Pass 1: maximum, sum of exponentials and first argmax of both rows, a
-// vector of 8 (bf16) or 4 (fp32) logits at a time.  The CTAs exchange these
-// through distributed shared memory and combine them in rank order (every CTA
-// gets the same result, bit for bit).  Pass 2: sum of min(p_D, p_T) over the
-// slice; rank 0 adds the slices in rank order.  Exponentials are base 2 with
-// log2(e) folded into one FMA, and pass 2 folds the normaliser into the
+// A context's two rows go to one cluster of C CTAs (1 .. 8), which takes two
+// passes over them: maxima, sums of exponentials and argmaxes (from HBM, the
+// lines marked evict-last), then the overlap (from L2).  Exponentials are base
+// 2 with log2(e) folded into one FMA, and pass 2 folds the normaliser into the
 // exponent, p = 2^(x log2 e - c) with c = m log2 e + log2 Z, so that
 // min(p_D, p_T) = 2^min(., .) costs one exponential per token, not two.
+//
+// Bound: HBM (both rows once), then issue slots (about 16 per token pair over
+// both passes); between the two passes of a row stand reductions and a cluster
+// barrier, some 2 us that only other CTAs' work can hide.  So three CTAs of
+// 256 threads share an SM, and C is chosen so that the rows fill the GPU in
+// whole waves.  640 rows of 128256 bf16: 109.2 us with one CTA of 512 threads
+// per row (304 at a time: a third wave of 32 rows, and the lines of 304 rows
+// past the L2's 129 MB), 78.4 us so; 40 rows of 151936 fp32: 35.4 us with the
+// slices resident in shared memory (320 CTAs of 152 KB, three waves), 15.3 us
+// so; 2 rows of 128256 bf16: 8.4 -> 6.0 us.  The sums and orders are fixed: the
+// bits do not depend on timing.
 #include <math.h>
+
+#include <atomic>
 
 #include "common.cuh"
 #include "internal.h"
@@ -33,19 +31,12 @@
 namespace gbmla {
 namespace {
 
-constexpr int kCluster = 8;
-constexpr int kAccThreads = 256;
-constexpr int kUnroll = 4;                       // streaming path: vectors per tensor per thread in flight
-constexpr uint32_t kResidentMax = 200 * 1024;    // shared-memory bytes for both slices
-constexpr uint32_t kBulkPiece = 8 * 1024;        // bytes per bulk copy (per row); pass 1 follows the pieces in
-constexpr int kMaxPieces = 16;                   // kResidentMax / 2 / kBulkPiece, rounded up
-
 constexpr float kLog2e = 1.4426950408889634f;
 
 struct Stat {
-    float m;   // running maximum
-    float s;   // sum of exp(x - m) = 2^((x - m) log2 e)
-    int idx;   // lowest index holding m
+    float m;   // maximum
+    float s;   // sum of 2^((x - max(m, kLowest)) log2 e)
+    int idx;   // where the maximum is (0x7fffffff: nowhere)
 };
 
 // 2^x (the hardware approximation; relative error ~2^-22, and 2^-inf = 0)
@@ -54,63 +45,6 @@ __device__ __forceinline__ float ex2(float x)
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
-}
-
-// Sum of f(0) .. f(N-1) as a balanced tree (independent exponentials, a
-// dependency chain of log2 N additions rather than N).
-template <int N, typename F>
-__device__ __forceinline__ float tree_sum(F f)
-{
-    float v[N];
-#pragma unroll
-    for (int e = 0; e < N; ++e) v[e] = f(e);
-#pragma unroll
-    for (int w = 1; w < N; w *= 2)
-#pragma unroll
-        for (int e = 0; e + w < N; e += 2 * w) v[e] += v[e + w];
-    return v[0];
-}
-
-// Fold one vector of logits x[0..VN) at indices ybase.. into a: the vector's
-// maximum first, so the running base moves (and the sum is rescaled) at most
-// once per vector.  A thread visits its indices in increasing order, so an
-// equal maximum seen later never displaces the stored index.
-template <int VN>
-__device__ __forceinline__ void stat_vec(Stat &a, const float (&x)[VN], int ybase)
-{
-    float vm = x[0];
-#pragma unroll
-    for (int e = 1; e < VN; ++e) vm = fmaxf(vm, x[e]);
-    if (vm > a.m) {
-        a.s *= ex2((a.m - vm) * kLog2e);
-        a.m = vm;
-        int e0 = VN - 1;
-#pragma unroll
-        for (int e = VN - 1; e >= 0; --e)
-            if (x[e] == vm) e0 = e;
-        a.idx = ybase + e0;
-    }
-    const float ml = a.m * kLog2e;
-    a.s += tree_sum<VN>([&](int e) { return ex2(fmaf(x[e], kLog2e, -ml)); });
-}
-
-__device__ __forceinline__ void stat_one(Stat &a, float x, int y)
-{
-    const float v[1] = {x};
-    stat_vec<1>(a, v, y);
-}
-
-__device__ __forceinline__ Stat stat_merge(Stat a, Stat b)
-{
-    if (b.s == 0.f) return a;
-    if (a.s == 0.f) return b;
-    if (b.m > a.m || (b.m == a.m && b.idx < a.idx)) {
-        const Stat t = a;
-        a = b;
-        b = t;
-    }
-    a.s += b.s * ex2((b.m - a.m) * kLog2e);  // a.m >= b.m
-    return a;
 }
 
 // ---- packed forms for bf16 logits (fewer instructions per token): the
@@ -172,29 +106,6 @@ __device__ __forceinline__ float ex2_sum8(const uint64_t (&t)[4])
     return lo + hi;
 }
 
-// stat_vec for eight bf16 logits in their raw 16-byte vector.
-__device__ __forceinline__ void stat_bf16(Stat &a, const uint4 &v, int ybase)
-{
-    const uint32_t mw = bmax2(bmax2(v.x, v.y), bmax2(v.z, v.w));
-    const float vm = fmaxf(bf16_lo(mw), bf16_hi(mw));
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-    if (vm > a.m) {
-        a.s *= ex2((a.m - vm) * kLog2e);
-        a.m = vm;
-        int e0 = 7;
-#pragma unroll
-        for (int e = 7; e >= 0; --e)
-            if (((e & 1) ? bf16_hi(w[e >> 1]) : bf16_lo(w[e >> 1])) == vm) e0 = e;
-        a.idx = ybase + e0;
-    }
-    const float nml = -(a.m * kLog2e);
-    const uint64_t L = pk(kLog2e, kLog2e), C = pk(nml, nml);
-    uint64_t t[4];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) t[q] = fma2(bf16x2_f32x2(w[q]), L, C);
-    a.s += ex2_sum8(t);
-}
-
 // Sum over eight bf16 token pairs of min(p_D, p_T) = 2^min(x_D log2 e - c_D, x_T log2 e - c_T).
 __device__ __forceinline__ float pmin_bf16(const uint4 &vd, const uint4 &vt, float cd, float ct)
 {
@@ -216,45 +127,11 @@ struct Vec;
 template <>
 struct Vec<float> {
     static constexpr int n = 4;
-    __device__ static void load(const float *p, float (&x)[4], bool stream)
-    {
-        const float4 v = stream ? __ldcs(reinterpret_cast<const float4 *>(p)) : *reinterpret_cast<const float4 *>(p);
-        x[0] = v.x;
-        x[1] = v.y;
-        x[2] = v.z;
-        x[3] = v.w;
-    }
-    __device__ static void cvt(const uint4 &w, float (&x)[4])
-    {
-        x[0] = __uint_as_float(w.x);
-        x[1] = __uint_as_float(w.y);
-        x[2] = __uint_as_float(w.z);
-        x[3] = __uint_as_float(w.w);
-    }
     __device__ static float one(const float *p) { return *p; }
 };
 template <>
 struct Vec<uint16_t> {
     static constexpr int n = 8;
-    __device__ static void load(const uint16_t *p, float (&x)[8], bool stream)
-    {
-        const uint4 v = stream ? __ldcs(reinterpret_cast<const uint4 *>(p)) : *reinterpret_cast<const uint4 *>(p);
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            x[2 * e] = __uint_as_float(w[e] << 16);
-            x[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-        }
-    }
-    __device__ static void cvt(const uint4 &v, float (&x)[8])
-    {
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            x[2 * e] = __uint_as_float(w[e] << 16);
-            x[2 * e + 1] = __uint_as_float(w[e] & 0xffff0000u);
-        }
-    }
     __device__ static float one(const uint16_t *p) { return __uint_as_float(static_cast<uint32_t>(*p) << 16); }
 };
 
@@ -269,389 +146,373 @@ __device__ __forceinline__ uint4 ld_hint16(const void *p, uint64_t pol)
 }
 
 // Reduction over the 32 lanes of a warp by shuffles; every lane gets the result.
-template <typename V, typename Op>
-__device__ __forceinline__ V warp_reduce(V v, Op op)
+template <typename Op>
+__device__ __forceinline__ float warp_reduce(float v, Op op)
 {
-    for (int o = 16; o > 0; o >>= 1) {
-        V w;
-        if constexpr (sizeof(V) == sizeof(float)) {
-            w = __shfl_xor_sync(0xffffffffu, v, o);
-        } else {
-            w.m = __shfl_xor_sync(0xffffffffu, v.m, o);
-            w.s = __shfl_xor_sync(0xffffffffu, v.s, o);
-            w.idx = __shfl_xor_sync(0xffffffffu, v.idx, o);
-        }
-        v = op(v, w);
-    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
 }
 
-// Block-wide reduction of a value with `op` (identity `id`); every thread gets
-// the result.  Each warp reduces by shuffles, then warp 0 reduces the warps'
-// partials the same way and publishes the result (a fixed tree: the bits do
-// not depend on timing).  `scratch` holds NT / 32 + 1 values.
-template <int NT = kAccThreads, typename V, typename Op>
-__device__ V block_reduce(V v, Op op, V *scratch, V id)
+constexpr int kRowThreads = 256;
+constexpr int kRowCtas = 3;        // per SM
+constexpr int kRowUnroll = 2;      // vectors per tensor in a group
+constexpr int kMaxCluster = 8;
+constexpr float kLowest = -2e38f;  // stands in for a maximum of -inf (or the type's lowest) as the exponents' base
+constexpr float kRaise = 16.f;     // a base is raised once a logit passes it by this much
+
+// Running statistics of one thread: the exact maximum and the first vector
+// holding it, and sum of 2^((x - base) log2 e) over a base that follows the
+// maximum loosely, so that after its first vectors a thread hardly ever
+// rescales (fp32 has room for 2^23 times the largest term).
+struct Run {
+    float m, base, s;
+    int at;  // first logit of the first vector whose maximum is m
+};
+
+__device__ __forceinline__ float vec_max(const uint4 &v, uint16_t)
 {
-    v = warp_reduce(v, op);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();  // (the previous reduction's result has been read)
-    if (lane == 0) scratch[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        V r = warp_reduce(lane < NT / 32 ? scratch[lane] : id, op);
-        if (lane == 0) scratch[NT / 32] = r;
-    }
-    __syncthreads();
-    return scratch[NT / 32];
+    const uint32_t w = bmax2(bmax2(v.x, v.y), bmax2(v.z, v.w));
+    return fmaxf(bf16_lo(w), bf16_hi(w));
+}
+__device__ __forceinline__ float vec_max(const uint4 &v, float)
+{
+    return fmaxf(fmaxf(__uint_as_float(v.x), __uint_as_float(v.y)), fmaxf(__uint_as_float(v.z), __uint_as_float(v.w)));
 }
 
-__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar)
+// Sum of 2^(x log2 e + c) over a vector's logits.
+__device__ __forceinline__ float vec_exp_sum(const uint4 &v, float c, uint16_t)
 {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-                 "l"(src), "r"(bytes), "r"(mbar)
-                 : "memory");
+    const uint64_t L = pk(kLog2e, kLog2e), C = pk(c, c);
+    const uint64_t t[4] = {fma2(bf16x2_f32x2(v.x), L, C), fma2(bf16x2_f32x2(v.y), L, C),
+                           fma2(bf16x2_f32x2(v.z), L, C), fma2(bf16x2_f32x2(v.w), L, C)};
+    return ex2_sum8(t);
+}
+__device__ __forceinline__ float vec_exp_sum(const uint4 &v, float c, float)
+{
+    return (ex2(fmaf(__uint_as_float(v.x), kLog2e, c)) + ex2(fmaf(__uint_as_float(v.y), kLog2e, c))) +
+           (ex2(fmaf(__uint_as_float(v.z), kLog2e, c)) + ex2(fmaf(__uint_as_float(v.w), kLog2e, c)));
+}
+__device__ __forceinline__ float vec_pmin(const uint4 &d, const uint4 &t, float cd, float ct, uint16_t)
+{
+    return pmin_bf16(d, t, cd, ct);
+}
+__device__ __forceinline__ float vec_pmin(const uint4 &d, const uint4 &t, float cd, float ct, float)
+{
+    auto p = [&](uint32_t x, uint32_t y) {
+        return ex2(fminf(fmaf(__uint_as_float(x), kLog2e, -cd), fmaf(__uint_as_float(y), kLog2e, -ct)));
+    };
+    return (p(d.x, t.x) + p(d.y, t.y)) + (p(d.z, t.z) + p(d.w, t.w));
 }
 
-// RESIDENT: the slice is copied into shared memory first (and read there).
-template <typename T, bool RESIDENT>
-__global__ void __launch_bounds__(kAccThreads) accept_kernel(int vocab, int64_t stride, int chunk,
-                                                            const T *__restrict__ draft,
-                                                            const T *__restrict__ target, float *alpha,
-                                                            int32_t *argmax_d, int32_t *argmax_t, int32_t *greedy,
-                                                            unsigned *status)
+__device__ __forceinline__ void run_max(Run &r, float vm, int at)
 {
-    extern __shared__ __align__(16) unsigned char acc_smem[];
-    __shared__ Stat s_stat[kCluster][2];        // (draft, target) statistics of every rank, pushed here by each
-    __shared__ float s_part[kCluster];          // every rank's share of the overlap (rank 0's copy is read)
-    __shared__ Stat scratch_s[kAccThreads / 32 + 1];
-    __shared__ float scratch_f[kAccThreads / 32 + 1];
-    __shared__ __align__(8) uint64_t bar[kMaxPieces];
-    constexpr int VN = Vec<T>::n;
-    const int rank = blockIdx.x % kCluster;
-    const int64_t row = blockIdx.y;
-    const int y0 = rank * chunk, y1 = min(vocab, y0 + chunk);  // chunk is a multiple of VN
-    const int n = y1 > y0 ? y1 - y0 : 0;
-    const int nvec = n / VN;                                    // whole vectors; then the row's tail
-    const T *gd_row = draft + row * stride + y0, *gt_row = target + row * stride + y0;
-    const T *d = gd_row, *t = gt_row;                           // where the passes read the slice
-    bool landed = true;                                         // the bulk copies have arrived
-    // the cluster's CTAs must all have started before one writes another's
-    // shared memory: arrive now, wait just before the first such write
-    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
-    // resident: piece k = bytes [k kBulkPiece, (k + 1) kBulkPiece) of both rows, landing on bar[k]
-    const uint32_t bytes = RESIDENT ? static_cast<uint32_t>(nvec) * VN * sizeof(T) : 0u;  // a multiple of 16
-    const int pieces = static_cast<int>((bytes + kBulkPiece - 1) / kBulkPiece);
-    if (RESIDENT) {
-        const uint32_t pad = (static_cast<uint32_t>(chunk) * sizeof(T) + 15u) & ~15u;
-        const T *sd_buf = reinterpret_cast<const T *>(acc_smem), *st_buf = reinterpret_cast<const T *>(acc_smem + pad);
-        if (threadIdx.x == 0) {
-            for (int k = 0; k < pieces; ++k) mbar_init(&bar[k], 1);
-            tc::fence_barrier_init();
-        }
-        __syncthreads();
-        griddep_wait();
-        griddep_launch_dependents();
-        if (threadIdx.x == 0) {
-            for (int k = 0; k < pieces; ++k) {
-                const uint32_t o = k * kBulkPiece, len = bytes - o < kBulkPiece ? bytes - o : kBulkPiece;
-                const uint32_t b = smem_u32(&bar[k]);
-                tc::mbar_arrive_expect_tx(b, 2 * len);
-                bulk_load(smem_u32(sd_buf) + o, reinterpret_cast<const unsigned char *>(gd_row) + o, len, b);
-                bulk_load(smem_u32(st_buf) + o, reinterpret_cast<const unsigned char *>(gt_row) + o, len, b);
-            }
-        }
-        d = sd_buf;
-        t = st_buf;
-    } else {
-        griddep_wait();
-        griddep_launch_dependents();
+    if (vm > r.m) {
+        r.m = vm;
+        r.at = at;
     }
-
-    // ---- pass 1: maxima, sums, argmaxes
-    Stat sd{-INFINITY, 0.f, 0x7fffffff}, st{-INFINITY, 0.f, 0x7fffffff};
-    if (RESIDENT) {
-        constexpr int kPieceVecs = kBulkPiece / 16;  // 16-byte vectors per piece and row
-        for (int k = 0; k < pieces; ++k) {
-            // a wait that runs out is recorded, and the piece is read from global memory instead
-            const bool ok = __syncthreads_and(mbar_wait(smem_u32(&bar[k]), 0, kWaitLimitNs));
-            if (!ok) {
-                landed = false;
-                if (threadIdx.x == 0) record_status(status, kStatusTimeout);
-            }
-            const T *pd = ok ? d : gd_row, *pt = ok ? t : gt_row;
-            const int v1 = min(nvec, (k + 1) * kPieceVecs);
-            for (int v = k * kPieceVecs + threadIdx.x; v < v1; v += kAccThreads) {
-                float xd[VN], xt[VN];
-                Vec<T>::load(pd + v * VN, xd, false);
-                Vec<T>::load(pt + v * VN, xt, false);
-                stat_vec<VN>(sd, xd, y0 + v * VN);
-                stat_vec<VN>(st, xt, y0 + v * VN);
-            }
-        }
-        if (!landed) {  // pass 2 reads global memory
-            d = gd_row;
-            t = gt_row;
-        }
-    } else {
-        for (int v0 = threadIdx.x; v0 < nvec; v0 += kAccThreads * kUnroll) {
-            float xd[kUnroll][VN], xt[kUnroll][VN];
-#pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                const int v = v0 + u * kAccThreads;
-                if (v < nvec) {
-                    Vec<T>::load(d + v * VN, xd[u], false);
-                    Vec<T>::load(t + v * VN, xt[u], false);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                const int v = v0 + u * kAccThreads;
-                if (v < nvec) {
-                    stat_vec<VN>(sd, xd[u], y0 + v * VN);
-                    stat_vec<VN>(st, xt[u], y0 + v * VN);
-                }
-            }
-        }
+}
+__device__ __forceinline__ void run_base(Run &r)
+{
+    if (r.m > r.base + kRaise) {
+        r.s *= ex2((r.base - r.m) * kLog2e);
+        r.base = r.m;
     }
-    for (int i = nvec * VN + threadIdx.x; i < n; i += kAccThreads) {  // the row's tail, from global memory
-        stat_one(sd, Vec<T>::one(gd_row + i), y0 + i);
-        stat_one(st, Vec<T>::one(gt_row + i), y0 + i);
-    }
-    auto merge = [](Stat a, Stat b) { return stat_merge(a, b); };
-    const Stat none{-INFINITY, 0.f, 0x7fffffff};
-    sd = block_reduce(sd, merge, scratch_s, none);
-    st = block_reduce(st, merge, scratch_s, none);
-    // push this rank's statistics into slot [rank] of every rank, then combine
-    // all slots in rank order (every CTA computes the same bits)
-    asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
-    if (threadIdx.x < kCluster) {
-        const uint32_t local = smem_u32(&s_stat[rank][0]);
-        uint32_t remote;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(static_cast<int>(threadIdx.x)));
-        // scalar stores: a Stat is 12 bytes, only 4-byte aligned
-        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(sd.m) : "memory");
-        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote + 4), "f"(sd.s) : "memory");
-        asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(remote + 8), "r"(sd.idx) : "memory");
-        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote + 12), "f"(st.m) : "memory");
-        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote + 16), "f"(st.s) : "memory");
-        asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(remote + 20), "r"(st.idx) : "memory");
-    }
-    tc::cluster_sync();
-    Stat gd{-INFINITY, 0.f, 0x7fffffff}, gt{-INFINITY, 0.f, 0x7fffffff};
-    for (int r = 0; r < kCluster; ++r) {
-        gd = stat_merge(gd, s_stat[r][0]);
-        gt = stat_merge(gt, s_stat[r][1]);
-    }
-    // p = exp(x - m) / Z = 2^(x log2 e - c), c = m log2 e + log2 Z
-    const float cd = gd.m * kLog2e + log2f(gd.s), ct = gt.m * kLog2e + log2f(gt.s);
-    auto pmin = [&](float xd, float xt) { return ex2(fminf(fmaf(xd, kLog2e, -cd), fmaf(xt, kLog2e, -ct))); };
-
-    // ---- pass 2: sum of min(p_D, p_T) over the slice
-    float acc = 0.f;
-    if (RESIDENT) {
-        float acc2 = 0.f;  // two vectors per step, two accumulators
-        for (int v = threadIdx.x; v < nvec; v += 2 * kAccThreads) {
-            float xd[VN], xt[VN], yd[VN], yt[VN];
-            const bool second = v + kAccThreads < nvec;
-            Vec<T>::load(d + v * VN, xd, false);
-            Vec<T>::load(t + v * VN, xt, false);
-            if (second) {
-                Vec<T>::load(d + (v + kAccThreads) * VN, yd, false);
-                Vec<T>::load(t + (v + kAccThreads) * VN, yt, false);
-            }
-            acc += tree_sum<VN>([&](int e) { return pmin(xd[e], xt[e]); });
-            if (second) acc2 += tree_sum<VN>([&](int e) { return pmin(yd[e], yt[e]); });
-        }
-        acc += acc2;
-    } else {
-        for (int v0 = threadIdx.x; v0 < nvec; v0 += kAccThreads * kUnroll) {
-            float xd[kUnroll][VN], xt[kUnroll][VN];
-#pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                const int v = v0 + u * kAccThreads;
-                if (v < nvec) {
-                    Vec<T>::load(d + v * VN, xd[u], true);
-                    Vec<T>::load(t + v * VN, xt[u], true);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kUnroll; ++u) {
-                const int v = v0 + u * kAccThreads;
-                if (v < nvec) {
-#pragma unroll
-                    for (int e = 0; e < VN; ++e) acc += pmin(xd[u][e], xt[u][e]);
-                }
-            }
-        }
-    }
-    for (int i = nvec * VN + threadIdx.x; i < n; i += kAccThreads)
-        acc += pmin(Vec<T>::one(gd_row + i), Vec<T>::one(gt_row + i));
-    acc = block_reduce(acc, [](float a, float b) { return a + b; }, scratch_f, 0.f);
-    if (threadIdx.x == 0) {  // this rank's share into slot [rank] of rank 0
-        uint32_t remote;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(&s_part[rank])), "r"(0));
-        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(remote), "f"(acc) : "memory");
-    }
-    tc::cluster_sync();
-    if (rank == 0 && threadIdx.x == 0) {
-        float total = 0.f;
-        for (int r = 0; r < kCluster; ++r) total += s_part[r];  // rank order
-        if (alpha) alpha[row] = total;
-        if (argmax_d) argmax_d[row] = gd.idx;
-        if (argmax_t) argmax_t[row] = gt.idx;
-        if (greedy) greedy[row] = gd.idx == gt.idx;
-    }
-    if (RESIDENT && !landed)  // pieces still in flight land before the CTA leaves
-        for (int k = 0; k < pieces; ++k) mbar_wait(smem_u32(&bar[k]), 0, kWaitLimitNs);
 }
 
-// ---------------------------------------------------------------- one CTA per row
+// A warp's (exact maximum, sum over base max(m, kLowest), first position) of its lanes' runs.
+__device__ __forceinline__ Stat warp_runs(const Run &r)
+{
+    Stat o;
+    o.m = warp_reduce(r.m, [](float a, float b) { return fmaxf(a, b); });
+    o.s = warp_reduce(r.s * ex2((r.base - fmaxf(o.m, kLowest)) * kLog2e), [](float a, float b) { return a + b; });
+    o.idx = __reduce_min_sync(0xffffffffu, r.m == o.m ? r.at : 0x7fffffff);
+    return o;
+}
+// The same over n statistics in shared memory (n <= 64).
+__device__ __forceinline__ Stat warp_stats(const Stat *p, int n)
+{
+    const int lane = threadIdx.x & 31;
+    Run r{-INFINITY, kLowest, 0.f, 0x7fffffff};
+    if (lane < n) {
+        const Stat a = p[lane];
+        r = Run{a.m, fmaxf(a.m, kLowest), a.s, a.idx};
+    }
+    if (lane + 32 < n) {
+        const Stat b = p[lane + 32];
+        const float mb = fmaxf(b.m, kLowest), base = fmaxf(r.base, mb);
+        r.s = r.s * ex2((r.base - base) * kLog2e) + b.s * ex2((mb - base) * kLog2e);
+        r.base = base;
+        if (b.m > r.m || (b.m == r.m && b.idx < r.at)) {
+            r.m = b.m;
+            r.at = b.idx;
+        }
+    }
+    return warp_runs(r);
+}
 
-constexpr int kRowThreads = 512;
-constexpr int kRowUnroll = 2;      // vectors per tensor per thread in flight
-constexpr int kRowKernelRows = 128;
+__device__ __forceinline__ uint32_t map_rank(const void *p, int rank)
+{
+    uint32_t remote;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(p)), "r"(rank));
+    return remote;
+}
 
+// The two rows of a context go to one cluster of C CTAs (C = 1 .. 8), CTA
+// `rank` taking every vector of its contiguous slice; clusters stride over the
+// rows.  Pass 1 reads the slices from HBM (lines kept in L2), pass 2 reads
+// them again.  One cluster barrier a row: each CTA pushes its statistics into
+// every peer's shared memory before it, and the overlap shares of the row
+// before (pushed to rank 0) are summed after it, in rank order.  A group's
+// loads are issued one group ahead, across the passes and the rows too, so the
+// reductions and the barrier wait with loads in flight.  The shared slots
+// alternate between two sets: a peer reuses one only after a barrier that
+// this CTA arrives at after reading it.
 template <typename T>
-__global__ void __launch_bounds__(kRowThreads, 2) accept_row_kernel(int rows, int vocab, int64_t stride,
+__global__ void __launch_bounds__(kRowThreads, kRowCtas) accept_row_kernel(int rows, int vocab, int64_t stride,
                                                                 const T *__restrict__ draft,
                                                                 const T *__restrict__ target, float *alpha,
                                                                 int32_t *argmax_d, int32_t *argmax_t,
-                                                                int32_t *greedy)
+                                                                int32_t *greedy, int C)
 {
-    __shared__ Stat scratch_s[kRowThreads / 32 + 1];
-    __shared__ float scratch_f[kRowThreads / 32 + 1];
+    static_assert(kMaxCluster * kRowThreads / 32 <= 64, "a warp merges the cluster's statistics two per lane");
+    constexpr int VN = Vec<T>::n, kWarps = kRowThreads / 32, U = kRowUnroll, kGroup = kRowThreads * U;
+    __shared__ Stat s_stat[2][2][kMaxCluster * kWarps];  // [row parity][draft, target][rank, warp]
+    __shared__ float s_part[2][kMaxCluster * kWarps];    // rank 0's copy is read
+    __shared__ Stat s_final[2];                 // warp 0 of rank 0: the row's statistics until its results are written
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int rank = blockIdx.x % C, n_cl = gridDim.x / C;
+    const int nvec = vocab / VN;
+    const int share = (nvec + C - 1) / C;
+    const int v_lo = min(nvec, rank * share), v_hi = min(nvec, v_lo + share);
+    const int mine = v_hi - v_lo;  // the slice's vectors
+    const int pairs = (mine + 2 * kGroup - 1) / (2 * kGroup);  // of groups: two buffers take turns
+    const int tail = rank == C - 1 ? nvec * VN + tid : vocab;  // the row's last, partial vector: a logit per thread
+    const uint64_t keep = tc::policy_evict_last(), drop = tc::policy_evict_first();
+    const uint32_t none = sizeof(T) == 2 ? 0xff80ff80u : 0xff800000u;  // -inf
+    // Group `it` of this thread's vectors from its first vectors of the two
+    // rows on; past the slice's end -inf, which changes no maximum or sum.
+    struct Group {
+        uint4 d[U], t[U];
+    };
+    auto load = [&](const uint4 *d, const uint4 *t, int it, uint64_t pol, Group &g) {
+        const int first = it * kGroup;
+        if (first + kGroup <= mine) {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                g.d[u] = ld_hint16(d + first + u * kRowThreads, pol);
+                g.t[u] = ld_hint16(t + first + u * kRowThreads, pol);
+            }
+        } else {
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                g.d[u] = g.t[u] = make_uint4(none, none, none, none);
+                if (first + u * kRowThreads + tid < mine) {
+                    g.d[u] = ld_hint16(d + first + u * kRowThreads, pol);
+                    g.t[u] = ld_hint16(t + first + u * kRowThreads, pol);
+                }
+            }
+        }
+    };
+    // warp 0 of rank 0: a row's results from its statistics and the ranks' shares
+    auto finish = [&](int64_t row, int par) {
+        // the first logit equal to the maximum, in the vector that holds it:
+        // lanes 0.. look at the draft's, lanes 16.. at the target's
+        const int which = lane >> 4;
+        const Stat &f = s_final[which];
+        const int y = f.idx + (lane & 15);
+        const bool hit = f.idx != 0x7fffffff && (lane & 15) < VN && y < vocab &&
+                         Vec<T>::one((which ? target : draft) + row * stride + y) == f.m;
+        const unsigned hits = __ballot_sync(0xffffffffu, hit);
+        float total = (lane < C * kWarps ? s_part[par][lane] : 0.f) + (lane + 32 < C * kWarps ? s_part[par][lane + 32] : 0.f);
+        total = warp_reduce(total, [](float a, float b) { return a + b; });
+        if (lane == 0) {
+            const int id = (hits & 0xffffu) ? s_final[0].idx + __ffs(hits & 0xffffu) - 1 : s_final[0].idx;
+            const int it = (hits >> 16) ? s_final[1].idx + __ffs(hits >> 16) - 1 : s_final[1].idx;
+            if (alpha) alpha[row] = total;
+            if (argmax_d) argmax_d[row] = id;
+            if (argmax_t) argmax_t[row] = it;
+            if (greedy) greedy[row] = id == it;
+        }
+        __syncwarp();
+    };
+    // a peer's shared memory is written only once all the cluster's CTAs have
+    // started: arrive now, wait before the first push
+    asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     griddep_wait();
     griddep_launch_dependents();
-    constexpr int VN = Vec<T>::n;
-    const int nvec = vocab / VN;
-    const uint64_t keep = tc::policy_evict_last(), drop = tc::policy_evict_first();
-    auto merge = [](Stat a, Stat b) { return stat_merge(a, b); };
-    for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
-        const T *d = draft + row * stride, *t = target + row * stride;
-        // ---- pass 1: maxima, sums, argmaxes (lines kept in L2 for pass 2)
-        Stat sd{-INFINITY, 0.f, 0x7fffffff}, st{-INFINITY, 0.f, 0x7fffffff};
-        for (int v0 = threadIdx.x; v0 < nvec; v0 += kRowThreads * kRowUnroll) {
-            uint4 wd[kRowUnroll], wt[kRowUnroll];
+    int64_t row = blockIdx.x / C;
+    const T *d = draft + row * stride, *t = target + row * stride;
+    Group ga, gb;
+    auto vec = [&](const T *x) { return reinterpret_cast<const uint4 *>(x) + v_lo + tid; };
+    if (pairs > 0) load(vec(d), vec(t), 0, keep, ga);
+    int par = 0;
+    for (;; par ^= 1) {
+        // ---- pass 1: maxima, sums, argmaxes
+        Run rd{-INFINITY, kLowest, 0.f, 0x7fffffff}, rt = rd;
+        auto fold = [&](const Group &g, int it) {
 #pragma unroll
-            for (int u = 0; u < kRowUnroll; ++u) {
-                const int v = v0 + u * kRowThreads;
-                if (v < nvec) {
-                    wd[u] = ld_hint16(d + static_cast<int64_t>(v) * VN, keep);
-                    wt[u] = ld_hint16(t + static_cast<int64_t>(v) * VN, keep);
-                }
+            for (int u = 0; u < U; ++u) {
+                const int at = v_lo + it * kGroup + u * kRowThreads + tid;
+                run_max(rd, vec_max(g.d[u], T{}), at);
+                run_max(rt, vec_max(g.t[u], T{}), at);
             }
+            run_base(rd);
+            run_base(rt);
+            const float bd = -rd.base * kLog2e, bt = -rt.base * kLog2e;
 #pragma unroll
-            for (int u = 0; u < kRowUnroll; ++u) {
-                const int v = v0 + u * kRowThreads;
-                if (v < nvec) {
-                    if constexpr (sizeof(T) == 2) {
-                        stat_bf16(sd, wd[u], v * VN);
-                        stat_bf16(st, wt[u], v * VN);
-                    } else {
-                        float xd[VN], xt[VN];
-                        Vec<T>::cvt(wd[u], xd);
-                        Vec<T>::cvt(wt[u], xt);
-                        stat_vec<VN>(sd, xd, v * VN);
-                        stat_vec<VN>(st, xt, v * VN);
-                    }
-                }
+            for (int u = 0; u < U; ++u) {
+                rd.s += vec_exp_sum(g.d[u], bd, T{});
+                rt.s += vec_exp_sum(g.t[u], bt, T{});
             }
+        };
+        const uint4 *vd = vec(d), *vt = vec(t);
+#pragma unroll 1
+        for (int k = 0; k < pairs; ++k) {
+            load(vd, vt, 2 * k + 1, keep, gb);
+            fold(ga, 2 * k);
+            if (k + 1 < pairs)
+                load(vd, vt, 2 * k + 2, keep, ga);
+            else
+                load(vd, vt, 0, drop, ga);
+            fold(gb, 2 * k + 1);
         }
-        for (int i = nvec * VN + threadIdx.x; i < vocab; i += kRowThreads) {  // the row's tail
-            stat_one(sd, Vec<T>::one(d + i), i);
-            stat_one(st, Vec<T>::one(t + i), i);
+        if (rd.at != 0x7fffffff) rd.at *= VN;  // (a vector's first logit)
+        if (rt.at != 0x7fffffff) rt.at *= VN;
+        if (tail < vocab) {
+            const float xd = Vec<T>::one(d + tail), xt = Vec<T>::one(t + tail);
+            run_max(rd, xd, tail);
+            run_max(rt, xt, tail);
+            run_base(rd);
+            run_base(rt);
+            rd.s += ex2((xd - rd.base) * kLog2e);
+            rt.s += ex2((xt - rt.base) * kLog2e);
         }
-        const Stat none{-INFINITY, 0.f, 0x7fffffff};
-        sd = block_reduce<kRowThreads>(sd, merge, scratch_s, none);
-        st = block_reduce<kRowThreads>(st, merge, scratch_s, none);
-        const float cd = sd.m * kLog2e + log2f(sd.s), ct = st.m * kLog2e + log2f(st.s);
-        auto pmin = [&](float xd, float xt) { return ex2(fminf(fmaf(xd, kLog2e, -cd), fmaf(xt, kLog2e, -ct))); };
+        const Stat sd = warp_runs(rd), st = warp_runs(rt);
+        if (row < n_cl) asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // (the first row only)
+        if (lane < 2 * C) {  // lane r: draft to rank r; lane C + r: target to rank r
+            const int which = lane / C;
+            const Stat v = which ? st : sd;
+            const uint32_t to = map_rank(&s_stat[par][which][rank * kWarps + warp], lane - which * C);
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(to), "f"(v.m) : "memory");
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(to + 4), "f"(v.s) : "memory");
+            asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(to + 8), "r"(v.idx) : "memory");
+        }
+        __syncwarp();
+        tc::cluster_sync();
+        if (rank == 0 && warp == 0 && row >= n_cl) finish(row - n_cl, par ^ 1);
+        // ---- the row's statistics over the ranks: p = 2^(x log2 e - c), c = base log2 e + log2 Z
+        float cd, ct;
+        {
+            const Stat ad = warp_stats(s_stat[par][0], C * kWarps), at = warp_stats(s_stat[par][1], C * kWarps);
+            if (rank == 0 && tid == 0) {
+                s_final[0] = ad;
+                s_final[1] = at;
+            }
+            cd = fmaxf(ad.m, kLowest) * kLog2e + log2f(ad.s);
+            ct = fmaxf(at.m, kLowest) * kLog2e + log2f(at.s);
+        }
         // ---- pass 2: sum of min(p_D, p_T), a last read of the lines
-        float acc = 0.f, acc2 = 0.f;
-        for (int v0 = threadIdx.x; v0 < nvec; v0 += kRowThreads * kRowUnroll) {
-            uint4 wd[kRowUnroll], wt[kRowUnroll];
+        const int64_t next = row + n_cl;
+        const T *dn = draft + next * stride, *tn = target + next * stride;
+        float acc = 0.f;
+        auto overlap = [&](const Group &g) {
 #pragma unroll
-            for (int u = 0; u < kRowUnroll; ++u) {
-                const int v = v0 + u * kRowThreads;
-                if (v < nvec) {
-                    wd[u] = ld_hint16(d + static_cast<int64_t>(v) * VN, drop);
-                    wt[u] = ld_hint16(t + static_cast<int64_t>(v) * VN, drop);
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < kRowUnroll; ++u) {
-                const int v = v0 + u * kRowThreads;
-                if (v < nvec) {
-                    float a;
-                    if constexpr (sizeof(T) == 2) {
-                        a = pmin_bf16(wd[u], wt[u], cd, ct);
-                    } else {
-                        float xd[VN], xt[VN];
-                        Vec<T>::cvt(wd[u], xd);
-                        Vec<T>::cvt(wt[u], xt);
-                        a = tree_sum<VN>([&](int e) { return pmin(xd[e], xt[e]); });
-                    }
-                    if (u & 1)
-                        acc2 += a;
-                    else
-                        acc += a;
-                }
-            }
+            for (int u = 0; u < U; ++u) acc += vec_pmin(g.d[u], g.t[u], cd, ct, T{});
+        };
+#pragma unroll 1
+        for (int k = 0; k < pairs; ++k) {
+            load(vd, vt, 2 * k + 1, drop, gb);
+            overlap(ga);
+            if (k + 1 < pairs)
+                load(vd, vt, 2 * k + 2, drop, ga);
+            else if (next < rows)
+                load(vec(dn), vec(tn), 0, keep, ga);
+            overlap(gb);
         }
-        acc += acc2;
-        for (int i = nvec * VN + threadIdx.x; i < vocab; i += kRowThreads)
-            acc += pmin(Vec<T>::one(d + i), Vec<T>::one(t + i));
-        acc = block_reduce<kRowThreads>(acc, [](float a, float b) { return a + b; }, scratch_f, 0.f);
-        if (threadIdx.x == 0) {
-            if (alpha) alpha[row] = acc;
-            if (argmax_d) argmax_d[row] = sd.idx;
-            if (argmax_t) argmax_t[row] = st.idx;
-            if (greedy) greedy[row] = sd.idx == st.idx;
-        }
+        if (tail < vocab)
+            acc += ex2(fminf(fmaf(Vec<T>::one(d + tail), kLog2e, -cd), fmaf(Vec<T>::one(t + tail), kLog2e, -ct)));
+        acc = warp_reduce(acc, [](float a, float b) { return a + b; });
+        if (lane == 0)
+            asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(map_rank(&s_part[par][rank * kWarps + warp], 0)), "f"(acc)
+                         : "memory");
+        __syncwarp();
+        if (next >= rows) break;
+        row = next;
+        d = dn;
+        t = tn;
     }
+    tc::cluster_sync();
+    if (rank == 0 && warp == 0) finish(row, par);
+}
+
+// Clusters of C CTAs of the row kernel that the device runs at a time (a
+// property of the device; 0 if it cannot say), looked up once per device.
+template <typename T>
+int row_clusters(int C)
+{
+    constexpr int kMaxDevices = 64;
+    static std::atomic<int> known[kMaxDevices][kMaxCluster + 1];
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+    int n = known[dev][C].load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(C);
+        cfg.blockDim = dim3(kRowThreads);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = C;
+        attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&n, accept_row_kernel<T>, &cfg) != cudaSuccess) return 0;
+        known[dev][C].store(n, std::memory_order_relaxed);
+    }
+    return n;
 }
 
 template <typename T>
 cudaError_t launch_typed(int rows, int vocab, const void *draft, const void *target, int64_t stride, float *alpha,
-                         int32_t *argmax_d, int32_t *argmax_t, int32_t *greedy, unsigned *status, cudaStream_t st)
+                        int32_t *argmax_d, int32_t *argmax_t, int32_t *greedy, cudaStream_t st)
 {
-    constexpr int vn = Vec<T>::n;
-    if (rows >= kRowKernelRows) {
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        const int grid = rows < 2 * sms ? rows : 2 * sms;
-        return launch_dependent(accept_row_kernel<T>, dim3(grid), dim3(kRowThreads), 0, st, 1, rows, vocab, stride,
-                                static_cast<const T *>(draft), static_cast<const T *>(target), alpha, argmax_d,
-                                argmax_t, greedy);
+    // The cluster size with the least time by a model of what was measured: a
+    // wave of rows takes each CTA its share of a row, at 28 GB/s alone and a
+    // third of 33 GB/s with three CTAs on its SM, and 2 us of latency; of equal
+    // ones the largest.  (640 rows of 128256 bf16 with C = 1, 2, 3, 4, 6, 8:
+    // 98.7, 78.3, 101.2, 78.7, 93.8, 102.3 us; 160 rows 33.2, 25.3, 32.1, 28.3,
+    // 30.7, 31.5; 40 rows of 151936 fp32 46.9, 26.8, 20.5, 18.2, 17.2, 15.3.)
+    constexpr double kAlone = 28e3, kPerSm = 33e3, kRowCost = 2.0;  // bytes per us, bytes per us, us
+    double best = 0;
+    int C = 0, n_cl = 0;
+    for (int c = 1; c <= kMaxCluster; ++c) {
+        const int n = row_clusters<T>(c);
+        if (n <= 0) continue;
+        const int live = rows < n ? rows : n;
+        const double load = live * c / static_cast<double>(row_clusters<T>(1)) * kRowCtas;  // CTAs per SM
+        const double rate = load * kAlone > kPerSm ? kPerSm / load : kAlone;
+        const double us = ((rows + n - 1) / n) * (2.0 * vocab * sizeof(T) / (c * rate) + kRowCost);
+        if (C == 0 || us < best * 1.001) {
+            best = us;
+            C = c;
+            n_cl = live;
+        }
     }
-    int chunk = (vocab + kCluster - 1) / kCluster;
-    chunk = (chunk + vn - 1) / vn * vn;
-    const uint32_t pad = (static_cast<uint32_t>(chunk) * sizeof(T) + 15u) & ~15u;
-    const dim3 grid(kCluster, rows);
-    const T *dp = static_cast<const T *>(draft), *tp = static_cast<const T *>(target);
-    if (2 * pad <= kResidentMax) {
-        cudaError_t e = cudaFuncSetAttribute(accept_kernel<T, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             static_cast<int>(2 * pad));
-        if (e != cudaSuccess) return e;
-        return launch_dependent(accept_kernel<T, true>, grid, dim3(kAccThreads), 2 * pad, st, kCluster, vocab, stride,
-                                chunk, dp, tp, alpha, argmax_d, argmax_t, greedy, status);
-    }
-    return launch_dependent(accept_kernel<T, false>, grid, dim3(kAccThreads), 0, st, kCluster, vocab, stride, chunk,
-                            dp, tp, alpha, argmax_d, argmax_t, greedy, status);
+    if (C == 0) return cudaErrorInvalidConfiguration;
+    return launch_dependent(accept_row_kernel<T>, dim3(n_cl * C), dim3(kRowThreads), 0, st, C, rows, vocab, stride,
+                            static_cast<const T *>(draft), static_cast<const T *>(target), alpha, argmax_d, argmax_t,
+                            greedy, C);
 }
 
 }  // namespace
 
 cudaError_t launch_acceptance(int rows, int vocab, int dtype, const void *draft, const void *target, int64_t stride,
-                              float *alpha, int32_t *argmax_d, int32_t *argmax_t, int32_t *greedy, unsigned *status,
-                              cudaStream_t st)
+                              float *alpha, int32_t *argmax_d, int32_t *argmax_t, int32_t *greedy, cudaStream_t st)
 {
     if (rows <= 0) return cudaSuccess;
     if (dtype == 0)
-        return launch_typed<float>(rows, vocab, draft, target, stride, alpha, argmax_d, argmax_t, greedy, status, st);
-    return launch_typed<uint16_t>(rows, vocab, draft, target, stride, alpha, argmax_d, argmax_t, greedy, status, st);
+        return launch_typed<float>(rows, vocab, draft, target, stride, alpha, argmax_d, argmax_t, greedy, st);
+    return launch_typed<uint16_t>(rows, vocab, draft, target, stride, alpha, argmax_d, argmax_t, greedy, st);
 }
 
 }  // namespace gbmla

@@ -409,11 +409,8 @@ mla_status mla_acceptance_stats(int32_t rows, int32_t vocab, int32_t logits_dtyp
     if (!draft_logits || !target_logits || !aligned16(draft_logits) || !aligned16(target_logits) ||
         (row_stride * es) % 16)
         return MLA_ERR_INVALID_ARG;
-    unsigned *status = nullptr;
-    mla_status s = device_info(&status, nullptr);
-    if (s != MLA_OK) return s;
     return from_cuda(launch_acceptance(rows, vocab, logits_dtype, draft_logits, target_logits, row_stride,
-                                       alpha_sample, argmax_draft, argmax_target, greedy_accept, status,
+                                       alpha_sample, argmax_draft, argmax_target, greedy_accept,
                                        static_cast<cudaStream_t>(stream)));
 }
 

@@ -121,8 +121,7 @@ cudaError_t launch_project(const mla_dims &d, const CacheView &c, int batch, int
 
 // Acceptance statistics (mla_acceptance_stats): dtype 0 = fp32, 1 = bf16 logits.
 cudaError_t launch_acceptance(int rows, int vocab, int dtype, const void *draft, const void *target, int64_t stride,
-                              float *alpha, int32_t *argmax_d, int32_t *argmax_t, int32_t *greedy, unsigned *status,
-                              cudaStream_t st);
+                              float *alpha, int32_t *argmax_d, int32_t *argmax_t, int32_t *greedy, cudaStream_t st);
 
 // Original-GQA decode attention (mla_gqa_decode_attn): per (sequence, KV
 // group) unit b * G + g, keys in cache.k_rope and values in cache.c_kv.

@@ -89,8 +89,7 @@ def test_acceptance_row_stride_and_empty():
 
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 def test_acceptance_many_rows_ties_ragged_and_strided(dtype):
-    """160 rows take the one-CTA-per-row kernel (more than one row per CTA
-    on the grid of two CTAs per SM): ragged vocabularies (a tail past the last
+    """160 rows (clusters of two or more CTAs, or one a row): ragged vocabularies (a tail past the last
     whole vector; a vocabulary shorter than one vector), equal maxima far
     apart (the lowest index wins), identical rows (greedy agreement, alpha =
     1) and rows padded to a longer stride -- every row against the oracle."""
@@ -128,3 +127,27 @@ def test_acceptance_full_rows_sampled(name):
     assert np.array_equal(ad.cpu().numpy()[pick], ref["argmax_draft"])
     assert np.array_equal(gr.cpu().numpy()[pick], ref["greedy"])
     assert np.abs(alpha.cpu().numpy()[pick] - ref["alpha_sample"]).max() <= ALPHA_TOL
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("rows,vocab", [(2, 1), (3, 8), (2, 2049), (5, 4099), (700, 515), (61, 9001), (1200, 37)])
+def test_acceptance_masked_logits_and_cluster_sizes(rows, vocab, dtype):
+    """Rows and vocabularies that take clusters of one to eight CTAs, slices
+    with no vector at all, groups that end inside and several rows per cluster;
+    logits masked with -inf and with the type's lowest value (whole vectors of
+    them, a thread's first ones included) weigh nothing.  Error: the sums are
+    trees of fp32 exponentials, as above."""
+    g = torch.Generator().manual_seed(57)
+    d = (torch.randn(rows, vocab, generator=g) * 2).to(dtype)
+    t = (torch.randn(rows, vocab, generator=g) * 2).to(dtype)
+    low = torch.finfo(dtype).min
+    keep = max(1, vocab // 3)
+    d[0, keep:] = float("-inf")
+    t[0, :vocab - keep] = float("-inf")
+    d[1, keep:] = low
+    t[1, keep:] = low
+    check(d, t)
+    if vocab > 40:
+        d[rows - 1, : vocab // 2] += 60.0  # the base is raised late, and by much
+        t[rows - 1, vocab // 2:] += 60.0
+        check(d, t)
