@@ -105,93 +105,131 @@ __device__ __forceinline__ uint64_t *o_free_bar(B &b, int i)
 template <int N>
 struct Shared {
     float red[4][N];   // per TMEM-quadrant column partials
-    float m_used[N];   // exponent base of each query column (log2 domain)
+    alignas(16) float neg_m[N];  // minus the exponent base of each query column (0 while it has none)
+    float m_used[N];   // exponent base of each query column (log2 domain; -inf: no key seen)
     float alpha[N];    // rescale factor of the current tile
     float lsum[N];     // softmax denominators at the epilogue (one O^T buffer)
     float inv_l[N];    // 1 / softmax denominator of the last closed sequence (two buffers)
     int lim[N];        // last visible position of each column (-1: padding column)
-    int need_max;
-    int any_rescale;
     int abort;         // any role gave up: producer / MMA stop issuing
-    int sm_fail;       // softmax warps gave up (read only after a named barrier)
     uint32_t tmem_base;
 };
 
-// Tiles [t_begin, t_end) of the flattened tile list, sequence by sequence.
+// The n tiles of a partition (from tile t_begin of the flattened list on),
+// sequence by sequence; the same in every lane of a warp.  Tiles count from
+// the partition's first.
 struct Walk {
     const int32_t *kv;
-    int batch, q_len, max_kv;
-    int b;
-    int64_t seq_start, nb, t, t_begin, t_end;
+    int q_len, max_kv, batch;
+    int b, seq_start, nb, t, n;  // the current sequence, its first tile (negative: it began earlier) and tile count
 
-    __device__ void init(const int32_t *kv_len, int batch_, int q_len_, int max_kv_, int64_t tb, int64_t te)
+    __device__ void init(const TcArgs &a, int64_t t_begin, int n_tiles)
     {
-        kv = kv_len;
-        batch = batch_;
-        q_len = q_len_;
-        max_kv = max_kv_;
-        t = tb;
-        t_begin = tb;
-        t_end = te;
-        seq_start = 0;
-        nb = 0;
-        for (b = 0; b < batch; ++b) {
-            nb = seq_tiles(kv[b], q_len, max_kv);
-            if (seq_start + nb > t) break;
-            seq_start += nb;
+        kv = a.kv_len;
+        batch = a.batch;
+        q_len = a.q_len;
+        max_kv = a.max_kv;
+        t = 0;
+        n = n_tiles;
+        // the sequence holding tile t_begin, 32 sequences at a time (the whole warp)
+        const int lane = threadIdx.x & 31;
+        int64_t before = -t_begin;
+        for (int b0 = 0;; b0 += 32) {
+            const int64_t nt = b0 + lane < batch ? seq_tiles(kv[b0 + lane], q_len, max_kv) : 0;
+            int64_t incl = nt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const unsigned hit = __ballot_sync(0xffffffffu, before + incl > 0);
+            if (hit || b0 + 32 >= batch) {
+                const int src = hit ? __ffs(hit) - 1 : 31;
+                b = b0 + src;
+                nb = static_cast<int>(__shfl_sync(0xffffffffu, nt, src));
+                seq_start = static_cast<int>(before + __shfl_sync(0xffffffffu, incl - nt, src));
+                return;
+            }
+            before += __shfl_sync(0xffffffffu, incl, 31);
         }
     }
-    __device__ bool done() const { return t >= t_end; }
-    __device__ int tile() const { return static_cast<int>(t - seq_start); }
-    __device__ bool first() const { return t == t_begin || t == seq_start; }
-    __device__ bool last() const { return t + 1 == t_end || t + 1 == seq_start + nb; }
-    __device__ bool last_of_partition() const { return t + 1 == t_end; }
+    __device__ bool done() const { return t >= n; }
+    __device__ int tile() const { return t - seq_start; }
+    __device__ bool first() const { return t == 0 || t == seq_start; }
+    __device__ bool last() const { return t + 1 == n || t + 1 == seq_start + nb; }
+    __device__ bool last_of_partition() const { return t + 1 == n; }
+    __device__ bool whole() const { return seq_start >= 0 && seq_start + nb <= n; }  // all its tiles are here
     __device__ void next()
     {
         ++t;
-        if (t < t_end && t >= seq_start + nb) {
+        if (t < n && t >= seq_start + nb) {
             seq_start += nb;
             for (++b; b < batch; ++b) {
-                nb = seq_tiles(kv[b], q_len, max_kv);
+                nb = static_cast<int>(seq_tiles(kv[b], q_len, max_kv));
                 if (nb > 0) break;
             }
         }
     }
 };
 
-// Where the boxes of tile j of sequence b live: a contiguous cache loads
-// the tile as one 128-row box, a paged cache as one 64-row box per page.
+// Where the boxes of a tile live: a contiguous cache loads the tile as one
+// 128-row box, a paged cache as one 64-row box per page.
 struct TileLoc {
     int nh;            // boxes to load (0 if the first page is bad)
     uint32_t bytes;    // bytes the boxes deliver
-    int32_t tok0[2], blk[2];
+    int32_t tok0, blk[2];
 };
 
-__device__ __forceinline__ TileLoc locate(const TcArgs &a, int b, int j)
-{
-    TileLoc L;
-    if (!a.paged) {
-        L.nh = 1;
-        L.bytes = kTile * 128;
-        L.blk[0] = b;
-        L.tok0[0] = j * kTile;
-        return L;
+// The tiles of a partition in order, for a producer warp (the same in every
+// lane).  Page ids are read 32 at a time, one per lane, so that no load from
+// the block table stands between a free slot and its refill.
+struct TileStream {
+    Walk w;
+    TileLoc at;
+    int page_b, page_0, page_id;
+
+    __device__ void init(const TcArgs &a, int64_t t_begin, int n_tiles)
+    {
+        w.init(a, t_begin, n_tiles);
+        page_b = -1;
+        page_0 = page_id = 0;
+        locate(a);
     }
-    const int kv = a.kv_len[b];
-    L.nh = (kv - j * kTile > kHalf) ? 2 : 1;
-    for (int h = 0; h < L.nh; ++h) {
-        const int32_t pg = a.block_table[static_cast<int64_t>(b) * a.bt_stride + 2 * j + h];
-        if (pg < 0 || pg >= a.num_pages) {
-            record_status(a.status, kStatusBounds);
-            L.nh = h;
-            break;
+    __device__ void next(const TcArgs &a)
+    {
+        w.next();
+        if (!w.done()) locate(a);
+    }
+    __device__ void locate(const TcArgs &a)
+    {
+        const int b = w.b, j = w.tile();
+        if (!a.paged) {
+            at.nh = 1;
+            at.bytes = kChunkBytes;
+            at.blk[0] = b;
+            at.tok0 = j * kTile;
+            return;
         }
-        L.blk[h] = pg;
-        L.tok0[h] = 0;
+        const int lane = threadIdx.x & 31;
+        const int pages = (a.kv_len[b] + kHalf - 1) / kHalf;
+        if (b != page_b || 2 * j + 1 >= page_0 + 32) {
+            page_b = b;
+            page_0 = 2 * j;
+            page_id = page_0 + lane < pages ? a.block_table[static_cast<int64_t>(b) * a.bt_stride + page_0 + lane] : 0;
+        }
+        at.nh = pages - 2 * j > 1 ? 2 : 1;
+        at.tok0 = 0;
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            at.blk[h] = __shfl_sync(0xffffffffu, page_id, 2 * j + h - page_0);
+            if (h < at.nh && (at.blk[h] < 0 || at.blk[h] >= a.num_pages)) {
+                if (lane == 0) record_status(a.status, kStatusBounds);
+                at.nh = h;
+            }
+        }
+        at.bytes = static_cast<uint32_t>(at.nh) * kHalf * 128;
     }
-    L.bytes = static_cast<uint32_t>(L.nh) * kHalf * 128;
-    return L;
-}
+};
 
 // A ring position: slot index and how many full passes over the ring came before.
 struct RingPos {
@@ -205,21 +243,51 @@ struct RingPos {
     }
 };
 
-// Non-blocking test: has the phase with this parity completed?
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-
 __device__ __forceinline__ void named_sync_softmax()
 {
     asm volatile("bar.sync 1, %0;" ::"n"(32 * kSoftmaxWarps) : "memory");
+}
+
+// The same barrier with a vote: does any softmax thread pass true?
+__device__ __forceinline__ bool softmax_any(bool p)
+{
+    uint32_t r;
+    asm volatile(
+        "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}\n"
+        : "=r"(r)
+        : "r"(static_cast<uint32_t>(p)), "n"(32 * kSoftmaxWarps)
+        : "memory");
+    return r != 0;
+}
+
+// Two fp32 values in a 64-bit register, and the two-wide operations on them.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi)
+{
+    uint64_t r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+    return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float &lo, float &hi)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c)
+{
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b)
+{
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ float ex2(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
 // Reduce 16 columns over the 32 lanes of a warp: afterwards lane l holds, in
@@ -287,25 +355,24 @@ __device__ __forceinline__ float *lse_rows(const TcArgs &a, int b, int part, boo
 
 // Per-thread constants of a softmax warp.
 struct SmCtx {
-    int lane, tid, quarter, half, tok, n_own, group, part, nrc, ncc, cs, n_items;
+    int lane, tid, quarter, half, tok, n_own, group, part, nrc, n_items;
     uint32_t lane_base, tmem, o_col0;
-    unsigned char *ring, *p_buf;  // p_buf: NP buffers of NB x [128 tok x 32 B]
+    unsigned char *p_buf;  // NP buffers of NB x [128 tok x 32 B]
     uint64_t lim_ns;
-    int64_t t_begin, t_end;
+    int64_t t_begin;
 };
 
-// The whole warp waits; a failure marks sm_fail, which the softmax
-// warps read only after their next named barrier, so they all leave together.
-template <int N>
-__device__ __forceinline__ void sm_wait(const SmCtx &c, const TcArgs &a, Shared<N> &ss, uint64_t *bar,
+// The whole warp waits; once a wait has run out the warp waits no more, and the
+// softmax warps leave together at their next vote (softmax_any).
+__device__ __forceinline__ void sm_wait(const SmCtx &c, const TcArgs &a, int *abort, bool &failed, uint64_t *bar,
                                         uint32_t parity)
 {
-    if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(bar), parity, c.lim_ns)) && c.lane == 0) {
+    if (failed || mbar_wait_warp(smem_u32(bar), parity, c.lim_ns)) return;
+    failed = true;
+    if (c.lane == 0) {
         record_status(a.status, kStatusTimeout);
-        atomicOr(&ss.sm_fail, 1);
-        ss.abort = 1;
+        *abort = 1;
     }
-    __syncwarp();
 }
 
 // Scores of one 16-column block in the log2 domain, masked where needed.
@@ -341,12 +408,12 @@ __device__ __forceinline__ void sm_block_max(const SmCtx &c, const TcArgs &a, Sh
 // Normalised partial output and log-sum-exp of sequence b, whose last tile
 // in this partition was t_end_seg, in one step (one O^T buffer).
 template <int N, int KOWN>
-__device__ __forceinline__ void sm_epilogue(const SmCtx &c, const TcArgs &a, Shared<N> &ss, Bars &bars,
-                                            float (&l_part)[KOWN][16], int b, int64_t t_end_seg, bool whole)
+__device__ __forceinline__ bool sm_epilogue(const SmCtx &c, const TcArgs &a, Shared<N> &ss, Bars &bars,
+                                            uint64_t (&l_part)[KOWN][8], int b, int t_end_seg, bool whole,
+                                            bool &failed)
 {
-    sm_wait<N>(c, a, ss, &bars.pv_done[t_end_seg % kPBufs<N>], static_cast<uint32_t>((t_end_seg / kPBufs<N>) & 1));
-    named_sync_softmax();
-    if (ss.sm_fail) return;
+    sm_wait(c, a, &ss.abort, failed, &bars.pv_done[t_end_seg % kPBufs<N>], static_cast<uint32_t>((t_end_seg / kPBufs<N>) & 1));
+    if (softmax_any(failed)) return false;
     tc::fence_after_sync();
 #pragma unroll
     for (int ob = 0; ob < KOWN; ++ob) {
@@ -354,7 +421,7 @@ __device__ __forceinline__ void sm_epilogue(const SmCtx &c, const TcArgs &a, Sha
             const int cb = c.half + 3 * ob;
             float v[16];
 #pragma unroll
-            for (int e = 0; e < 16; ++e) v[e] = l_part[ob][e];
+            for (int e = 0; e < 8; ++e) unpack2(l_part[ob][e], v[2 * e], v[2 * e + 1]);
             const float ls = reduce16<false>(v, c.lane);
             if (c.lane < 16) ss.red[c.quarter][cb * 16 + c.lane] = ls;
         }
@@ -394,12 +461,13 @@ __device__ __forceinline__ void sm_epilogue(const SmCtx &c, const TcArgs &a, Sha
     tc::fence_before_sync();
     __syncwarp();
     if (c.lane == 0) tc::mbar_arrive(smem_u32(&bars.o_free));
+    return true;
 }
 
 // Closing a sequence b of this partition (no wait on its value products):
 // its softmax denominators (1 / l kept for the drain) and its log-sum-exp.
 template <int N, int KOWN>
-__device__ __forceinline__ void sm_close(const SmCtx &c, const TcArgs &a, Shared<N> &ss, float (&l_part)[KOWN][16],
+__device__ __forceinline__ void sm_close(const SmCtx &c, const TcArgs &a, Shared<N> &ss, uint64_t (&l_part)[KOWN][8],
                                          int b, bool whole)
 {
 #pragma unroll
@@ -408,7 +476,7 @@ __device__ __forceinline__ void sm_close(const SmCtx &c, const TcArgs &a, Shared
             const int cb = c.half + 3 * ob;
             float v[16];
 #pragma unroll
-            for (int e = 0; e < 16; ++e) v[e] = l_part[ob][e];
+            for (int e = 0; e < 8; ++e) unpack2(l_part[ob][e], v[2 * e], v[2 * e + 1]);
             const float ls = reduce16<false>(v, c.lane);
             if (c.lane < 16) ss.red[c.quarter][cb * 16 + c.lane] = ls;
         }
@@ -428,12 +496,11 @@ __device__ __forceinline__ void sm_close(const SmCtx &c, const TcArgs &a, Shared
 // The normalised partial output of sequence b (closed by sm_close), whose
 // last tile here was t_end_seg, from O^T buffer obuf; then the buffer is free.
 template <int N, int KOWN>
-__device__ __forceinline__ void sm_drain(const SmCtx &c, const TcArgs &a, Shared<N> &ss, BarsT<N> &bars, int b,
-                                         int64_t t_end_seg, int obuf, bool whole)
+__device__ __forceinline__ bool sm_drain(const SmCtx &c, const TcArgs &a, Shared<N> &ss, BarsT<N> &bars, int b,
+                                         int t_end_seg, int obuf, bool whole, bool &failed)
 {
-    sm_wait<N>(c, a, ss, &bars.pv_done[t_end_seg % kPBufs<N>], static_cast<uint32_t>((t_end_seg / kPBufs<N>) & 1));
-    named_sync_softmax();
-    if (ss.sm_fail) return;
+    sm_wait(c, a, &ss.abort, failed, &bars.pv_done[t_end_seg % kPBufs<N>], static_cast<uint32_t>((t_end_seg / kPBufs<N>) & 1));
+    if (softmax_any(failed)) return false;
     tc::fence_after_sync();
     const int valid_cols = a.rows - c.group * N;  // columns past it are padding
     float *out = out_rows(a, b, c.part, whole) + static_cast<int64_t>(c.group) * N * a.rank + c.tok;
@@ -456,125 +523,148 @@ __device__ __forceinline__ void sm_drain(const SmCtx &c, const TcArgs &a, Shared
     tc::fence_before_sync();
     __syncwarp();
     if (c.lane == 0) tc::mbar_arrive(smem_u32(o_free_bar(bars, obuf)));
+    return true;
 }
 
+// Exponents s scale - m of one 16-column block (log2 domain, pairs of columns),
+// masked where needed; returns their maximum.
+template <int N>
+__device__ __forceinline__ float sm_exponents(const TcArgs &a, const Shared<N> &ss, uint32_t s_base, int cb, int pos,
+                                              bool need_mask, uint64_t (&x)[8])
+{
+    uint32_t r[16];
+    tc::ld_32x32b_x16(s_base + cb * 16, r);
+    const float4 *nm = reinterpret_cast<const float4 *>(ss.neg_m + cb * 16);
+    const uint64_t scale = pack2(a.scale_log2, a.scale_log2);
+    tc::wait_ld();
+    float mx = -INFINITY;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const float4 m = nm[q];
+        x[2 * q] = fma2(pack2(__uint_as_float(r[4 * q]), __uint_as_float(r[4 * q + 1])), scale, pack2(m.x, m.y));
+        x[2 * q + 1] = fma2(pack2(__uint_as_float(r[4 * q + 2]), __uint_as_float(r[4 * q + 3])), scale, pack2(m.z, m.w));
+    }
+    if (need_mask) {
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            float lo, hi;
+            unpack2(x[e], lo, hi);
+            if (pos > ss.lim[cb * 16 + 2 * e]) lo = -INFINITY;
+            if (pos > ss.lim[cb * 16 + 2 * e + 1]) hi = -INFINITY;
+            x[e] = pack2(lo, hi);
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        float lo, hi;
+        unpack2(x[e], lo, hi);
+        mx = fmaxf(mx, fmaxf(lo, hi));
+    }
+    return mx;
+}
+
+// Online softmax of the partition's tiles.  Per tile each thread reads its
+// scores from TMEM once, as exponents over the column's base m; one barrier
+// carries the vote on whether a base has to move (a score above it by more
+// than 2^8, or a sequence's first tile), which is the only other reason to
+// meet.  (Two passes over TMEM, exp2f of scalar arithmetic and five barriers a
+// tile took 7500 cycles a tile at N = 80, twice the tensor pipe's share.)
 template <int N>
 __device__ __forceinline__ void softmax_role(const SmCtx &c, const TcArgs &a, Shared<N> &ss, BarsT<N> &bars)
 {
     constexpr int NB = N / 16;
     constexpr int KOWN = (NB + 2) / 3;
-    float l_part[KOWN][16];
+    constexpr int NP = kPBufs<N>;
+    uint64_t l_part[KOWN][8];  // running sums of the weights, pairs of columns, over this thread's tokens
     // the sequence open here, with kWhole set when all its tiles lie in this
     // partition (its rows then go to the final buffers, when given)
     int b_cur = -1;
     int u = -1;  // sequences begun here (the PV warp counts the same ones)
-    int64_t t_prev = -1;  // the previous tile (one O^T buffer: the drain runs at the next sequence's first tile)
+    int t_prev = -1;  // the previous tile (one O^T buffer: the drain runs at the next sequence's first tile)
     // a closed sequence whose drain waits for the next sequence's first P (two O^T buffers)
     int d_b = -1, d_t = -1;
+    bool failed = false, stop = false;
     const int cc = c.tid - kSoftmaxBase;
     Walk w;
-    w.init(a.kv_len, a.batch, a.q_len, a.max_kv, c.t_begin, c.t_end);
-    for (int64_t t = 0; !w.done(); ++t, w.next()) {
+    w.init(a, c.t_begin, c.n_items);
+    for (; !w.done(); w.next()) {
+        const int t = w.t;
         const bool first = w.first(), last = w.last();
         const int b = w.b, j = w.tile();
         const int kv = a.kv_len[b];
         const int sb = static_cast<int>(t & 1);
-        sm_wait<N>(c, a, ss, &bars.s_full[sb], static_cast<uint32_t>((t >> 1) & 1));
-        named_sync_softmax();
-        if (ss.sm_fail) break;
+        sm_wait(c, a, &ss.abort, failed, &bars.s_full[sb], static_cast<uint32_t>((t >> 1) & 1));
         tc::fence_after_sync();
         if (first) {
             if constexpr (kOBufs<N> == 1) {
-                if (b_cur >= 0) {
-                    sm_epilogue<N, KOWN>(c, a, ss, bars, l_part, b_cur & ~kWhole, t_prev, (b_cur & kWhole) != 0);
-                    if (ss.sm_fail) break;
+                if (b_cur >= 0 && !sm_epilogue<N, KOWN>(c, a, ss, bars, l_part, b_cur & ~kWhole, t_prev,
+                                                        (b_cur & kWhole) != 0, failed)) {
+                    stop = true;
+                    break;
                 }
             }
-            b_cur = b | (w.seq_start >= w.t_begin && w.seq_start + w.nb <= w.t_end ? kWhole : 0);
+            b_cur = b | (w.whole() ? kWhole : 0);
             ++u;
 #pragma unroll
             for (int ob = 0; ob < KOWN; ++ob)
 #pragma unroll
-                for (int e = 0; e < 16; ++e) l_part[ob][e] = 0.f;
+                for (int e = 0; e < 8; ++e) l_part[ob][e] = 0;
             if (cc < N) {
                 const int row = c.group * N + cc;
                 ss.lim[cc] = row < a.rows ? kv - a.q_len + row / a.heads : -1;
             }
-            named_sync_softmax();
         }
         t_prev = t;
         const int pos = j * kTile + c.tok;
         // the mask matters only where a token lies past the earliest query's last key
         const bool need_mask = j * kTile + kTile - 1 > kv - a.q_len;
         const uint32_t s_base = c.tmem + c.lane_base + sb * N;
-        // ---- pass 1: exponent bases (exact column maxima on a sequence's first
-        // tile, else only when a score passes the current base by more than 2^8)
-        if (first) {
+        uint64_t x[KOWN][8];
+        bool moved = false;
+#pragma unroll 1
+        for (bool move = first;; move = false, moved = true) {
+            float mx = -INFINITY;
+            if (!move) {
+#pragma unroll
+                for (int ob = 0; ob < KOWN; ++ob)
+                    if (ob < c.n_own)
+                        mx = fmaxf(mx, sm_exponents<N>(a, ss, s_base, c.half + 3 * ob, pos, need_mask, x[ob]));
+            }
+            if (moved || !softmax_any(move || mx > 8.f || failed)) break;
+            // ---- bases: exact column maxima on a sequence's first tile, else
+            // raised where a score passed by more than 2^8
+            if (softmax_any(failed)) {
+                stop = true;
+                break;
+            }
             sm_block_max<N, KOWN>(c, a, ss, s_base, pos, need_mask);
             named_sync_softmax();
             if (cc < N) {
-                ss.m_used[cc] = fmaxf(fmaxf(ss.red[0][cc], ss.red[1][cc]), fmaxf(ss.red[2][cc], ss.red[3][cc]));
-                ss.alpha[cc] = 1.f;
-            }
-            if (c.tid == kSoftmaxBase) ss.any_rescale = 0;
-        } else {
-            bool over = false;
-#pragma unroll
-            for (int ob = 0; ob < KOWN; ++ob) {
-                if (ob < c.n_own) {
-                    const int cb = c.half + 3 * ob;
-                    float s[16];
-                    sm_scores<N>(a, ss, s_base, cb, pos, need_mask, s);
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) over |= s[e] > ss.m_used[cb * 16 + e] + 8.f;
+                const float tmax = fmaxf(fmaxf(ss.red[0][cc], ss.red[1][cc]), fmaxf(ss.red[2][cc], ss.red[3][cc]));
+                float m = first ? tmax : ss.m_used[cc], alpha = 1.f;
+                if (!first && tmax != -INFINITY && (m == -INFINITY || tmax > m + 8.f)) {
+                    alpha = m == -INFINITY ? 0.f : ex2(m - tmax);
+                    m = tmax;
                 }
+                ss.m_used[cc] = m;
+                ss.neg_m[cc] = m == -INFINITY ? 0.f : -m;
+                ss.alpha[cc] = alpha;
             }
-            if (__any_sync(0xffffffffu, over) && c.lane == 0) ss.need_max = 1;
             named_sync_softmax();
-            if (ss.need_max) {  // uniform: written before the barrier, read after it
-                sm_block_max<N, KOWN>(c, a, ss, s_base, pos, need_mask);
-                named_sync_softmax();
-                if (cc < N) {
-                    const float tmax = fmaxf(fmaxf(ss.red[0][cc], ss.red[1][cc]), fmaxf(ss.red[2][cc], ss.red[3][cc]));
-                    const float m_old = ss.m_used[cc];
-                    float alpha = 1.f;
-                    if (tmax != -INFINITY && (m_old == -INFINITY || tmax > m_old + 8.f)) {
-                        alpha = m_old == -INFINITY ? 0.f : exp2f(m_old - tmax);
-                        ss.m_used[cc] = tmax;
-                    }
-                    ss.alpha[cc] = alpha;
-                }
-                if (c.tid == kSoftmaxBase) {
-                    ss.any_rescale = 1;
-                    ss.need_max = 0;
-                }
-            } else if (c.tid == kSoftmaxBase) {
-                ss.any_rescale = 0;
-            }
-        }
-        named_sync_softmax();
-        // ---- P(t) goes to buffer t % NP, free again once PV(t - NP) has
-        // completed; O^T is rescaled (rarely: only when a base moves) once
-        // PV(t-1) has completed.  Each wait is on the next phase of its barrier.
-        constexpr int NP = kPBufs<N>;
-        if (t >= NP) sm_wait<N>(c, a, ss, &bars.pv_done[t % NP], static_cast<uint32_t>(((t - NP) / NP) & 1));
-        if (ss.any_rescale)  // never on a sequence's first tile
-            sm_wait<N>(c, a, ss, &bars.pv_done[(t - 1) % NP], static_cast<uint32_t>(((t - 1) / NP) & 1));
-        named_sync_softmax();
-        if (ss.sm_fail) break;
-        tc::fence_after_sync();
-        {
-            if (ss.any_rescale) {
+            if (!first) {
+                // O^T is rescaled once PV(t-1) has completed
+                sm_wait(c, a, &ss.abort, failed, &bars.pv_done[(t - 1) % NP], static_cast<uint32_t>(((t - 1) / NP) & 1));
+                tc::fence_after_sync();
 #pragma unroll
                 for (int ob = 0; ob < KOWN; ++ob) {
                     if (ob < c.n_own) {
                         const int cb = c.half + 3 * ob;
                         float al[16];
 #pragma unroll
-                        for (int e = 0; e < 16; ++e) {
-                            al[e] = ss.alpha[cb * 16 + e];
-                            l_part[ob][e] *= al[e];
-                        }
+                        for (int e = 0; e < 16; ++e) al[e] = ss.alpha[cb * 16 + e];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) l_part[ob][e] = fma2(l_part[ob][e], pack2(al[2 * e], al[2 * e + 1]), 0);
+#pragma unroll 1
                         for (int m = 0; m < c.nrc; ++m) {
                             const uint32_t ta = c.tmem + c.lane_base + c.o_col0 +
                                                 static_cast<uint32_t>((u % kOBufs<N>) * 4 * N + m * N + cb * 16);
@@ -588,36 +678,39 @@ __device__ __forceinline__ void softmax_role(const SmCtx &c, const TcArgs &a, Sh
                 }
             }
         }
-        // ---- pass 2: P = 2^(s - m) in bf16 (MN-major, 16-column SW32 atoms), running sums
+        if (stop) break;
+        tc::fence_before_sync();
+        __syncwarp();
+        if (c.lane == 0) tc::mbar_arrive(smem_u32(&bars.s_free[sb]));  // S(t) is in registers
+        // ---- P(t) = 2^x in bf16 (MN-major, 16-column SW32 atoms) into buffer
+        // t % NP, free again once PV(t - NP) has completed; running sums.
+        // Each wait is on the next phase of its barrier.
+        if (t >= NP)
+            sm_wait(c, a, &ss.abort, failed, &bars.pv_done[t % NP], static_cast<uint32_t>(((t - NP) / NP) & 1));
 #pragma unroll
         for (int ob = 0; ob < KOWN; ++ob) {
             if (ob < c.n_own) {
                 const int cb = c.half + 3 * ob;
-                float s[16];
-                sm_scores<N>(a, ss, s_base, cb, pos, need_mask, s);
                 uint32_t pk[8];
 #pragma unroll
-                for (int e = 0; e < 16; e += 2) {
-                    const float p0 = s[e] == -INFINITY ? 0.f : exp2f(s[e] - ss.m_used[cb * 16 + e]);
-                    const float p1 = s[e + 1] == -INFINITY ? 0.f : exp2f(s[e + 1] - ss.m_used[cb * 16 + e + 1]);
-                    const __nv_bfloat162 pb = __floats2bfloat162_rn(p0, p1);
-                    l_part[ob][e] += __low2float(pb);  // the weights the MMA multiplies by
-                    l_part[ob][e + 1] += __high2float(pb);
-                    pk[e / 2] = *reinterpret_cast<const uint32_t *>(&pb);
+                for (int e = 0; e < 8; ++e) {
+                    float lo, hi;
+                    unpack2(x[ob][e], lo, hi);
+                    const __nv_bfloat162 pb = __floats2bfloat162_rn(ex2(lo), ex2(hi));
+                    pk[e] = *reinterpret_cast<const uint32_t *>(&pb);
+                    // the weights the MMA multiplies by
+                    l_part[ob][e] = add2(l_part[ob][e], pack2(__uint_as_float(pk[e] << 16), __uint_as_float(pk[e] & 0xffff0000u)));
                 }
-                unsigned char *row = c.p_buf + (t % kPBufs<N>) * (N / 16) * (kTile * 32) + cb * (kTile * 32) + c.tok * 32;
+                unsigned char *row = c.p_buf + (t % NP) * (N / 16) * (kTile * 32) + cb * (kTile * 32) + c.tok * 32;
                 const int sw = (c.tok >> 2) & 1;
                 *reinterpret_cast<uint4 *>(row + (sw * 16)) = make_uint4(pk[0], pk[1], pk[2], pk[3]);
                 *reinterpret_cast<uint4 *>(row + ((1 ^ sw) * 16)) = make_uint4(pk[4], pk[5], pk[6], pk[7]);
             }
         }
-        tc::fence_before_sync();
-        __syncwarp();
-        if (c.lane == 0) tc::mbar_arrive(smem_u32(&bars.s_free[sb]));
         tc::fence_proxy_async_smem();
         tc::fence_before_sync();
         __syncwarp();
-        if (c.lane == 0) tc::mbar_arrive(smem_u32(&bars.p_full[t % kPBufs<N>]));
+        if (c.lane == 0) tc::mbar_arrive(smem_u32(&bars.p_full[t % NP]));
         if constexpr (kOBufs<N> == 2) {
             // Due now, in this order: the previous sequence's drain (deferred
             // until this first P was out, so that it overlaps this tile's value
@@ -647,17 +740,19 @@ __device__ __forceinline__ void softmax_role(const SmCtx &c, const TcArgs &a, Sh
                 }
                 if (db >= 0) {
                     named_sync_softmax();
-                    sm_drain<N, KOWN>(c, a, ss, bars, db & ~kWhole, dt, dbuf, (db & kWhole) != 0);
-                    if (ss.sm_fail) break;
+                    if (!sm_drain<N, KOWN>(c, a, ss, bars, db & ~kWhole, dt, dbuf, (db & kWhole) != 0, failed)) {
+                        stop = true;
+                        break;
+                    }
                 }
             }
-            if (ss.sm_fail) break;
+            if (stop) break;
         }
     }
     named_sync_softmax();
     if constexpr (kOBufs<N> == 1) {
-        if (b_cur >= 0 && !ss.sm_fail)
-            sm_epilogue<N, KOWN>(c, a, ss, bars, l_part, b_cur & ~kWhole, t_prev, (b_cur & kWhole) != 0);
+        if (b_cur >= 0 && !stop)
+            sm_epilogue<N, KOWN>(c, a, ss, bars, l_part, b_cur & ~kWhole, t_prev, (b_cur & kWhole) != 0, failed);
     }
 }
 
@@ -715,10 +810,7 @@ __global__ void __maxnreg__(128)
         if constexpr (kOBufs<N> == 2) mbar_init(o_free_bar(bars, 1), kSoftmaxWarps);
         mbar_init(&bars.drain_qk, 1);
         mbar_init(&bars.drain_pv, 1);
-        ss.need_max = 0;
-        ss.any_rescale = 0;
         ss.abort = 0;
-        ss.sm_fail = 0;
         tc::fence_barrier_init();
     }
     if (warp == 1) {
@@ -757,135 +849,103 @@ __global__ void __maxnreg__(128)
 
     if (warp == 0 || warp == 3) {
         // ================================================================ TMA producers
-        // A tensor-TMA instruction occupies its issuing thread for a long,
-        // nearly size-independent time, so the loads are spread over lanes
-        // and warps, each lane an independent in-order stream.  Warp 0: lane
-        // s < CA refills QK-ring slot s (chunks s, s + CA, ... of the QK pass,
-        // nqc per tile: positional keys, then the latent chunks) -- with
-        // streamed queries the chunk's cache box(es) and then its query box
-        // (the first pass's query box waits for the next pass, after
-        // griddepcontrol.wait); with resident queries lanes 16..16+ncc load
-        // the query boxes of each sequence.  Warp 3: lane s < CB refills
-        // PV-ring slot s (chunks s, s + CB, ... of the PV pass, ncc per
-        // tile).  The lanes of a warp poll their own barrier without
-        // blocking in one converged loop, and every lane whose slot is free
-        // issues in the same pass.  A lane waits only on phases of its own
-        // barrier, in order, so every parity test is on the next phase.
+        // Warp 0 refills the QK ring (nqc chunks per tile: positional keys,
+        // then the latent chunks; with streamed queries each chunk's query box
+        // behind it), warp 3 the PV ring (the ncc latent chunks again).  Each
+        // runs its ring in order with the whole warp converged and one elected
+        // lane issuing; what a load needs besides a free slot is known a tile
+        // ahead.  (One such warp fills 117 GB/s per SM from L2 and saturates
+        // HBM with 64 KB in flight.  A lane per slot, polling and computing
+        // its coordinates by division when its slot came free, kept every slot
+        // 2.5 us from release to refilled: 67 GB/s.)
         if (n_items > 0) {
-            if (lane == 0 && warp == 0) {
+            const bool is_qk = warp == 0;
+            if (is_qk) {
                 tc::prefetch_tensormap(&map_c);
                 tc::prefetch_tensormap(&map_r);
                 tc::prefetch_tensormap(&map_q);
             }
-            enum { kQK, kPV, kQuery, kIdle };
-            const int kind = warp == 3 ? (lane < CB ? kPV : kIdle)
-                                       : (lane < CA ? kQK : (!SQ && lane >= 16 && lane < 16 + nqc) ? kQuery : kIdle);
-            const int slot = lane;
-            const int per_tile = kind == kQK ? nqc : ncc;
-            const int ring_len = kind == kQK ? CA : CB;
-            Walk w;
-            w.init(a.kv_len, a.batch, a.q_len, a.max_kv, t_begin, t_end);
-            const int64_t total = static_cast<int64_t>(n_items) * per_tile;
-            int64_t c = slot;  // ring lanes: next chunk of this lane's pass
-            int64_t k = 0;     // jobs this lane has issued (ring round / sequence)
-            bool has = (kind == kQK || kind == kPV) ? c < total : kind == kQuery;
-            bool ok = true;
-            uint64_t wait_t0 = 0;
-            // griddepcontrol.wait still to do before the first query load
-            bool q_pending = SQ ? kind == kQK : kind == kQuery;
-            // streamed queries: the query box of the chunk issued in the first
-            // pass, which waits for that pass's griddepcontrol.wait
-            bool q_owed = false;
-            int q_owed_x = 0, q_owed_y = 0;
-            bool first_pass = true;           // the ring lanes issue their first cache loads in it
+            // the QK pass keeps latent lines in L2 for the PV pass, which reads
+            // them a last time; the positional keys are read once
             const uint64_t pol_keep = tc::policy_evict_last(), pol_drop = tc::policy_evict_first();
-            uint32_t wbar = 0, fbar = 0, dst = 0;
-            if (kind == kQK) {
-                wbar = smem_u32(&bars.qk_empty[slot]);
-                fbar = smem_u32(&bars.qk_full[slot]);
-                dst = smem_u32(ring_a + slot * kSlotA);
-            } else if (kind == kPV) {
-                wbar = smem_u32(&bars.pv_empty[slot]);
-                fbar = smem_u32(&bars.pv_full[slot]);
-                dst = smem_u32(ring_b + slot * kChunkBytes);
-            } else if (kind == kQuery) {
-                wbar = smem_u32(&bars.q_free);
-                fbar = smem_u32(&bars.q_full);
-                dst = smem_u32(q_buf + (lane - 16) * N * 128);
-            }
-            while (true) {
-                if (kind == kQuery) has = has && !w.done();
-                if (!__any_sync(0xffffffffu, (has || q_owed) && ok)) break;
-                if (any_abort()) break;
-                bool progressed = false;
-                if (q_pending && !first_pass) {
-                    griddep_wait();
-                    q_pending = false;
-                    if (SQ && q_owed) {
-                        tc::tma_load_2d_hint(dst + kChunkBytes, &map_q, q_owed_x, q_owed_y, fbar, pol_keep);
-                        q_owed = false;
-                        progressed = true;
+            bool ok = true;
+            RingPos rp{0, 0};
+            TileStream ts;
+            ts.init(a, t_begin, n_items);
+            if (is_qk) {
+                const uint32_t ring = smem_u32(ring_a);
+                auto cache_box = [&](int i) {  // chunk i of the tile into the slot at rp
+                    const uint32_t full = smem_u32(&bars.qk_full[rp.slot]), dst = ring + rp.slot * kSlotA;
+                    tc::mbar_arrive_expect_tx_elect(full, ts.at.bytes + (SQ ? N * 128 : 0));
+                    const CUtensorMap *map = i == 0 ? &map_r : &map_c;
+                    const int col = i == 0 ? 0 : 64 * (i - 1);
+                    const uint64_t pol = i == 0 ? pol_drop : pol_keep;
+                    if (ts.at.nh > 0) tc::tma_load_3d_hint_elect(dst, map, col, ts.at.tok0, ts.at.blk[0], full, pol);
+                    if (ts.at.nh > 1)
+                        tc::tma_load_3d_hint_elect(dst + kHalf * 128, map, col, ts.at.tok0, ts.at.blk[1], full, pol);
+                };
+                // the query columns chunk i multiplies: the positional part lies
+                // behind the latent part in each query row
+                auto query_box = [&](int i, int slot, int b) {
+                    tc::tma_load_2d_hint_elect(ring + slot * kSlotA + kChunkBytes, &map_q, 64 * (i == 0 ? ncc : i - 1),
+                                               b * a.rows + group * N, smem_u32(&bars.qk_full[slot]), pol_keep);
+                };
+                // The ring's first round: its cache boxes go out before the
+                // previous launch (which writes the queries) has completed.
+                const int64_t total = static_cast<int64_t>(n_items) * nqc;
+                const int head = total < CA ? static_cast<int>(total) : CA;
+                int i = 0;
+                for (; rp.slot < head && rp.round == 0; rp.advance(CA)) {
+                    cache_box(i);
+                    if (++i == nqc) {
+                        i = 0;
+                        ts.next(a);
                     }
                 }
-                if (has && ok && !(kind == kQuery && q_pending)) {
-                    const bool ready = k == 0 || mbar_test(wbar, static_cast<uint32_t>((k - 1) & 1));
-                    if (!ready) {
-                        const uint64_t now = global_ns();
-                        if (wait_t0 == 0)
-                            wait_t0 = now;
-                        else if (now - wait_t0 > lim_ns)
-                            ok = false;
-                    } else {
-                        wait_t0 = 0;
-                        progressed = true;
-                        if (kind == kQuery) {
-                            const int box = lane - 16;
-                            if (box == 0) tc::mbar_arrive_expect_tx(fbar, nqc * N * 128);
-                            tc::tma_load_2d(dst, &map_q, 64 * box, w.b * a.rows + group * N, fbar);
-                            do {
-                                w.next();
-                            } while (!w.done() && !w.first());
-                        } else {
-                            const int64_t tile = c / per_tile;
-                            const int i = static_cast<int>(c - tile * per_tile);
-                            while (w.t < t_begin + tile) w.next();
-                            const TileLoc L = locate(a, w.b, w.tile());
-                            // QK pass: chunk 0 = positional keys, 1.. = latent; PV pass: latent
-                            const bool keys = kind == kQK && i == 0;
-                            const CUtensorMap *map = keys ? &map_r : &map_c;
-                            const int col = keys ? 0 : 64 * (kind == kQK ? i - 1 : i);
-                            const bool sq = SQ && kind == kQK;
-                            tc::mbar_arrive_expect_tx(fbar, L.bytes + (sq ? N * 128 : 0));
-                            // the QK pass keeps latent lines in L2 for the PV pass, which reads
-                            // them a last time; the positional keys are read once
-                            const uint64_t pol = (kind == kQK && !keys) ? pol_keep : pol_drop;
-                            for (int h = 0; h < L.nh; ++h)
-                                tc::tma_load_3d_hint(dst + h * kHalf * 128, map, col, L.tok0[h], L.blk[h], fbar,
-                                                     pol);
-                            if (sq) {
-                                // the query columns this chunk multiplies: the positional
-                                // part behind the latent part in each query row
-                                const int qx = 64 * (keys ? ncc : i - 1);
-                                const int qy = w.b * a.rows + group * N;
-                                if (q_pending) {
-                                    q_owed = true;
-                                    q_owed_x = qx;
-                                    q_owed_y = qy;
-                                } else {
-                                    tc::tma_load_2d_hint(dst + kChunkBytes, &map_q, qx, qy, fbar, pol_keep);
-                                }
-                            }
-                            c += ring_len;
-                            has = c < total;
+                griddep_wait();
+                if constexpr (SQ) {
+                    Walk w;
+                    w.init(a, t_begin, n_items);
+                    for (int s = 0, k = 0; s < head; ++s) {
+                        query_box(k, s, w.b);
+                        if (++k == nqc) {
+                            k = 0;
+                            w.next();
                         }
-                        ++k;
                     }
                 }
-                if (!__any_sync(0xffffffffu, progressed)) __nanosleep(32);
-                first_pass = false;
+                while (!ts.w.done() && ok && !any_abort()) {
+                    for (; i < nqc; ++i) {
+                        ok = mbar_wait_warp(smem_u32(&bars.qk_empty[rp.slot]), (rp.round - 1) & 1, lim_ns);
+                        if (!ok) break;
+                        cache_box(i);
+                        if constexpr (SQ) query_box(i, rp.slot, ts.w.b);
+                        rp.advance(CA);
+                    }
+                    i = 0;
+                    ts.next(a);
+                }
+            } else {
+                const uint32_t ring = smem_u32(ring_b);
+                for (; !ts.w.done() && ok && !any_abort(); ts.next(a)) {
+                    for (int m = 0; m < nrc; ++m, rp.advance(CB / 2)) {
+                        const uint32_t full = smem_u32(&bars.pv_full[rp.slot]), dst = ring + rp.slot * 2 * kChunkBytes;
+                        ok = rp.round == 0 || mbar_wait_warp(smem_u32(&bars.pv_empty[rp.slot]), (rp.round - 1) & 1, lim_ns);
+                        if (!ok) break;
+                        tc::mbar_arrive_expect_tx_elect(full, 2 * ts.at.bytes);
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) {
+                            if (ts.at.nh > 0)
+                                tc::tma_load_3d_hint_elect(dst + k * kChunkBytes, &map_c, 64 * (2 * m + k), ts.at.tok0,
+                                                           ts.at.blk[0], full, pol_drop);
+                            if (ts.at.nh > 1)
+                                tc::tma_load_3d_hint_elect(dst + k * kChunkBytes + kHalf * 128, &map_c, 64 * (2 * m + k),
+                                                           ts.at.tok0, ts.at.blk[1], full, pol_drop);
+                        }
+                    }
+                }
             }
-            if (q_pending) griddep_wait();  // (no query was loaded: keep the wait before leaving)
-            if (!ok) {
+            if (!ok && lane == 0) {
                 record_status(a.status, kStatusTimeout);
                 ss.abort = 1;
             }
@@ -909,15 +969,13 @@ __global__ void __maxnreg__(128)
                 return tmpl | static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
             };
             Walk w;
-            w.init(a.kv_len, a.batch, a.q_len, a.max_kv, t_begin, t_end);
+            w.init(a, t_begin, n_items);
             RingPos rp{0, 0};
             bool ok = true;
             auto wait = [&](uint64_t *bar, uint32_t parity) {
-                if (ok) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(bar), parity, lim_ns));
+                if (ok) ok = mbar_wait_warp(smem_u32(bar), parity, lim_ns);
                 return ok;
             };
-            // a consumed slot is handed back to its producer lane
-            auto release = [&](uint64_t *bar) { tc::commit_elect(smem_u32(bar)); };
             if (is_qk) {
                 const uint32_t id_qk = tc::idesc_bf16_f32(128, N, false, false);
                 const uint32_t ring_base = smem_u32(ring_a);
@@ -925,7 +983,15 @@ __global__ void __maxnreg__(128)
                 for (int t = 0; t < n_items && ok; ++t, w.next()) {
                     if (any_abort()) break;
                     if (!SQ && w.first()) {
+                        // resident queries: this warp's products of the last sequence
+                        // have read the buffer (q_free); load the next one's
                         ++seg;
+                        if (seg == 0) griddep_wait();
+                        if (seg > 0 && !wait(&bars.q_free, (seg - 1) & 1)) break;
+                        tc::mbar_arrive_expect_tx_elect(smem_u32(&bars.q_full), nqc * N * 128);
+                        for (int i = 0; i < nqc; ++i)
+                            tc::tma_load_2d_hint_elect(q_base + i * N * 128, &map_q, 64 * i, w.b * a.rows + group * N,
+                                                       smem_u32(&bars.q_full), tc::policy_evict_first());
                         if (!wait(&bars.q_full, seg & 1)) break;
                     }
                     const int sb = t & 1;
@@ -936,11 +1002,9 @@ __global__ void __maxnreg__(128)
                         tc::fence_after_sync();
                         const uint32_t cb = ring_base + rp.slot * kSlotA;
                         const uint32_t qb = SQ ? cb + kChunkBytes : q_base + (i == 0 ? ncc : i - 1) * N * 128;
-#pragma unroll
-                        for (int kk = 0; kk < 4; ++kk)
-                            tc::mma_bf16_elect(d_s, with_addr(dq, cb + kk * 32), with_addr(dq, qb + kk * 32), id_qk,
-                                               (i | kk) != 0);
-                        release(&bars.qk_empty[rp.slot]);
+                        // four steps of 16 columns (32 bytes); then the slot goes back
+                        tc::mma4_bf16_commit_elect(d_s, with_addr(dq, cb), with_addr(dq, qb), id_qk, i != 0, 2, 2,
+                                                   smem_u32(&bars.qk_empty[rp.slot]));
                         rp.advance(CA);
                     }
                     if (!ok) break;
@@ -972,33 +1036,35 @@ __global__ void __maxnreg__(128)
                     const int v = a.kv_len[w.b] - w.tile() * kTile;
                     const bool tail = w.last() && v < kTile;
                     const int v16 = tail ? (v + 15) / 16 * 16 : kTile;
-                    for (int m = 0; m < nrc && ok; ++m) {
-                        // chunks 2m, 2m+1 sit in adjacent slots (CB and ncc are even)
-                        const int s0 = rp.slot;
-                        if (!wait(&bars.pv_full[s0], rp.round & 1) || !wait(&bars.pv_full[s0 + 1], rp.round & 1)) break;
+                    const uint32_t pb = p_base + (t % kPBufs<N>) * (N / 16) * (kTile * 32);
+                    for (int m = 0; m < nrc && ok; ++m, rp.advance(CB / 2)) {
+                        // ring entry: chunks 2m and 2m + 1, side by side
+                        if (!wait(&bars.pv_full[rp.slot], rp.round & 1)) break;
                         tc::fence_after_sync();
+                        unsigned char *entry = ring_b + rp.slot * 2 * kChunkBytes;
                         if (v16 > v) {
                             const int nz = (v16 - v) * 8;  // 16-byte pieces per chunk
                             for (int idx = lane; idx < 2 * nz; idx += 32) {
                                 const int k = idx / nz, r = idx - k * nz;
-                                uint4 *dst = reinterpret_cast<uint4 *>(ring_b + (s0 + k) * kChunkBytes +
-                                                                       (v + r / 8) * 128) + r % 8;
+                                uint4 *dst = reinterpret_cast<uint4 *>(entry + k * kChunkBytes + (v + r / 8) * 128) + r % 8;
                                 *dst = make_uint4(0, 0, 0, 0);
                             }
                             tc::fence_proxy_async_smem();
                             __syncwarp();
                         }
-                        const uint32_t cb = ring_base + s0 * kChunkBytes;
-                        const uint32_t pb = p_base + (t % kPBufs<N>) * (N / 16) * (kTile * 32);
+                        const uint32_t cb = ring_base + rp.slot * 2 * kChunkBytes;
                         const uint32_t d_o = tmem + o_cur + m * N;
-                        for (int kk = 0; kk < v16 / 16; ++kk)
-                            tc::mma_bf16_elect(d_o, with_addr(dc, cb + kk * 16 * 128),
-                                               with_addr(dp, pb + kk * 16 * 32), id_pv,
-                                               (first_pv && kk == 0) ? 0u : 1u);
-                        release(&bars.pv_empty[s0]);
-                        release(&bars.pv_empty[s0 + 1]);
-                        rp.advance(CB);
-                        rp.advance(CB);
+                        const uint32_t empty = smem_u32(&bars.pv_empty[rp.slot]);
+                        if (v16 == kTile) {
+                            tc::mma8_bf16_commit_elect(d_o, with_addr(dc, cb), with_addr(dp, pb), id_pv, first_pv ? 0u : 1u,
+                                                       16 * 128 / 16, 16 * 32 / 16, empty);
+                        } else {
+                            for (int kk = 0; kk < v16 / 16; ++kk)
+                                tc::mma_bf16_elect(d_o, with_addr(dc, cb + kk * 16 * 128),
+                                                   with_addr(dp, pb + kk * 16 * 32), id_pv,
+                                                   (first_pv && kk == 0) ? 0u : 1u);
+                            tc::commit_elect(empty);
+                        }
                     }
                     if (!ok) break;
                     tc::commit_elect(smem_u32(&bars.pv_done[t % kPBufs<N>]));
@@ -1026,17 +1092,13 @@ __global__ void __maxnreg__(128)
         c.group = group;
         c.part = part;
         c.nrc = nrc;
-        c.ncc = ncc;
-        c.cs = CB;
         c.n_items = n_items;
         c.lane_base = static_cast<uint32_t>(c.quarter * 32) << 16;
         c.tmem = tmem;
         c.o_col0 = o_col0;
-        c.ring = ring_b;
         c.p_buf = p_buf;
         c.lim_ns = lim_ns;
         c.t_begin = t_begin;
-        c.t_end = t_end;
         softmax_role<N>(c, a, ss, bars);
     }
 

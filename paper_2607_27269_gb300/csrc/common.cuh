@@ -73,6 +73,18 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint64_
     }
 }
 
+// The same for a whole converged warp: true in every lane, or false in every lane.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, uint64_t limit_ns)
+{
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    const uint64_t t0 = global_ns();
+    for (;;) {
+        for (int i = 0; i < 32; ++i)
+            if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+        if (__any_sync(0xffffffffu, global_ns() - t0 > limit_ns)) return false;
+    }
+}
+
 // ---------------------------------------------------------------- dependent launch
 // The kernels of a decode step are launched as programmatic dependents of
 // the previous launch: a kernel's prologue (barrier set-up, TMEM allocation,

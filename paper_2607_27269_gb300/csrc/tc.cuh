@@ -92,6 +92,50 @@ __device__ __forceinline__ void mma_bf16_elect(uint32_t d_tmem, uint64_t a_desc,
         : "memory");
 }
 
+// Four steps of a product whose operands advance by `da` and `db` (16-byte
+// units) per step, then a commit to `mbar`: one election for all of it.
+__device__ __forceinline__ void mma4_bf16_commit_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                                       uint32_t accumulate, uint32_t da, uint32_t db, uint32_t mbar)
+{
+    const uint64_t a1 = a_desc + da, a2 = a1 + da, a3 = a2 + da, b1 = b_desc + db, b2 = b1 + db, b3 = b2 + db;
+    asm volatile(
+        "{\n .reg .pred p, t, e;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n setp.eq.b32 t, 0, 0;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %5, %6, %3, t;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %7, %8, %3, t;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %9, %10, %3, t;\n"
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%11];\n}\n" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "l"(a1), "l"(b1), "l"(a2), "l"(b2), "l"(a3), "l"(b3),
+        "r"(mbar)
+        : "memory");
+}
+
+// Eight steps, likewise.
+__device__ __forceinline__ void mma8_bf16_commit_elect(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
+                                                       uint32_t accumulate, uint32_t da, uint32_t db, uint32_t mbar)
+{
+    const uint64_t a1 = a_desc + da, a2 = a1 + da, a3 = a2 + da, b1 = b_desc + db, b2 = b1 + db, b3 = b2 + db;
+    asm volatile(
+        "{\n .reg .pred p, t, e;\n .reg .b64 x, y;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 p, %4, 0;\n"
+        " setp.eq.b32 t, 0, 0;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %5, %6, %3, t;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %7, %8, %3, t;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], %9, %10, %3, t;\n"
+        " add.s64 x, %1, %12;\n add.s64 y, %2, %13;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, t;\n"
+        " add.s64 x, %5, %12;\n add.s64 y, %6, %13;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, t;\n"
+        " add.s64 x, %7, %12;\n add.s64 y, %8, %13;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, t;\n"
+        " add.s64 x, %9, %12;\n add.s64 y, %10, %13;\n"
+        " @e tcgen05.mma.cta_group::1.kind::f16 [%0], x, y, %3, t;\n"
+        " @e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%11];\n}\n" ::"r"(d_tmem),
+        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate), "l"(a1), "l"(b1), "l"(a2), "l"(b2), "l"(a3), "l"(b3),
+        "r"(mbar), "l"(static_cast<uint64_t>(4 * da)), "l"(static_cast<uint64_t>(4 * db))
+        : "memory");
+}
+
 __device__ __forceinline__ void commit_elect(uint32_t mbar)
 {
     asm volatile(
@@ -221,6 +265,38 @@ __device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap
     asm volatile(
         "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, "
         "%3, %4}], [%5], %6;" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(mbar), "l"(policy)
+        : "memory");
+}
+
+// Warp-collective forms (the whole warp converged, one elected lane issues).
+__device__ __forceinline__ void mbar_arrive_expect_tx_elect(uint32_t mbar, uint32_t bytes)
+{
+    asm volatile(
+        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+        " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}\n" ::"r"(mbar),
+        "r"(bytes)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_load_2d_hint_elect(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1,
+                                                       uint32_t mbar, uint64_t policy)
+{
+    asm volatile(
+        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+        " @e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, "
+        "{%2, %3}], [%4], %5;\n}\n" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(mbar), "l"(policy)
+        : "memory");
+}
+
+__device__ __forceinline__ void tma_load_3d_hint_elect(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1,
+                                                       int32_t c2, uint32_t mbar, uint64_t policy)
+{
+    asm volatile(
+        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n"
+        " @e cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, "
+        "{%2, %3, %4}], [%5], %6;\n}\n" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(mbar), "l"(policy)
         : "memory");
 }
