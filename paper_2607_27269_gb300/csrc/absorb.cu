@@ -41,6 +41,7 @@ struct AbArgs {
     const int32_t *kv_len;
     uint16_t *q_abs;
     unsigned *status;
+    int early_weights;
 };
 
 struct __align__(8) AbBars {
@@ -48,16 +49,6 @@ struct __align__(8) AbBars {
     uint64_t tfull[2], tempty[2];
     uint64_t drain;
 };
-
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1, int32_t c2,
-                                            int32_t c3, uint32_t mbar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
-        "[%6];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(mbar)
-        : "memory");
-}
 
 __device__ __forceinline__ void unpack8(const uint4 v, float *x)
 {
@@ -151,8 +142,11 @@ __global__ void __launch_bounds__(kAbThreads) absorb_kernel(const __grid_constan
     tc::fence_after_sync();
     // the queries come from the previous launch; this kernel writes no cache,
     // so its dependents (the attention core) may launch at once
-    griddep_wait();
-    griddep_launch_dependents();
+    const bool early = a.early_weights && warp == 0;  // the first weight tiles go out before the wait
+    if (!early) {
+        griddep_wait();
+        griddep_launch_dependents();
+    }
     const uint32_t tmem = tmem_base;
     const int nmine = a.items > static_cast<int>(blockIdx.x)
                           ? (a.items - 1 - static_cast<int>(blockIdx.x)) / static_cast<int>(gridDim.x) + 1
@@ -166,32 +160,54 @@ __global__ void __launch_bounds__(kAbThreads) absorb_kernel(const __grid_constan
     };
 
     if (warp == 0) {
-        // ---- K chunks of A (query rows) and B (W_UK columns) by TMA, item after item
-        if (lane == 0) {
-            tc::prefetch_tensormap(&map_a);
-            tc::prefetch_tensormap(&map_b);
-            tc::prefetch_tensormap(&map_c);
-        }
+        // ---- K chunks of A (query rows) and B (W_UK columns) by TMA, item
+        // after item (converged warp, one elected lane issues)
+        tc::prefetch_tensormap(&map_a);
+        tc::prefetch_tensormap(&map_b);
+        tc::prefetch_tensormap(&map_c);
+        const int jobs = nmine * nkc, head = jobs < kAbStages ? jobs : kAbStages;
         int issued = 0;
-        for (int job = 0; job < nmine * nkc; ++job) {
-            const int j = job / nkc, kc = job - j * nkc, s = job % kAbStages, round = job / kAbStages;
-            if (round >= 1 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.empty[s]), (round - 1) & 1, lim))) {
+        int g = 0, mt = 0, nh = 0, j = 0, kc = 0;  // the next job's item and K chunk
+        auto load_b = [&](int s) {
+            const uint32_t fb = smem_u32(&bars.full[s]);
+            tc::mbar_arrive_expect_tx_elect(fb, static_cast<uint32_t>(a.RT) * 128 + b_bytes);
+            tc::tma_load_3d_elect(smem_u32(sb + s * (kAbMaxN * 128)), &map_b, 0, g * a.K + 64 * kc, nh * (a.ni / 64), fb);
+        };
+        auto load_a = [&](int s) {
+            tc::tma_load_4d_elect(smem_u32(sa + s * kABytes), &map_a, 64 * kc, 0, g, mt * a.R, smem_u32(&bars.full[s]));
+        };
+        auto seek = [&](int job) {
+            j = job / nkc;
+            kc = job - j * nkc;
+            item_of(j, &g, &mt, &nh);
+        };
+        auto step = [&]() {
+            if (++kc == nkc) {
+                kc = 0;
+                item_of(++j, &g, &mt, &nh);
+            }
+        };
+        seek(0);
+        for (int s = 0; s < head; ++s, step()) load_b(s);
+        if (early) {
+            griddep_wait();
+            griddep_launch_dependents();
+        }
+        seek(0);
+        for (int s = 0; s < head; ++s, step()) load_a(s);
+        issued = head;
+        for (int s = 0, par = 0; issued < jobs; step()) {
+            if (!mbar_wait_warp(smem_u32(&bars.empty[s]), par, lim)) {
                 if (lane == 0) record_status(a.status, kStatusTimeout);
                 break;
             }
-            issued = job + 1;
-            // lane 0 loads the A box, lane 1 the B box (one tensor-TMA
-            // instruction occupies its thread for a long time, whatever its size)
-            int g, mt, nh;
-            item_of(j, &g, &mt, &nh);
-            const uint32_t fb = smem_u32(&bars.full[s]);
-            if (lane == 0) tc::mbar_arrive_expect_tx(fb, static_cast<uint32_t>(a.RT) * 128 + b_bytes);
-            __syncwarp();
-            if (lane == 0) tma_load_4d(smem_u32(sa + s * kABytes), &map_a, 64 * kc, 0, g, mt * a.R, fb);
-            if (lane == 1)
-                tc::tma_load_3d(smem_u32(sb + s * (kAbMaxN * 128)), &map_b, 0, g * a.K + 64 * kc, nh * (a.ni / 64),
-                                fb);
-            __syncwarp();
+            ++issued;
+            load_b(s);
+            load_a(s);
+            if (++s == kAbStages) {
+                s = 0;
+                par ^= 1;
+            }
         }
         // no copy may still be landing when the CTA exits: wait (bounded) for
         // the last load of every stage; after a normal run all have landed
@@ -209,21 +225,19 @@ __global__ void __launch_bounds__(kAbThreads) absorb_kernel(const __grid_constan
         bool ok = true;
         for (int j = 0; j < nmine && ok; ++j) {
             const int buf = j & 1;
-            if (j >= 2) ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.tempty[buf]), ((j >> 1) - 1) & 1, lim));
+            if (j >= 2) ok = mbar_wait_warp(smem_u32(&bars.tempty[buf]), ((j >> 1) - 1) & 1, lim);
             if (!ok) break;
             tc::fence_after_sync();
             const uint32_t d = tmem + static_cast<uint32_t>(buf * a.ni);
             for (int kc = 0; kc < nkc && ok; ++kc) {
                 const int job = j * nkc + kc, s = job % kAbStages;
-                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.full[s]), (job / kAbStages) & 1, lim));
+                ok = mbar_wait_warp(smem_u32(&bars.full[s]), (job / kAbStages) & 1, lim);
                 if (!ok) break;
                 tc::fence_after_sync();
                 const uint32_t ab = smem_u32(sa + s * kABytes), bb = smem_u32(sb + s * (kAbMaxN * 128));
-#pragma unroll
-                for (int kk = 0; kk < 4; ++kk)
-                    tc::mma_bf16_elect(d, with_addr(da, ab + kk * 32), with_addr(db, bb + kk * 16 * 128), idesc,
-                                       (kc | kk) != 0);
-                tc::commit_elect(smem_u32(&bars.empty[s]));
+                // four steps of 16 along K: 32 bytes of A, 16 rows of the N-major B
+                tc::mma4_bf16_commit_elect(d, with_addr(da, ab), with_addr(db, bb), idesc, kc != 0, 2, 16 * 128 / 16,
+                                           smem_u32(&bars.empty[s]));
             }
             if (ok) tc::commit_elect(smem_u32(&bars.tfull[buf]));
         }
@@ -369,7 +383,7 @@ cudaError_t get_encoder_ab()
 // The persistent kernel, or cudaErrorNotSupported for a shape it does not serve.
 cudaError_t launch_absorb_persistent(const mla_dims &d, int batch, int q_len, const void *q_nope, const void *q_pe,
                                      const int32_t *kv_len, const void *w_uk, void *q_abs, unsigned *status,
-                                     cudaStream_t st)
+                                     cudaStream_t st, bool early_weights)
 {
     const int H = d.num_heads, G = d.num_kv_groups, hpg = H / G;
     if (d.d_nope % 64 || d.d_nope > 256 || d.rank % 64 || hpg > 128 || d.d_rope > 128 || d.d_rope % 16)
@@ -417,6 +431,7 @@ cudaError_t launch_absorb_persistent(const mla_dims &d, int batch, int q_len, co
     a.kv_len = kv_len;
     a.q_abs = static_cast<uint16_t *>(q_abs);
     a.status = status;
+    a.early_weights = early_weights;
     cudaError_t e = get_encoder_ab();
     if (e != cudaSuccess) return e;
     CUtensorMap ma, mb, mc;
@@ -475,9 +490,10 @@ cudaError_t launch_absorb_persistent(const mla_dims &d, int batch, int q_len, co
 
 cudaError_t launch_absorb(const mla_dims &d, int batch, int q_len, const void *q_nope, const void *q_pe,
                           const int32_t *kv_len, const void *w_uk, void *q_abs, unsigned *status,
-                          cudaStream_t st)
+                          cudaStream_t st, bool early_weights)
 {
-    const cudaError_t pe = launch_absorb_persistent(d, batch, q_len, q_nope, q_pe, kv_len, w_uk, q_abs, status, st);
+    const cudaError_t pe = launch_absorb_persistent(d, batch, q_len, q_nope, q_pe, kv_len, w_uk, q_abs, status, st,
+                                                    early_weights);
     if (pe != cudaErrorNotSupported) return pe;  // else the grouped GEMM serves the shape
     const int H = d.num_heads, G = d.num_kv_groups, hpg = H / G;
     // rows of group g: (b, i, head g*hpg + hh); q_lat = q_nope W_UK[g] (W_UK: d_nope x rank)
@@ -496,6 +512,7 @@ cudaError_t launch_absorb(const mla_dims &d, int batch, int q_len, const void *q
     p.C = q_abs;
     p.ldc = d.rank + d.d_rope;
     p.status = status;
+    p.early_weights = early_weights;
     // one launch: the GEMM's first column tile also rotates the positional query
     return launch_absorb_gemm(p, d, q_pe, kv_len, q_len, st);
 }

@@ -243,7 +243,8 @@ mla_status mla_cache_append_impl(const mla_dims *dims, const mla_cache *cache, i
 }
 
 mla_status mla_absorb_q_impl(const mla_dims *dims, int32_t batch, int32_t q_len, const void *q_nope,
-                             const void *q_pe, const int32_t *kv_len, const void *w_uk, void *q_abs, void *stream, bool launch)
+                             const void *q_pe, const int32_t *kv_len, const void *w_uk, void *q_abs, void *stream, bool launch,
+                             bool early_weights = false)
 {
     mla_status s = check_dims(dims);
     if (s != MLA_OK) return s;
@@ -256,7 +257,7 @@ mla_status mla_absorb_q_impl(const mla_dims *dims, int32_t batch, int32_t q_len,
     unsigned *status = nullptr;
     if ((s = device_info(&status, nullptr)) != MLA_OK) return s;
     return from_cuda(launch_absorb(*dims, batch, q_len, q_nope, q_pe, kv_len, w_uk, q_abs, status,
-                                   static_cast<cudaStream_t>(stream)));
+                                   static_cast<cudaStream_t>(stream), early_weights));
 }
 
 mla_status mla_decode_attn_impl(const mla_dims *dims, const mla_cache *cache, int32_t batch, int32_t q_len,
@@ -318,7 +319,8 @@ mla_status mla_combine_impl(const mla_dims *dims, int32_t batch, int32_t q_len, 
 }
 
 mla_status mla_out_proj_impl(const mla_dims *dims, int32_t batch, int32_t q_len, const float *o_lat,
-                             const void *w_uv, const void *w_o, void *o, void *out, void *stream, bool launch)
+                             const void *w_uv, const void *w_o, void *o, void *out, void *stream, bool launch,
+                             bool early_weights = false)
 {
     mla_status s = check_dims(dims);
     if (s != MLA_OK) return s;
@@ -332,7 +334,7 @@ mla_status mla_out_proj_impl(const mla_dims *dims, int32_t batch, int32_t q_len,
     unsigned *status = nullptr;
     if ((s = device_info(&status, nullptr)) != MLA_OK) return s;
     return from_cuda(launch_out_proj(*dims, batch, q_len, o_lat, w_uv, w_o, o, out, status,
-                                     static_cast<cudaStream_t>(stream)));
+                                     static_cast<cudaStream_t>(stream), early_weights));
 }
 
 }  // namespace
@@ -651,14 +653,16 @@ mla_status mla_decode_step(const mla_dims *dims, const mla_cache *cache, int32_t
         const bool go = pass == 1;
         mla_status s = MLA_OK;
         if (c_new) s = mla_cache_append_impl(dims, cache, batch, q_len, c_new, kr_new, start_pos, stream, go);
-        if (s == MLA_OK) s = mla_absorb_q_impl(dims, batch, q_len, q_nope, q_pe, kv_len, w_uk, q_abs, stream, go);
+        // (behind another launch of this call the weights are known to be final)
+        if (s == MLA_OK)
+            s = mla_absorb_q_impl(dims, batch, q_len, q_nope, q_pe, kv_len, w_uk, q_abs, stream, go, c_new != nullptr);
         if (s == MLA_OK)
             s = mla_decode_attn_impl(dims, cache, batch, q_len, kv_len, max_kv_len, q_abs, num_splits, o_part,
                                      lse_part, stream, go, direct ? o_lat : nullptr, direct ? lse : nullptr);
         if (s == MLA_OK)
             s = mla_combine_impl(dims, batch, q_len, num_splits, kv_len, max_kv_len, o_part, lse_part, o_lat, lse,
                                  stream, go, direct);
-        if (s == MLA_OK) s = mla_out_proj_impl(dims, batch, q_len, o_lat, w_uv, w_o, o, out, stream, go);
+        if (s == MLA_OK) s = mla_out_proj_impl(dims, batch, q_len, o_lat, w_uv, w_o, o, out, stream, go, true);
         if (s != MLA_OK) return s;
     }
     return MLA_OK;

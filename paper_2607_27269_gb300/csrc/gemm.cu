@@ -158,7 +158,7 @@ __device__ void proj_epilogue(const GroupGemm &p, const ProjEpi &e, uint32_t t_l
             uint32_t v[16];
             tc::ld_32x32b_x16(t_lane + j, v);
             tc::wait_ld();
-            if (ok) store16_bf16(crow + ty * BN + j, v);
+            if (ok && ty * BN + j < e.rank) store16_bf16(crow + ty * BN + j, v);  // (the last tile may reach past the latent)
         }
         return;
     }
@@ -198,16 +198,6 @@ struct __align__(8) GemmBars {
     uint64_t full[kStages], raw_full[kStages], conv_done[kStages], empty[kStages], done;
 };
 
-__device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1, int32_t c2,
-                                            int32_t c3, uint32_t mbar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
-        "[%6];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(mbar)
-        : "memory");
-}
-
 // BN: columns per CTA.  NMAJ: the weight is N-major.  AF32: A is fp32.
 // PROJ: the projection (K-major weights map_b, map_b2, map_b3 by column region).
 template <int BN, bool NMAJ, bool AF32, bool PROJ>
@@ -221,6 +211,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
     static_assert(!PROJ || (!NMAJ && !AF32), "the projection reads bf16 h and K-major weights");
     constexpr int kABytes = 128 * 128;     // 128 rows x 64 K, bf16, SW128 K-major
     constexpr int kRawBytes = AF32 ? 2 * 128 * 128 : 0;  // two 32-column fp32 boxes
+    constexpr uint32_t kTmem = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;  // accumulator columns
     constexpr int kBBytes = BN * 128;      // BN x 64 K (K-major) or 64 K x BN (N-major)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     __shared__ GemmBars bars;
@@ -265,16 +256,19 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
         tc::fence_barrier_init();
     }
     if (warp == 1) {
-        tc::tmem_alloc(smem_u32(&tmem_base), BN < 32 ? 32 : BN);
+        tc::tmem_alloc(smem_u32(&tmem_base), kTmem);
         tc::tmem_relinquish();
     }
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    griddep_wait();  // the activations come from the previous launch
+    // the activations come from the previous launch; with early_weights the
+    // producer sends for the first weight tiles before it waits
+    const bool early = !PROJ && p.early_weights && warp == 0;
+    if (!early) griddep_wait();
     // the projection writes the cache: its dependents launch only once it has
     // completed (the attention kernel loads cache tiles before its own wait)
-    if (!PROJ) griddep_launch_dependents();
+    if (!PROJ && !early) griddep_launch_dependents();
     const uint32_t tmem = tmem_base;
     auto bail = [&]() {
         record_status(p.status, kStatusTimeout);
@@ -283,7 +277,10 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
     bool ep_ok = false;  // split K: this epilogue thread saw its CTA's MMAs complete
 
     if (warp == 0) {
-        // ---- A and weight tiles by TMA
+        // ---- A and weight tiles by TMA (converged warp, one elected lane
+        // issues: with a lone lane and a division per chunk this loop took
+        // 0.45 us a chunk and was the kernel's pace -- W_O of 640 rows 15 us
+        // for 32 chunks, the projection of 640 rows 18.5)
         const CUtensorMap *mb = &map_b;
         int brow = g * p.N + n0;
         uint32_t bbytes = kBBytes;
@@ -293,38 +290,48 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
             brow = region == 0 ? n0 : region == 1 ? 0 : (ty - pe.tiles_lat - 1) * BN;
             bbytes = pe.box_bytes[region];
         }
-        if (lane == 0) {
-            tc::prefetch_tensormap(&map_a);
-            tc::prefetch_tensormap(mb);
+        tc::prefetch_tensormap(mb);
+        tc::prefetch_tensormap(&map_a);
+        auto load_b = [&](int c, int s) {
+            const uint32_t fb = smem_u32(&bars.full[s]), dst = smem_u32(sb + s * kBBytes);
+            tc::mbar_arrive_expect_tx_elect(fb, bbytes + (AF32 ? 0u : a_bytes));
+            if (NMAJ) {
+                // rows = K of group g, columns = N: one 64 x 64 box per 64 columns
+#pragma unroll
+                for (int j = 0; j < BN / 64; ++j)
+                    tc::tma_load_2d_elect(dst + j * 64 * 128, &map_b, n0 + 64 * j, g * p.K + 64 * c, fb);
+            } else {
+                tc::tma_load_2d_elect(dst, mb, 64 * c, brow, fb);
+            }
+        };
+        auto load_a = [&](int c, int s) {
+            if (AF32) {
+                const uint32_t rb = smem_u32(&bars.raw_full[s]), rdst = smem_u32(sr + s * kRawBytes);
+                tc::mbar_arrive_expect_tx_elect(rb, 2 * a_bytes);
+                tc::tma_load_4d_elect(rdst, &map_a, 64 * c, 0, g, mt * R, rb);
+                tc::tma_load_4d_elect(rdst + 128 * 128, &map_a, 64 * c + 32, 0, g, mt * R, rb);
+            } else {
+                tc::tma_load_4d_elect(smem_u32(sa + s * AS), &map_a, 64 * c, 0, g, mt * R, smem_u32(&bars.full[s]));
+            }
+        };
+        const int head = nkl < NS ? nkl : NS;  // the ring's first round
+        for (int s = 0; s < head; ++s) load_b(c_begin + s, s);
+        if (early) {
+            griddep_wait();
+            griddep_launch_dependents();
         }
-        for (int cc = 0; cc < nkl; ++cc) {
-            const int c = c_begin + cc, s = cc % NS, round = cc / NS;
-            if (round >= 1 && !__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.empty[s]), (round - 1) & 1, lim))) {
+        for (int s = 0; s < head; ++s) load_a(c_begin + s, s);
+        for (int c = c_begin + head, s = 0, par = 0; c < c_begin + nkl; ++c) {
+            if (!mbar_wait_warp(smem_u32(&bars.empty[s]), par, lim)) {
                 if (lane == 0) bail();
                 break;
             }
-            if (lane == 0) {
-                const uint32_t fb = smem_u32(&bars.full[s]);
-                tc::mbar_arrive_expect_tx(fb, bbytes + (AF32 ? 0u : a_bytes));
-                const uint32_t dst = smem_u32(sb + s * kBBytes);
-                if (NMAJ) {
-                    // rows = K of group g, columns = N: one 64 x 64 box per 64 columns
-                    for (int j = 0; j < BN / 64; ++j)
-                        tc::tma_load_2d(dst + j * 64 * 128, &map_b, n0 + 64 * j, g * p.K + 64 * c, fb);
-                } else {
-                    tc::tma_load_2d(dst, mb, 64 * c, brow, fb);
-                }
-                if (AF32) {
-                    const uint32_t rb = smem_u32(&bars.raw_full[s]);
-                    tc::mbar_arrive_expect_tx(rb, 2 * a_bytes);
-                    const uint32_t rdst = smem_u32(sr + s * kRawBytes);
-                    tma_load_4d(rdst, &map_a, 64 * c, 0, g, mt * R, rb);
-                    tma_load_4d(rdst + 128 * 128, &map_a, 64 * c + 32, 0, g, mt * R, rb);
-                } else {
-                    tma_load_4d(smem_u32(sa + s * AS), &map_a, 64 * c, 0, g, mt * R, fb);
-                }
+            load_b(c, s);
+            load_a(c, s);
+            if (++s == NS) {
+                s = 0;
+                par ^= 1;
             }
-            __syncwarp();
         }
     } else if (warp == 1) {
         // ---- MMA issuer (converged warp, one elected lane issues)
@@ -336,20 +343,19 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
             return tmpl | static_cast<uint64_t>((saddr & 0x3FFFFu) >> 4);
         };
         bool ok = true;
-        for (int cc = 0; cc < nkl && ok; ++cc) {
-            const int s = cc % NS, par = (cc / NS) & 1;
-            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.full[s]), par, lim) &&
-                                             (!AF32 || mbar_wait(smem_u32(&bars.conv_done[s]), par, lim)));
+        for (int cc = 0, s = 0, par = 0; cc < nkl; ++cc) {
+            ok = mbar_wait_warp(smem_u32(&bars.full[s]), par, lim) &&
+                 (!AF32 || mbar_wait_warp(smem_u32(&bars.conv_done[s]), par, lim));
             if (!ok) break;
             tc::fence_after_sync();
-            const uint32_t a_base = smem_u32(AF32 ? sr + s * kRawBytes : sa + s * AS), b_base = smem_u32(sb + s * kBBytes);
-#pragma unroll
-            for (int kk = 0; kk < 4; ++kk) {
-                const uint32_t b_addr = NMAJ ? b_base + kk * 16 * 128 : b_base + kk * 32;
-                tc::mma_bf16_elect(tmem, with_addr(da, a_base + kk * 32), with_addr(db, b_addr), idesc,
-                                   (cc | kk) != 0);
+            // four steps of 16 along K: 32 bytes of a K-major operand, 16 rows of an N-major one
+            tc::mma4_bf16_commit_elect(tmem, with_addr(da, smem_u32(AF32 ? sr + s * kRawBytes : sa + s * AS)),
+                                       with_addr(db, smem_u32(sb + s * kBBytes)), idesc, cc != 0, 2, NMAJ ? 16 * 128 / 16 : 2,
+                                       smem_u32(&bars.empty[s]));
+            if (++s == NS) {
+                s = 0;
+                par ^= 1;
             }
-            tc::commit_elect(smem_u32(&bars.empty[s]));
         }
         if (!ok && lane == 0) bail();
         tc::commit_elect(smem_u32(&bars.done));
@@ -357,9 +363,8 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
         if (AF32) {
             // ---- fp32 -> bf16: thread r converts tile row r (two 128-byte swizzled fp32 rows)
             const int r = tid - 64;
-            for (int cc = 0; cc < nkl; ++cc) {
-                const int s = cc % NS, par = (cc / NS) & 1;
-                if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.raw_full[s]), par, lim))) {
+            for (int cc = 0, s = 0, par = 0; cc < nkl; ++cc) {
+                if (!mbar_wait_warp(smem_u32(&bars.raw_full[s]), par, lim)) {
                     if (lane == 0) bail();
                     break;
                 }
@@ -382,6 +387,10 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
                 tc::fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) tc::mbar_arrive(smem_u32(&bars.conv_done[s]));
+                if (++s == NS) {
+                    s = 0;
+                    par ^= 1;
+                }
             }
         }
         if (!PROJ && pe.rope_src) {
@@ -425,7 +434,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
             }
         }
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31
-        const bool ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.done), 0, lim));
+        const bool ok = mbar_wait_warp(smem_u32(&bars.done), 0, lim);
         if (!ok) {
             if (lane == 0) bail();
         } else if (!fail) {
@@ -520,7 +529,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
     __syncthreads();
     if (warp == 1) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, BN < 32 ? 32 : BN);
+        tc::tmem_dealloc(tmem, kTmem);
     }
 }
 
@@ -696,7 +705,7 @@ cudaError_t launch_proj(const mla_dims &d, const CacheView &c, int batch, int n_
     p.lda = d.hidden;
     p.status = status;
     const int nq = w_q ? d.num_heads * (d.d_nope + d.d_rope) : 0;
-    const int rope_rows = d.d_rope < BN ? d.d_rope : BN, q_rows = nq < BN ? nq : BN;
+    const int lat_rows = d.rank < BN ? d.rank : BN, rope_rows = d.d_rope < BN ? d.d_rope : BN, q_rows = nq < BN ? nq : BN;
     ProjEpi pe{};
     pe.cache = c;
     pe.start_pos = start_pos;
@@ -709,13 +718,13 @@ cudaError_t launch_proj(const mla_dims &d, const CacheView &c, int batch, int n_
     pe.heads = d.num_heads;
     pe.style = d.rope_style;
     pe.turns = rope_turns(d.d_rope, d.rope_base);
-    pe.tiles_lat = d.rank / BN;
-    pe.box_bytes[0] = BN * 128;
+    pe.tiles_lat = (d.rank + BN - 1) / BN;
+    pe.box_bytes[0] = static_cast<uint32_t>(lat_rows) * 128;
     pe.box_bytes[1] = static_cast<uint32_t>(rope_rows) * 128;
     pe.box_bytes[2] = static_cast<uint32_t>(q_rows) * 128;
     const int rblk = rows_per_tile(p);
     CUtensorMap ma, m0, m1, m2;
-    if (!encode_a(p, rblk, false, &ma) || !encode_kmajor(w_dkv, d.rank, d.hidden, BN, &m0) ||
+    if (!encode_a(p, rblk, false, &ma) || !encode_kmajor(w_dkv, d.rank, d.hidden, lat_rows, &m0) ||
         !encode_kmajor(w_kr, d.d_rope, d.hidden, rope_rows, &m1))
         return cudaErrorInvalidValue;
     if (w_q) {
@@ -777,25 +786,34 @@ cudaError_t launch_project(const mla_dims &d, const CacheView &c, int batch, int
                            void *q_nope, void *q_pe, unsigned *status, cudaStream_t st)
 {
     if (batch <= 0 || n_new <= 0) return cudaSuccess;
-    // 128-column tiles once there are enough rows to be tensor-bound and the
-    // latent splits into whole 128-column tiles; 64 otherwise.  256-column
-    // tiles when they take fewer waves of CTAs by more than their extra bytes
-    // per K chunk (A 16 KB + B 32 KB against 16 + 16): the row tiles times the
-    // column tiles just past one wave at 128 (640 rows: 185 CTAs -> 95).
-    const int rows = batch * n_new;
-    if (rows > 32 && d.rank % 128 == 0) {
-        if (d.rank % 256 == 0) {
-            int dev = 0, sms = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            const int nq = w_q ? d.num_heads * (d.d_nope + d.d_rope) : 0;
-            const int64_t mt = (rows + 127) / 128;
-            auto waves = [&](int bn) { return (mt * (d.rank / bn + 1 + (nq + bn - 1) / bn) + sms - 1) / sms; };
-            if (sms > 0 && waves(256) * 48 < waves(128) * 32)
-                return launch_proj<256>(d, c, batch, n_new, h, w_dkv, w_kr, w_q, start_pos, q_nope, q_pe, status, st);
+    // The kernel is bound by filling shared memory (both tiles per K chunk from
+    // L2, about 130 GB/s per SM), one CTA per SM: so the column tile with the
+    // least waves of CTAs times the bytes a chunk loads, 16 KB of h and 128
+    // bytes per column; of equal ones the narrowest.  640 rows of the
+    // Llama-3.2-1B shape (4672 columns): 64, 128, 192 and 256 columns take 3 x
+    // 24, 2 x 32, 1 x 40 and 1 x 48 KB; 160 rows 1 x 24 with 64 columns.
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (sms <= 0) sms = 1;
+    const int nq = w_q ? d.num_heads * (d.d_nope + d.d_rope) : 0;
+    const int64_t mt = (static_cast<int64_t>(batch) * n_new + 127) / 128;
+    int bn = 64;
+    int64_t best = 0;
+    for (int w : {64, 128, 192, 256}) {
+        const int64_t ctas = mt * ((d.rank + w - 1) / w + 1 + (nq + w - 1) / w);
+        const int64_t cost = (ctas + sms - 1) / sms * (128 + w);
+        if (best == 0 || cost < best) {
+            best = cost;
+            bn = w;
         }
-        return launch_proj<128>(d, c, batch, n_new, h, w_dkv, w_kr, w_q, start_pos, q_nope, q_pe, status, st);
     }
+    if (bn == 256)
+        return launch_proj<256>(d, c, batch, n_new, h, w_dkv, w_kr, w_q, start_pos, q_nope, q_pe, status, st);
+    if (bn == 192)
+        return launch_proj<192>(d, c, batch, n_new, h, w_dkv, w_kr, w_q, start_pos, q_nope, q_pe, status, st);
+    if (bn == 128)
+        return launch_proj<128>(d, c, batch, n_new, h, w_dkv, w_kr, w_q, start_pos, q_nope, q_pe, status, st);
     return launch_proj<64>(d, c, batch, n_new, h, w_dkv, w_kr, w_q, start_pos, q_nope, q_pe, status, st);
 }
 

@@ -45,7 +45,7 @@ cudaError_t launch_append(const mla_dims &d, const CacheView &c, int batch, int 
 
 cudaError_t launch_absorb(const mla_dims &d, int batch, int q_len, const void *q_nope, const void *q_pe,
                           const int32_t *kv_len, const void *w_uk, void *q_abs, unsigned *status,
-                          cudaStream_t st);
+                          cudaStream_t st, bool early_weights = false);
 
 // CUDA-core attention core; `qgroups` query groups of kSimtRows rows each.
 constexpr int kSimtRows = 16;
@@ -83,7 +83,8 @@ cudaError_t launch_combine(int batch, int q_len, int num_heads, int rank, int ma
                            float *lse, cudaStream_t st, int groups = 1, bool skip_whole = false);
 
 cudaError_t launch_out_proj(const mla_dims &d, int batch, int q_len, const float *o_lat, const void *w_uv,
-                            const void *w_o, void *o, void *out, unsigned *status, cudaStream_t st);
+                            const void *w_o, void *o, void *out, unsigned *status, cudaStream_t st,
+                            bool early_weights = false);
 
 // Grouped GEMM of the projections: for each group g < G and row m < M,
 // C[phys(g, m), n] = sum_k A[phys(g, m), k] B_g(n, k) (bf16 result), with
@@ -102,6 +103,11 @@ struct GroupGemm {
     void *C;
     int64_t ldc;
     unsigned *status;
+    // The stream's previous launch is this library's and began (passed its own
+    // dependency wait) after everything before it had completed, so the
+    // weights are final and may be read before this kernel's wait.  Not so
+    // behind a caller's kernel that lets its dependents launch early.
+    int early_weights = 0;
     int stages, rblk, ksplit;  // set by the launcher
     int a_stride;              // bytes between A ring stages (set by the launcher)
 };

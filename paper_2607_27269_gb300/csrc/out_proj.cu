@@ -7,7 +7,8 @@
 namespace gbmla {
 
 cudaError_t launch_out_proj(const mla_dims &d, int batch, int q_len, const float *o_lat, const void *w_uv,
-                            const void *w_o, void *o, void *out, unsigned *status, cudaStream_t st)
+                            const void *w_o, void *o, void *out, unsigned *status, cudaStream_t st,
+                            bool early_weights)
 {
     const int H = d.num_heads, G = d.num_kv_groups, hpg = H / G;
     GroupGemm p;
@@ -25,6 +26,7 @@ cudaError_t launch_out_proj(const mla_dims &d, int batch, int q_len, const float
     p.C = o;
     p.ldc = d.d_v;
     p.status = status;
+    p.early_weights = early_weights;
     cudaError_t e = launch_group_gemm(p, st);
     if (e != cudaSuccess || w_o == nullptr || d.hidden == 0) return e;
     GroupGemm q;
@@ -42,6 +44,7 @@ cudaError_t launch_out_proj(const mla_dims &d, int batch, int q_len, const float
     q.C = out;
     q.ldc = d.hidden;
     q.status = status;
+    q.early_weights = 1;  // behind the W_UV product above
     return launch_group_gemm(q, st);
 }
 
