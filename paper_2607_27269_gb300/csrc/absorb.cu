@@ -41,7 +41,7 @@ struct AbArgs {
     const int32_t *kv_len;
     uint16_t *q_abs;
     unsigned *status;
-    int early_weights;
+    int beside;     // the previous launch is the same step's append
 };
 
 struct __align__(8) AbBars {
@@ -140,10 +140,13 @@ __global__ void __launch_bounds__(kAbThreads) absorb_kernel(const __grid_constan
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    // the queries come from the previous launch; this kernel writes no cache,
-    // so its dependents (the attention core) may launch at once
-    const bool early = a.early_weights && warp == 0;  // the first weight tiles go out before the wait
-    if (!early) {
+    // The queries come from the previous launch; this kernel writes no cache,
+    // so its dependents (the attention core) may launch at once.  Behind the
+    // append of the same step nothing here comes from the previous launch, and
+    // the append let this one start only after its own wait: one warp alone
+    // waits for it, so that the attention starts with the cache final, while
+    // the others go ahead (the step's first 2 us hidden).
+    if (!a.beside || warp == 4) {
         griddep_wait();
         griddep_launch_dependents();
     }
@@ -188,14 +191,10 @@ __global__ void __launch_bounds__(kAbThreads) absorb_kernel(const __grid_constan
             }
         };
         seek(0);
-        for (int s = 0; s < head; ++s, step()) load_b(s);
-        if (early) {
-            griddep_wait();
-            griddep_launch_dependents();
+        for (; issued < head; ++issued, step()) {
+            load_b(issued);
+            load_a(issued);
         }
-        seek(0);
-        for (int s = 0; s < head; ++s, step()) load_a(s);
-        issued = head;
         for (int s = 0, par = 0; issued < jobs; step()) {
             if (!mbar_wait_warp(smem_u32(&bars.empty[s]), par, lim)) {
                 if (lane == 0) record_status(a.status, kStatusTimeout);
@@ -383,7 +382,7 @@ cudaError_t get_encoder_ab()
 // The persistent kernel, or cudaErrorNotSupported for a shape it does not serve.
 cudaError_t launch_absorb_persistent(const mla_dims &d, int batch, int q_len, const void *q_nope, const void *q_pe,
                                      const int32_t *kv_len, const void *w_uk, void *q_abs, unsigned *status,
-                                     cudaStream_t st, bool early_weights)
+                                     cudaStream_t st, bool beside_append)
 {
     const int H = d.num_heads, G = d.num_kv_groups, hpg = H / G;
     if (d.d_nope % 64 || d.d_nope > 256 || d.rank % 64 || hpg > 128 || d.d_rope > 128 || d.d_rope % 16)
@@ -431,7 +430,7 @@ cudaError_t launch_absorb_persistent(const mla_dims &d, int batch, int q_len, co
     a.kv_len = kv_len;
     a.q_abs = static_cast<uint16_t *>(q_abs);
     a.status = status;
-    a.early_weights = early_weights;
+    a.beside = beside_append;
     cudaError_t e = get_encoder_ab();
     if (e != cudaSuccess) return e;
     CUtensorMap ma, mb, mc;
@@ -490,10 +489,10 @@ cudaError_t launch_absorb_persistent(const mla_dims &d, int batch, int q_len, co
 
 cudaError_t launch_absorb(const mla_dims &d, int batch, int q_len, const void *q_nope, const void *q_pe,
                           const int32_t *kv_len, const void *w_uk, void *q_abs, unsigned *status,
-                          cudaStream_t st, bool early_weights)
+                          cudaStream_t st, bool beside_append)
 {
     const cudaError_t pe = launch_absorb_persistent(d, batch, q_len, q_nope, q_pe, kv_len, w_uk, q_abs, status, st,
-                                                    early_weights);
+                                                    beside_append);
     if (pe != cudaErrorNotSupported) return pe;  // else the grouped GEMM serves the shape
     const int H = d.num_heads, G = d.num_kv_groups, hpg = H / G;
     // rows of group g: (b, i, head g*hpg + hh); q_lat = q_nope W_UK[g] (W_UK: d_nope x rank)
@@ -512,7 +511,7 @@ cudaError_t launch_absorb(const mla_dims &d, int batch, int q_len, const void *q
     p.C = q_abs;
     p.ldc = d.rank + d.d_rope;
     p.status = status;
-    p.early_weights = early_weights;
+    p.early_weights = beside_append;
     // one launch: the GEMM's first column tile also rotates the positional query
     return launch_absorb_gemm(p, d, q_pe, kv_len, q_len, st);
 }

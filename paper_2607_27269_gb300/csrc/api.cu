@@ -226,7 +226,8 @@ using namespace gbmla;
 namespace {
 
 mla_status mla_cache_append_impl(const mla_dims *dims, const mla_cache *cache, int32_t batch, int32_t n_new,
-                                 const void *c_new, const void *kr_new, const int32_t *start_pos, void *stream, bool launch)
+                                 const void *c_new, const void *kr_new, const int32_t *start_pos, void *stream, bool launch,
+                                 bool beside = false)
 {
     mla_status s = check_dims(dims);
     if (s != MLA_OK) return s;
@@ -239,12 +240,12 @@ mla_status mla_cache_append_impl(const mla_dims *dims, const mla_cache *cache, i
     unsigned *status = nullptr;
     if ((s = device_info(&status, nullptr)) != MLA_OK) return s;
     return from_cuda(launch_append(*dims, v, batch, n_new, c_new, kr_new, start_pos, status,
-                                   static_cast<cudaStream_t>(stream)));
+                                   static_cast<cudaStream_t>(stream), 1, beside));
 }
 
 mla_status mla_absorb_q_impl(const mla_dims *dims, int32_t batch, int32_t q_len, const void *q_nope,
                              const void *q_pe, const int32_t *kv_len, const void *w_uk, void *q_abs, void *stream, bool launch,
-                             bool early_weights = false)
+                             bool beside_append = false)
 {
     mla_status s = check_dims(dims);
     if (s != MLA_OK) return s;
@@ -257,7 +258,7 @@ mla_status mla_absorb_q_impl(const mla_dims *dims, int32_t batch, int32_t q_len,
     unsigned *status = nullptr;
     if ((s = device_info(&status, nullptr)) != MLA_OK) return s;
     return from_cuda(launch_absorb(*dims, batch, q_len, q_nope, q_pe, kv_len, w_uk, q_abs, status,
-                                   static_cast<cudaStream_t>(stream), early_weights));
+                                   static_cast<cudaStream_t>(stream), beside_append));
 }
 
 mla_status mla_decode_attn_impl(const mla_dims *dims, const mla_cache *cache, int32_t batch, int32_t q_len,
@@ -652,8 +653,8 @@ mla_status mla_decode_step(const mla_dims *dims, const mla_cache *cache, int32_t
     for (int pass = 0; pass < 2; ++pass) {  // every stage validated, then every stage launched
         const bool go = pass == 1;
         mla_status s = MLA_OK;
-        if (c_new) s = mla_cache_append_impl(dims, cache, batch, q_len, c_new, kr_new, start_pos, stream, go);
-        // (behind another launch of this call the weights are known to be final)
+        // the absorption needs nothing of the append and runs beside it
+        if (c_new) s = mla_cache_append_impl(dims, cache, batch, q_len, c_new, kr_new, start_pos, stream, go, true);
         if (s == MLA_OK)
             s = mla_absorb_q_impl(dims, batch, q_len, q_nope, q_pe, kv_len, w_uk, q_abs, stream, go, c_new != nullptr);
         if (s == MLA_OK)

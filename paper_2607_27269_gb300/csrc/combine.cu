@@ -30,14 +30,16 @@ __global__ void __launch_bounds__(kCombineThreads) combine_kernel(int batch, int
                                                                  float *lse_out, int groups, int skip_whole)
 {
     static_assert(SG == 1 || RPT == 1, "slot groups merge one row per thread");
-    griddep_wait();
-    griddep_launch_dependents();
     __shared__ int64_t red[64];
     __shared__ float xs[SG > 1 ? kCombineThreads * 10 : 1];
     const int b = blockIdx.y;  // unit b: sequence b / groups (groups > 1: one unit per KV group)
     int64_t T, t0;
     block_tile_sums(kv_len, batch, b, q_len, max_kv, red, &T, &t0, groups);
     const int64_t nb = seq_tiles(kv_len[b / groups], q_len, max_kv);
+    // The lengths (read above, as the attention kernel reads them before its
+    // own wait) are no output of the attention; the partials are.
+    griddep_wait();
+    griddep_launch_dependents();
     if (nb == 0 || T == 0) return;  // invalid length: recorded by the attention kernel
     const int k_first = part_of_tile(t0, T, S), k_last = part_of_tile(t0 + nb - 1, T, S);
     if (skip_whole && k_first == k_last) return;  // its one partition wrote the final rows itself

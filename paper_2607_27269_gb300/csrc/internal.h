@@ -35,17 +35,21 @@ struct AttnArgs {
     unsigned *status;
 };
 
-// groups > 1: `batch` counts (sequence, KV group) units, entry rows
+// beside: the next launch is an absorption that runs beside this one
+// (launch_absorb's beside_append).  groups > 1: `batch` counts (sequence, KV
+// group) units, entry rows
 // [sequence, n_new, group, .] (token-major, as a projection writes them),
 // start_pos indexed by sequence (unit / groups); rank = value width, d_rope =
 // key width (the original-GQA cache).
 cudaError_t launch_append(const mla_dims &d, const CacheView &c, int batch, int n_new, const void *c_new,
                           const void *kr_new, const int32_t *start_pos, unsigned *status, cudaStream_t st,
-                          int groups = 1);
+                          int groups = 1, bool beside = false);
 
+// beside_append: the stream's previous launch is the same step's append, with
+// `beside` set; the absorption runs beside it.
 cudaError_t launch_absorb(const mla_dims &d, int batch, int q_len, const void *q_nope, const void *q_pe,
                           const int32_t *kv_len, const void *w_uk, void *q_abs, unsigned *status,
-                          cudaStream_t st, bool early_weights = false);
+                          cudaStream_t st, bool beside_append = false);
 
 // CUDA-core attention core; `qgroups` query groups of kSimtRows rows each.
 constexpr int kSimtRows = 16;
