@@ -290,9 +290,9 @@ __device__ __forceinline__ float ex2(float x)
     return y;
 }
 
-// Reduce 16 columns over the 32 lanes of a warp: afterwards lane l holds, in
-// v[0], the reduction of column (l % 16).
-template <int CNT, bool MAX>
+// Sums of 16 columns over the 32 lanes of a warp: lane l gets, in v[0], the
+// sum of column l % 16.
+template <int CNT>
 __device__ __forceinline__ void halve_step(float *v, int lane)
 {
     const bool upper = (lane & CNT) != 0;
@@ -300,24 +300,32 @@ __device__ __forceinline__ void halve_step(float *v, int lane)
     for (int k = 0; k < CNT; ++k) {
         const float send = upper ? v[k] : v[k + CNT];
         const float keep = upper ? v[k + CNT] : v[k];
-        const float recv = __shfl_xor_sync(0xffffffffu, send, CNT);
-        v[k] = MAX ? fmaxf(keep, recv) : keep + recv;
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, send, CNT);
     }
 }
 
-template <bool MAX>
-__device__ __forceinline__ float reduce16(float (&v)[16], int lane)
+__device__ __forceinline__ float sum16(float (&v)[16], int lane)
 {
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-        const float o = __shfl_xor_sync(0xffffffffu, v[k], 16);
-        v[k] = MAX ? fmaxf(v[k], o) : v[k] + o;
-    }
-    halve_step<8, MAX>(v, lane);
-    halve_step<4, MAX>(v, lane);
-    halve_step<2, MAX>(v, lane);
-    halve_step<1, MAX>(v, lane);
+    for (int k = 0; k < 16; ++k) v[k] += __shfl_xor_sync(0xffffffffu, v[k], 16);
+    halve_step<8>(v, lane);
+    halve_step<4>(v, lane);
+    halve_step<2>(v, lane);
+    halve_step<1>(v, lane);
     return v[0];
+}
+
+// Maxima of 16 columns over the 32 lanes: lane l < 16 gets column l's.
+__device__ __forceinline__ float max16(const float (&v)[16], int lane)
+{
+    float mine = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) {
+        float m;
+        asm volatile("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(m) : "f"(v[k]));
+        mine = lane == k ? m : mine;
+    }
+    return mine;
 }
 
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16])
@@ -399,7 +407,7 @@ __device__ __forceinline__ void sm_block_max(const SmCtx &c, const TcArgs &a, Sh
             const int cb = c.half + 3 * ob;
             float s[16];
             sm_scores<N>(a, ss, s_base, cb, pos, need_mask, s);
-            const float mx = reduce16<true>(s, c.lane);
+            const float mx = max16(s, c.lane);
             if (c.lane < 16) ss.red[c.quarter][cb * 16 + c.lane] = mx;
         }
     }
@@ -422,7 +430,7 @@ __device__ __forceinline__ bool sm_epilogue(const SmCtx &c, const TcArgs &a, Sha
             float v[16];
 #pragma unroll
             for (int e = 0; e < 8; ++e) unpack2(l_part[ob][e], v[2 * e], v[2 * e + 1]);
-            const float ls = reduce16<false>(v, c.lane);
+            const float ls = sum16(v, c.lane);
             if (c.lane < 16) ss.red[c.quarter][cb * 16 + c.lane] = ls;
         }
     }
@@ -477,7 +485,7 @@ __device__ __forceinline__ void sm_close(const SmCtx &c, const TcArgs &a, Shared
             float v[16];
 #pragma unroll
             for (int e = 0; e < 8; ++e) unpack2(l_part[ob][e], v[2 * e], v[2 * e + 1]);
-            const float ls = reduce16<false>(v, c.lane);
+            const float ls = sum16(v, c.lane);
             if (c.lane < 16) ss.red[c.quarter][cb * 16 + c.lane] = ls;
         }
     }
