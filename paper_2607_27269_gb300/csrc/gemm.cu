@@ -262,6 +262,9 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
+    // a peer's shared memory is written only once its CTA has started: arrive
+    // now, wait before the first such write
+    if (!PROJ && ks > 1 && p.recv_off) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     // the activations come from the previous launch; with early_weights the
     // producer sends for the first weight tiles before it waits
     const bool early = !PROJ && p.early_weights && warp == 0;
@@ -469,18 +472,22 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
         }
     }
     if (!PROJ && ks > 1) {
-        // (1) every CTA of the cluster is past its MMAs, so every ring is free;
-        // (2) push this CTA's partial of each column slice to the slice's owner:
-        // CTA o owns columns [o cw, (o + 1) cw) and receives, in its ring,
-        // recv[r][row][cw + 4] from every rank r; (3) each owner sums its slice
-        // in rank order (four columns per step) and stores the bf16 result
+        // (1) push this CTA's partial of each column slice to the slice's owner:
+        // CTA o owns columns [o cw, (o + 1) cw) and receives, behind its ring
+        // (or in it, once every CTA of the cluster is past its MMAs),
+        // recv[r][row][cw + 4] from every rank r; (2) each owner sums its slice
+        // in rank order (four columns per step) and stores the bf16 result.
+        // Nothing is written to a peer after the second barrier.
         const int cw = BN / ks;
-        tc::cluster_sync();
+        if (p.recv_off)
+            asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA has started
+        else
+            tc::cluster_sync();
         if (warp >= 2 && ep_ok && !fail) {
             tc::fence_after_sync();
             const int q = warp & 3, i = q * 32 + lane;
             const uint32_t t_lane = tmem + (static_cast<uint32_t>(q * 32) << 16);
-            const uint32_t recv = smem_u32(smem);
+            const uint32_t recv = smem_u32(smem) + p.recv_off;
 #pragma unroll 1
             for (int j = 0; j < BN; j += 16) {
                 uint32_t v[16];
@@ -503,7 +510,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
         tc::cluster_sync();
         if (warp >= 2 && !fail) {
             const int q4 = cw / 4;
-            const float *recv = reinterpret_cast<const float *>(smem);
+            const float *recv = reinterpret_cast<const float *>(smem + p.recv_off);
             for (int idx = tid - 64; idx < RT * q4; idx += 128) {
                 const int i = idx / q4, c4 = (idx % q4) * 4;
                 const int me = m0 + i, n = n0 + kz * cw + c4;
@@ -517,13 +524,15 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
                 }
                 if (me >= p.M) continue;
                 uint16_t *dst = static_cast<uint16_t *>(p.C) + phys_row(p, g, me) * p.ldc + n;
-                const float a[4] = {acc.x, acc.y, acc.z, acc.w};
-#pragma unroll
-                for (int e = 0; e < 4; ++e)
-                    if (n + e < p.N) dst[e] = __bfloat16_as_ushort(__float2bfloat16_rn(a[e]));
+                const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y), hi = __floats2bfloat162_rn(acc.z, acc.w);
+                const uint32_t w[2] = {*reinterpret_cast<const uint32_t *>(&lo), *reinterpret_cast<const uint32_t *>(&hi)};
+                if (n + 4 <= p.N && p.ldc % 4 == 0) {
+                    *reinterpret_cast<uint2 *>(dst) = make_uint2(w[0], w[1]);
+                } else {
+                    for (int e = 0; e < 4 && n + e < p.N; ++e) dst[e] = static_cast<uint16_t>(w[e / 2] >> (16 * (e % 2)));
+                }
             }
         }
-        tc::cluster_sync();  // keep the cluster together until every CTA is done
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -573,9 +582,15 @@ bool encode_kmajor(const void *w, int64_t rows, int K, int box_rows, CUtensorMap
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Row blocks per tile: as many as fit 128 rows, but no more than there are
-// (a short A box leaves the tile's other rows stale; their results are dropped).
-int rows_per_tile(const GroupGemm &p) { return (128 / p.hpg) < (p.M / p.hpg) ? (128 / p.hpg) : (p.M / p.hpg); }
+// Row blocks per tile: the fewest tiles of at most 128 rows, evenly filled (160
+// rows: 80 + 80, not 128 + 32; a short A box leaves the tile's other rows
+// stale, and their results are dropped).
+int rows_per_tile(const GroupGemm &p)
+{
+    const int blocks = p.M / p.hpg, most = 128 / p.hpg;
+    const int tiles = (blocks + most - 1) / most;
+    return (blocks + tiles - 1) / tiles;
+}
 
 // Ring depth: as many stages as fit 192 KB, at most kStages and the K chunks.
 template <int BN, bool AF32>
@@ -672,9 +687,18 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     }
     q.rblk = rblk;
     q.ksplit = ks;
-    if (ks > 1) {  // the partials received from the cluster reuse the ring
-        const size_t need = 1024 + static_cast<size_t>(ks) * rt * (BN / ks + 4) * 4;
-        if (smem < need) smem = need;
+    q.recv_off = 0;
+    if (ks > 1) {
+        // the partials received from the cluster: behind the ring where two such
+        // CTAs (of short tiles) or one (of full tiles) still fit an SM, so that a
+        // CTA pushes as soon as its own MMAs are done; else in the ring
+        const size_t recv = static_cast<size_t>(ks) * rt * (BN / ks + 4) * 4;
+        if (smem + recv <= (rt <= 64 ? 112u : 224u) * 1024) {
+            q.recv_off = static_cast<int>(smem - 1024);
+            smem += recv;
+        } else if (smem < 1024 + recv) {
+            smem = 1024 + recv;
+        }
     }
     e = cudaFuncSetAttribute(gemm_tc_kernel<BN, NMAJ, AF32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
