@@ -926,8 +926,17 @@ __global__ void __maxnreg__(128)
                     for (; i < nqc; ++i) {
                         ok = mbar_wait_warp(smem_u32(&bars.qk_empty[rp.slot]), (rp.round - 1) & 1, lim_ns);
                         if (!ok) break;
-                        cache_box(i);
-                        if constexpr (SQ) query_box(i, rp.slot, ts.w.b);
+                        if (SQ && ts.at.nh > 0) {
+                            const uint32_t dst = ring + rp.slot * kSlotA;
+                            tc::tma_refill_q_elect(smem_u32(&bars.qk_full[rp.slot]), ts.at.bytes + N * 128,
+                                                   i == 0 ? &map_r : &map_c, i == 0 ? 0 : 64 * (i - 1), ts.at.tok0, dst,
+                                                   ts.at.blk[0], dst + kHalf * 128, ts.at.blk[1], ts.at.nh > 1,
+                                                   i == 0 ? pol_drop : pol_keep, &map_q, 64 * (i == 0 ? ncc : i - 1),
+                                                   ts.w.b * a.rows + group * N, dst + kChunkBytes, pol_keep);
+                        } else {
+                            cache_box(i);
+                            if constexpr (SQ) query_box(i, rp.slot, ts.w.b);
+                        }
                         rp.advance(CA);
                     }
                     i = 0;

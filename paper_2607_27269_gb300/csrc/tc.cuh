@@ -301,6 +301,44 @@ __device__ __forceinline__ void tma_load_3d_hint_elect(uint32_t dst, const CUten
         : "memory");
 }
 
+// One refill of a ring slot in one election: the bytes to expect on `mbar`, a
+// 3-d box at `dst`, a second one at `dst2` unless `one`, and (if `map_q`) a 2-d box at `dst_q`.
+__device__ __forceinline__ void tma_refill_elect(uint32_t mbar, uint32_t bytes, const CUtensorMap *map, int32_t c0, int32_t c1,
+                                                 uint32_t dst, int32_t blk, uint32_t dst2, int32_t blk2, uint32_t two,
+                                                 uint64_t policy)
+{
+    asm volatile(
+        "{\n .reg .pred e, f, t;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 t, %9, 0;\n and.pred f, e, t;\n"
+        " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+        " @e cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%5], [%2, {%3, "
+        "%4, %6}], [%0], %10;\n"
+        " @f cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%7], [%2, {%3, "
+        "%4, %8}], [%0], %10;\n}\n" ::"r"(mbar),
+        "r"(bytes), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(dst), "r"(blk), "r"(dst2), "r"(blk2),
+        "r"(two), "l"(policy)
+        : "memory");
+}
+
+// The same with a 2-d box (of another map) as the last load.
+__device__ __forceinline__ void tma_refill_q_elect(uint32_t mbar, uint32_t bytes, const CUtensorMap *map, int32_t c0,
+                                                   int32_t c1, uint32_t dst, int32_t blk, uint32_t dst2, int32_t blk2,
+                                                   uint32_t two, uint64_t policy, const CUtensorMap *map_q, int32_t q0,
+                                                   int32_t q1, uint32_t dst_q, uint64_t policy_q)
+{
+    asm volatile(
+        "{\n .reg .pred e, f, t;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 t, %9, 0;\n and.pred f, e, t;\n"
+        " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+        " @e cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%5], [%2, {%3, "
+        "%4, %6}], [%0], %10;\n"
+        " @f cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%7], [%2, {%3, "
+        "%4, %8}], [%0], %10;\n"
+        " @e cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%14], [%11, "
+        "{%12, %13}], [%0], %15;\n}\n" ::"r"(mbar),
+        "r"(bytes), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(dst), "r"(blk), "r"(dst2), "r"(blk2),
+        "r"(two), "l"(policy), "l"(reinterpret_cast<uint64_t>(map_q)), "r"(q0), "r"(q1), "r"(dst_q), "l"(policy_q)
+        : "memory");
+}
+
 __device__ __forceinline__ void tma_load_2d_elect(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1,
                                                   uint32_t mbar)
 {
