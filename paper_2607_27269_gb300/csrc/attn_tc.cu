@@ -949,16 +949,11 @@ __global__ void __maxnreg__(128)
                         const uint32_t full = smem_u32(&bars.pv_full[rp.slot]), dst = ring + rp.slot * 2 * kChunkBytes;
                         ok = rp.round == 0 || mbar_wait_warp(smem_u32(&bars.pv_empty[rp.slot]), (rp.round - 1) & 1, lim_ns);
                         if (!ok) break;
-                        tc::mbar_arrive_expect_tx_elect(full, 2 * ts.at.bytes);
-#pragma unroll
-                        for (int k = 0; k < 2; ++k) {
-                            if (ts.at.nh > 0)
-                                tc::tma_load_3d_hint_elect(dst + k * kChunkBytes, &map_c, 64 * (2 * m + k), ts.at.tok0,
-                                                           ts.at.blk[0], full, pol_drop);
-                            if (ts.at.nh > 1)
-                                tc::tma_load_3d_hint_elect(dst + k * kChunkBytes + kHalf * 128, &map_c, 64 * (2 * m + k),
-                                                           ts.at.tok0, ts.at.blk[1], full, pol_drop);
-                        }
+                        if (ts.at.nh > 0)
+                            tc::tma_refill_pair_elect(full, 2 * ts.at.bytes, &map_c, 128 * m, ts.at.tok0, dst, kChunkBytes,
+                                                      ts.at.blk[0], kHalf * 128, ts.at.blk[1], ts.at.nh > 1, pol_drop);
+                        else
+                            tc::mbar_arrive_expect_tx_elect(full, 0);
                     }
                 }
             }

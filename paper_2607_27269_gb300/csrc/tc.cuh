@@ -339,6 +339,42 @@ __device__ __forceinline__ void tma_refill_q_elect(uint32_t mbar, uint32_t bytes
         : "memory");
 }
 
+// A ring entry of two column chunks `step` bytes apart (columns c0 and c0 + 64)
+// in one election: one box per chunk, or two (the second `half` bytes further on).
+__device__ __forceinline__ void tma_refill_pair_elect(uint32_t mbar, uint32_t bytes, const CUtensorMap *map, int32_t c0,
+                                                      int32_t c1, uint32_t dst, uint32_t step, int32_t blk, uint32_t half,
+                                                      int32_t blk2, uint32_t two, uint64_t policy)
+{
+    asm volatile(
+        "{\n .reg .pred e, f, t;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 t, %9, 0;\n and.pred f, e, t;\n"
+        " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
+        " @e cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%5], [%2, {%3, "
+        "%4, %6}], [%0], %10;\n"
+        " @f cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%7], [%2, {%3, "
+        "%4, %8}], [%0], %10;\n"
+        " @e cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%11], [%2, {%13, "
+        "%4, %6}], [%0], %10;\n"
+        " @f cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%12], [%2, {%13, "
+        "%4, %8}], [%0], %10;\n}\n" ::"r"(mbar),
+        "r"(bytes), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(dst), "r"(blk), "r"(dst + half), "r"(blk2),
+        "r"(two), "l"(policy), "r"(dst + step), "r"(dst + step + half), "r"(c0 + 64)
+        : "memory");
+}
+
+// Bring a box (or two) into L2.
+__device__ __forceinline__ void prefetch_3d_elect(const CUtensorMap *map, int32_t c0, int32_t c1, int32_t blk, int32_t blk2,
+                                                  uint32_t boxes, uint64_t policy)
+{
+    asm volatile(
+        "{\n .reg .pred e, f, g;\n elect.sync _|e, 0xffffffff;\n setp.gt.and.u32 f, %5, 0, e;\n"
+        " setp.gt.and.u32 g, %5, 1, e;\n"
+        " @f cp.async.bulk.prefetch.tensor.3d.L2.global.L2::cache_hint [%0, {%1, %2, %3}], %6;\n"
+        " @g cp.async.bulk.prefetch.tensor.3d.L2.global.L2::cache_hint [%0, {%1, %2, %4}], %6;\n}\n" ::"l"(
+            reinterpret_cast<uint64_t>(map)),
+        "r"(c0), "r"(c1), "r"(blk), "r"(blk2), "r"(boxes), "l"(policy)
+        : "memory");
+}
+
 __device__ __forceinline__ void tma_load_2d_elect(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1,
                                                   uint32_t mbar)
 {
