@@ -10,8 +10,8 @@
 // weight tile loaded by TMA, the fp32 accumulator in TMEM.  A GEMM whose tiles
 // would occupy few SMs (few rows, deep K: the output projection of a small
 // batch) splits K over a cluster of up to four CTAs; each leaves its partial
-// tile in shared memory and the cluster sums the partials in a fixed order
-// through distributed shared memory, so the result does not depend on timing.
+// tile in shared memory, sends every other CTA its share of it, and sums its own
+// share of the partials in a fixed order, so the result does not depend on timing.
 //
 // The same kernel, with PROJ set, projects the step's hidden states (the step
 // before the cache append, Sec. 3.2 and Eq. 1): rows are the entries
@@ -31,6 +31,7 @@ namespace {
 
 __device__ __forceinline__ int64_t phys_row(const GroupGemm &p, int g, int m)
 {
+    if (p.hpg == 1) return static_cast<int64_t>(m) * p.blk + g;
     return static_cast<int64_t>(m / p.hpg) * p.blk + g * p.hpg + m % p.hpg;
 }
 
@@ -53,16 +54,58 @@ struct ProjEpi {
     int q_len;
 };
 
-__device__ __forceinline__ void store16_bf16(uint16_t *dst, const uint32_t (&v)[16])
+// The bf16 results of a warp's 32 tile rows x BN columns, from TMEM to memory:
+// 64 columns at a time go through a staging block (32 rows of 144 bytes: both
+// sides free of bank conflicts), so that eight lanes store 128 contiguous bytes
+// of a row.  store(col) returns, for a lane's eight columns from col, what
+// stores them for the warp's row r (called by every lane).  Each lane storing its
+// own row, 16 bytes a lane in 32 places, took 6800 cycles for the projection's 192
+// columns; this 3400, of which the stores (32 bytes a clock an SM) 2500.
+constexpr int kDrainRow = 144, kDrainWarp = 32 * kDrainRow, kDrainBytes = 4 * kDrainWarp;
+
+__device__ __forceinline__ uint16_t *shfl_ptr(uint16_t *p, int lane)
 {
-    uint32_t w[8];
+    return reinterpret_cast<uint16_t *>(__shfl_sync(0xffffffffu, reinterpret_cast<unsigned long long>(p), lane));
+}
+
+// 16 bytes to dst if ok: a predicated store, no branch
+__device__ __forceinline__ void store16_if(bool ok, uint16_t *dst, const uint4 &v)
+{
+    asm volatile("{.reg .pred p; setp.ne.u32 p, %0, 0; @p st.global.v4.b32 [%1], {%2, %3, %4, %5};}" ::"r"(
+                     static_cast<uint32_t>(ok)),
+                 "l"(dst), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w)
+                 : "memory");
+}
+
+template <int BN, class Store>
+__device__ __forceinline__ void drain_tile(uint32_t t_lane, unsigned char *stage, int lane, Store store)
+{
+#pragma unroll 1
+    for (int j = 0; j < BN; j += 64) {
+        uint32_t v[4][16];
 #pragma unroll
-    for (int e = 0; e < 8; ++e) {
-        const __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
-        w[e] = *reinterpret_cast<const uint32_t *>(&b);
+        for (int u = 0; u < 4; ++u) tc::ld_32x32b_x16(t_lane + j + 16 * u, v[u]);
+        tc::wait_ld();
+        __syncwarp();  // the block before has been read
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            uint32_t w[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int c = 8 * (k & 1) + 2 * e;
+                const __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float(v[k >> 1][c]), __uint_as_float(v[k >> 1][c + 1]));
+                w[e] = *reinterpret_cast<const uint32_t *>(&b);
+            }
+            *reinterpret_cast<uint4 *>(stage + lane * kDrainRow + 16 * k) = make_uint4(w[0], w[1], w[2], w[3]);
+        }
+        __syncwarp();
+        const auto row = store(j + 8 * (lane & 7));
+#pragma unroll
+        for (int rr = 0; rr < 8; ++rr) {
+            const int r = 4 * rr + (lane >> 3);
+            row(r, *reinterpret_cast<const uint4 *>(stage + r * kDrainRow + 16 * (lane & 7)));
+        }
     }
-    reinterpret_cast<uint4 *>(dst)[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    reinterpret_cast<uint4 *>(dst)[1] = make_uint4(w[4], w[5], w[6], w[7]);
 }
 
 // R_pos of the DR projected positional-key values x (fp32; the angle reduced
@@ -94,46 +137,33 @@ __device__ __forceinline__ void rotate_store(const float (&x)[64], int64_t pos, 
     for (int v = 0; v < DR / 8; ++v) reinterpret_cast<uint4 *>(row)[v] = reinterpret_cast<const uint4 *>(y)[v];
 }
 
-// Projection epilogue for tile row m (the entry h[m / n_new, m % n_new]);
-// every lane of the warp calls it (the TMEM loads are warp-collective).
+// Projection epilogue of a warp: `rows` tile rows from row m of this lane
+// (the entry h[m / n_new, m % n_new]); every lane of the warp calls it.
 template <int BN>
-__device__ void proj_epilogue(const GroupGemm &p, const ProjEpi &e, uint32_t t_lane, int m, bool row_ok)
+__device__ void proj_epilogue(const GroupGemm &p, const ProjEpi &e, uint32_t t_lane, unsigned char *stage, int lane, int m,
+                              int rows)
 {
     const int ty = blockIdx.y;
     if (ty > e.tiles_lat) {
-        // ---- queries: column c of W^Q is element c % dq of head c / dq
+        // ---- queries: column c of W^Q is element c % dq of head c / dq (eight
+        // columns from a multiple of eight are of one part of one head: d_nope
+        // and d_rope are multiples of eight)
         const int dq = e.d_nope + e.d_rope, nq = e.heads * dq;
-        const int c0 = (ty - e.tiles_lat - 1) * BN;
-#pragma unroll 1
-        for (int j = 0; j < BN; j += 16) {
-            uint32_t v[16];
-            tc::ld_32x32b_x16(t_lane + j, v);
-            tc::wait_ld();
-            const int c = c0 + j;
-            if (!row_ok || c >= nq) continue;
-            const int head = c / dq, el = c % dq;
-            const int64_t hrow = static_cast<int64_t>(m) * e.heads + head;
-            if (c + 16 <= nq && el + 16 <= e.d_nope) {
-                store16_bf16(e.q_nope + hrow * e.d_nope + el, v);
-            } else if (c + 16 <= nq && el >= e.d_nope && el + 16 <= dq) {
-                store16_bf16(e.q_pe + hrow * e.d_rope + (el - e.d_nope), v);
-            } else {
-                for (int u = 0; u < 16 && c + u < nq; ++u) {
-                    const int hu = (c + u) / dq, eu = (c + u) % dq;
-                    const int64_t r = static_cast<int64_t>(m) * e.heads + hu;
-                    const uint16_t b = __bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(v[u])));
-                    if (eu < e.d_nope)
-                        e.q_nope[r * e.d_nope + eu] = b;
-                    else
-                        e.q_pe[r * e.d_rope + (eu - e.d_nope)] = b;
-                }
-            }
-        }
+        const int c0 = (ty - e.tiles_lat - 1) * BN, mw = m - lane;
+        drain_tile<BN>(t_lane, stage, lane, [&](int col) {
+            const int c = c0 + col, head = c / dq, el = c - head * dq;
+            const int width = el < e.d_nope ? e.d_nope : e.d_rope;
+            uint16_t *dst = el < e.d_nope ? e.q_nope + el : e.q_pe + (el - e.d_nope);
+            dst += (static_cast<int64_t>(mw) * e.heads + head) * width;
+            const int64_t step = static_cast<int64_t>(e.heads) * width;  // row to row
+            const int rows_c = c < nq ? rows : 0;
+            return [=](int r, const uint4 &v) { store16_if(r < rows_c, dst + r * step, v); };
+        });
         return;
     }
     // ---- the entry's cache row: position start_pos[b] + k, through the block table when paged
     const CacheView &c = e.cache;
-    bool ok = row_ok;
+    bool ok = lane < rows;
     int64_t pos = 0, blk = 0, slot = 0;
     if (ok) {
         const int b = m / e.n_new, k = m % e.n_new;
@@ -152,14 +182,15 @@ __device__ void proj_epilogue(const GroupGemm &p, const ProjEpi &e, uint32_t t_l
     }
     if (ty < e.tiles_lat) {
         // ---- latent c = W^DKV h, rounded once
-        uint16_t *crow = static_cast<uint16_t *>(const_cast<void *>(c.c_kv)) + blk * c.c_blk + slot * c.c_tok;
-#pragma unroll 1
-        for (int j = 0; j < BN; j += 16) {
-            uint32_t v[16];
-            tc::ld_32x32b_x16(t_lane + j, v);
-            tc::wait_ld();
-            if (ok && ty * BN + j < e.rank) store16_bf16(crow + ty * BN + j, v);  // (the last tile may reach past the latent)
-        }
+        uint16_t *crow = ok ? static_cast<uint16_t *>(const_cast<void *>(c.c_kv)) + blk * c.c_blk + slot * c.c_tok : nullptr;
+        drain_tile<BN>(t_lane, stage, lane, [&](int col) {
+            const int n = ty * BN + col;
+            const bool in = n < e.rank;  // (the last tile may reach past the latent)
+            return [=](int r, const uint4 &v) {
+                uint16_t *row = shfl_ptr(crow, r);
+                store16_if(row && in, row + n, v);
+            };
+        });
         return;
     }
     // ---- positional key R_pos W^KR h (d_rope = 32 or 64 columns of this tile)
@@ -192,10 +223,13 @@ __device__ void proj_epilogue(const GroupGemm &p, const ProjEpi &e, uint32_t t_l
 // the 128B-swizzled K-major layout the MMA reads; an fp32 A (o_lat) lands as
 // two 32-column boxes in a staging tile, which four warps convert to bf16.
 constexpr int kStages = 16;  // most ring stages; fewer when K is short or shared memory runs out
+// Rows of one column group of a split-K partial as received: 1 mod 8, so that
+// lanes on different column groups of a row read different banks.
+__host__ __device__ constexpr int recv_rows(int rt) { return (rt + 7) / 8 * 8 + 1; }
 constexpr int kGemmThreads = 192;  // warp 0 TMA, warp 1 MMA, warps 2..5 convert / epilogue
 
 struct __align__(8) GemmBars {
-    uint64_t full[kStages], raw_full[kStages], conv_done[kStages], empty[kStages], done;
+    uint64_t full[kStages], raw_full[kStages], conv_done[kStages], empty[kStages], done, recv;
 };
 
 // BN: columns per CTA.  NMAJ: the weight is N-major.  AF32: A is fp32.
@@ -209,7 +243,6 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
                                                                const __grid_constant__ ProjEpi pe)
 {
     static_assert(!PROJ || (!NMAJ && !AF32), "the projection reads bf16 h and K-major weights");
-    constexpr int kABytes = 128 * 128;     // 128 rows x 64 K, bf16, SW128 K-major
     constexpr int kRawBytes = AF32 ? 2 * 128 * 128 : 0;  // two 32-column fp32 boxes
     constexpr uint32_t kTmem = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;  // accumulator columns
     constexpr int kBBytes = BN * 128;      // BN x 64 K (K-major) or 64 K x BN (N-major)
@@ -224,16 +257,14 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
     const int kz = blockIdx.x % ks;                      // this CTA's share: chunks [c_begin, c_end)
     const int c_begin = kz * nk / ks, nkl = (kz + 1) * nk / ks - c_begin;
     const int NS = p.stages;                             // ring stages (<= kStages)
-    // A stages sit a_stride apart: a full tile, or for a bf16 A of RT <= 64
-    // rows just those rows (rounded to 8).  The M = 128 MMA still reads 128
-    // rows from its stage base: the rows past RT come from the next stages or
-    // the B ring (inside the allocation), land in accumulator rows >= RT and
-    // are never stored.
+    // A stages sit a_stride apart: the tile's RT rows (rounded to 8).  The M = 128
+    // MMA still reads 128 rows from its stage base: the rows past RT come from
+    // the next stages or the B ring (inside the allocation), land in accumulator
+    // rows >= RT and are never stored.
     // An fp32 A has no A stages of its own: each converter thread writes its
     // bf16 row over the first half of its raw fp32 row, which it has read
-    // before (chunk j of the row is written after the step that read it), so
-    // a stage's bf16 tile is the first 16 KB of its raw stage.
-    const int AS = AF32 ? 0 : PROJ ? kABytes : p.a_stride;
+    // before, so a stage's bf16 tile is the first 16 KB of its raw stage.
+    const int AS = AF32 ? 0 : p.a_stride;
     unsigned char *sa = smem;                            // NS x A tile (bf16 A)
     unsigned char *sb = sa + NS * AS;                    // NS x B tile
     unsigned char *sr = sb + NS * kBBytes;               // NS x raw fp32 A, then its bf16 tile (AF32)
@@ -252,8 +283,11 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
             mbar_init(&bars.empty[s], 1);
         }
         mbar_init(&bars.done, 1);
+        mbar_init(&bars.recv, 1);
         fail = 0;
         tc::fence_barrier_init();
+        if (!PROJ && ks > 1)  // the slabs of the other CTAs
+            tc::mbar_arrive_expect_tx(smem_u32(&bars.recv), static_cast<uint32_t>((ks - 1) * (BN / ks) * recv_rows(RT) * 4));
     }
     if (warp == 1) {
         tc::tmem_alloc(smem_u32(&tmem_base), kTmem);
@@ -264,7 +298,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
     tc::fence_after_sync();
     // a peer's shared memory is written only once its CTA has started: arrive
     // now, wait before the first such write
-    if (!PROJ && ks > 1 && p.recv_off) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    if (!PROJ && ks > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     // the activations come from the previous launch; with early_weights the
     // producer sends for the first weight tiles before it waits
     const bool early = !PROJ && p.early_weights && warp == 0;
@@ -318,12 +352,15 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
             }
         };
         const int head = nkl < NS ? nkl : NS;  // the ring's first round
-        for (int s = 0; s < head; ++s) load_b(c_begin + s, s);
+        for (int s = 0; s < head; ++s) {
+            load_b(c_begin + s, s);
+            if (!early) load_a(c_begin + s, s);
+        }
         if (early) {
             griddep_wait();
             griddep_launch_dependents();
+            for (int s = 0; s < head; ++s) load_a(c_begin + s, s);
         }
-        for (int s = 0; s < head; ++s) load_a(c_begin + s, s);
         for (int c = c_begin + head, s = 0, par = 0; c < c_begin + nkl; ++c) {
             if (!mbar_wait_warp(smem_u32(&bars.empty[s]), par, lim)) {
                 if (lane == 0) bail();
@@ -364,7 +401,9 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
         tc::commit_elect(smem_u32(&bars.done));
     } else {
         if (AF32) {
-            // ---- fp32 -> bf16: thread r converts tile row r (two 128-byte swizzled fp32 rows)
+            // ---- fp32 -> bf16: thread r converts tile row r (two 128-byte
+            // swizzled fp32 rows), all of it read before the first write: in
+            // turns, each write held back the next read, 900 cycles a chunk
             const int r = tid - 64;
             for (int cc = 0, s = 0, par = 0; cc < nkl; ++cc) {
                 if (!mbar_wait_warp(smem_u32(&bars.raw_full[s]), par, lim)) {
@@ -374,15 +413,16 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
                 const uint4 *src0 = reinterpret_cast<const uint4 *>(sr + s * kRawBytes + r * 128);
                 const uint4 *src1 = reinterpret_cast<const uint4 *>(sr + s * kRawBytes + 128 * 128 + r * 128);
                 uint4 *dst = reinterpret_cast<uint4 *>(sr + s * kRawBytes + r * 128);  // over src0, in place
+                float4 x[16];
+#pragma unroll
+                for (int j = 0; j < 16; ++j)
+                    x[j] = *reinterpret_cast<const float4 *>(&(j < 8 ? src0 : src1)[(j & 7) ^ (r & 7)]);
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    // bf16 16-byte chunk j = fp32 chunks 2j, 2j + 1 (of box j / 4)
-                    const uint4 *src = j < 4 ? src0 : src1;
-                    const int q0 = (2 * j) & 7, q1 = (2 * j + 1) & 7;
-                    const float4 x = *reinterpret_cast<const float4 *>(&src[q0 ^ (r & 7)]);
-                    const float4 y = *reinterpret_cast<const float4 *>(&src[q1 ^ (r & 7)]);
-                    const __nv_bfloat162 b0 = __floats2bfloat162_rn(x.x, x.y), b1 = __floats2bfloat162_rn(x.z, x.w);
-                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(y.x, y.y), b3 = __floats2bfloat162_rn(y.z, y.w);
+                    // bf16 16-byte chunk j = fp32 chunks 2j, 2j + 1
+                    const float4 a = x[2 * j], b = x[2 * j + 1];
+                    const __nv_bfloat162 b0 = __floats2bfloat162_rn(a.x, a.y), b1 = __floats2bfloat162_rn(a.z, a.w);
+                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(b.x, b.y), b3 = __floats2bfloat162_rn(b.z, b.w);
                     dst[j ^ (r & 7)] =
                         make_uint4(*reinterpret_cast<const uint32_t *>(&b0), *reinterpret_cast<const uint32_t *>(&b1),
                                    *reinterpret_cast<const uint32_t *>(&b2), *reinterpret_cast<const uint32_t *>(&b3));
@@ -445,78 +485,95 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
             const int q = warp & 3;
             const int i = q * 32 + lane;  // tile row
             const int me = m0 + i;
-            const bool row_ok = i < RT && me < p.M;
             const uint32_t t_lane = tmem + (static_cast<uint32_t>(q * 32) << 16);
-            const int64_t orow = row_ok ? phys_row(p, g, me) : 0;
+            unsigned char *stage = smem + q * kDrainWarp;  // in the ring: its tiles have been read
             if (PROJ) {
-                proj_epilogue<BN>(p, pe, t_lane, me, row_ok);
+                const int rows = min(RT, p.M - m0) - q * 32;
+                proj_epilogue<BN>(p, pe, t_lane, stage, lane, me, rows);
             } else if (ks > 1) {
                 ep_ok = true;  // the partial is pushed once the whole cluster is past its MMAs
             } else {
-#pragma unroll 1
-            for (int j = 0; j < BN; j += 16) {
-                uint32_t v[16];
-                tc::ld_32x32b_x16(t_lane + j, v);
-                tc::wait_ld();
-                const int n = n0 + j;
-                if (!row_ok || n >= p.N) continue;
-                uint16_t *dst = static_cast<uint16_t *>(p.C) + orow * p.ldc + n;
-                if (n + 16 <= p.N) {
-                    store16_bf16(dst, v);
-                } else {
-                    for (int e = 0; e < 16 && n + e < p.N; ++e)
-                        dst[e] = __bfloat16_as_ushort(__float2bfloat16_rn(__uint_as_float(v[e])));
-                }
-            }
+                const bool vec = p.ldc % 8 == 0;  // 16-byte stores
+                uint16_t *crow = i < RT && me < p.M ? static_cast<uint16_t *>(p.C) + phys_row(p, g, me) * p.ldc : nullptr;
+                drain_tile<BN>(t_lane, stage, lane, [&](int col) {
+                    const int n = n0 + col;
+                    const bool full = vec && n + 8 <= p.N;
+                    const int left = full ? 0 : p.N - n;  // columns to store one by one
+                    return [=](int r, const uint4 &v) {
+                        uint16_t *row = shfl_ptr(crow, r);
+                        store16_if(row && full, row + n, v);
+                        if (row && left > 0) {
+                            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                            for (int e = 0; e < 8; ++e)
+                                if (e < left) row[n + e] = static_cast<uint16_t>(w[e / 2] >> (16 * (e % 2)));
+                        }
+                    };
+                });
             }
         }
     }
     if (!PROJ && ks > 1) {
-        // (1) push this CTA's partial of each column slice to the slice's owner:
-        // CTA o owns columns [o cw, (o + 1) cw) and receives, behind its ring
-        // (or in it, once every CTA of the cluster is past its MMAs),
-        // recv[r][row][cw + 4] from every rank r; (2) each owner sums its slice
-        // in rank order (four columns per step) and stores the bf16 result.
-        // Nothing is written to a peer after the second barrier.
-        const int cw = BN / ks;
-        if (p.recv_off)
-            asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA has started
-        else
-            tc::cluster_sync();
+        // (1) the CTA's partial into its ring (its own MMAs are done), a slab
+        // [four columns][row] for every owner: CTA o owns columns [o cw, (o + 1)
+        // cw); (2) one bulk copy a peer takes its slab there, behind the peer's
+        // ring, and completes on the peer's barrier; (3) each owner sums its slice in rank
+        // order (four columns per step) and stores the bf16 result.  Remote
+        // stores of the same 30 KB, 512 bytes a warp, and a cluster barrier took
+        // 2700 cycles where the copies take 1900.
+        const int cw = BN / ks, RP = recv_rows(RT);
+        asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA has started
         if (warp >= 2 && ep_ok && !fail) {
             tc::fence_after_sync();
             const int q = warp & 3, i = q * 32 + lane;
             const uint32_t t_lane = tmem + (static_cast<uint32_t>(q * 32) << 16);
-            const uint32_t recv = smem_u32(smem) + p.recv_off;
 #pragma unroll 1
-            for (int j = 0; j < BN; j += 16) {
-                uint32_t v[16];
-                tc::ld_32x32b_x16(t_lane + j, v);
-                tc::wait_ld();
-                if (i < RT) {
-                    const int o = j / cw;
-                    const uint32_t local = recv + static_cast<uint32_t>(((kz * RT + i) * (cw + 4) + (j - o * cw)) * 4);
-                    uint32_t remote;
-                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(o));
+            for (int j = 0; j < BN; j += 64) {
+                uint32_t v[4][16];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e)
-                        asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(remote + 16 * e),
-                                     "f"(__uint_as_float(v[4 * e])), "f"(__uint_as_float(v[4 * e + 1])),
-                                     "f"(__uint_as_float(v[4 * e + 2])), "f"(__uint_as_float(v[4 * e + 3]))
-                                     : "memory");
+                for (int u = 0; u < 4; ++u) tc::ld_32x32b_x16(t_lane + j + 16 * u, v[u]);
+                tc::wait_ld();
+                if (i < RT) {  // (the slabs of the owners follow one another: column c at group c / 4)
+                    float4 *dst = reinterpret_cast<float4 *>(smem) + j / 4 * RP + i;
+#pragma unroll
+                    for (int e = 0; e < 16; ++e)
+                        dst[e * RP] = make_float4(__uint_as_float(v[e / 4][4 * (e % 4)]), __uint_as_float(v[e / 4][4 * (e % 4) + 1]),
+                                                  __uint_as_float(v[e / 4][4 * (e % 4) + 2]),
+                                                  __uint_as_float(v[e / 4][4 * (e % 4) + 3]));
+                }
+                __syncwarp();
+            }
+            tc::fence_proxy_async_smem();
+        }
+        const uint32_t slab = static_cast<uint32_t>(cw * RP * 4);
+        bool got = false;
+        if (warp >= 2) {
+            asm volatile("bar.sync 1, 128;" ::: "memory");
+            if (warp == 2 && lane == 0 && ep_ok && !fail) {
+                for (int d = 1; d < ks; ++d) {
+                    const uint32_t o = static_cast<uint32_t>((kz + d) & (ks - 1));
+                    tc::bulk_copy_cluster(tc::mapa(smem_u32(smem) + p.recv_off + kz * slab, o), smem_u32(smem) + o * slab, slab,
+                                          tc::mapa(smem_u32(&bars.recv), o));
                 }
             }
+            got = mbar_wait_warp(smem_u32(&bars.recv), 0, lim);
+            if (!got && lane == 0) bail();
         }
-        tc::cluster_sync();
-        if (warp >= 2 && !fail) {
-            const int q4 = cw / 4;
-            const float *recv = reinterpret_cast<const float *>(smem + p.recv_off);
-            for (int idx = tid - 64; idx < RT * q4; idx += 128) {
-                const int i = idx / q4, c4 = (idx % q4) * 4;
-                const int me = m0 + i, n = n0 + kz * cw + c4;
+        __syncwarp();
+        // a CTA leaves once every copy from its shared memory has landed
+        asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+        if (got && !fail) {
+            const int q4 = cw / 4;  // 4, 8, 16 or 32: the 128 threads keep their columns and step 128 / q4 rows
+            const float4 *own = reinterpret_cast<const float4 *>(smem), *recv = reinterpret_cast<const float4 *>(smem + p.recv_off);
+            const int ce = (tid - 64) % q4, n = n0 + kz * cw + 4 * ce;
+#pragma unroll 2
+            for (int i = (tid - 64) / q4; i < RT; i += 128 / q4) {
+                const int me = m0 + i;
                 float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-                for (int r = 0; r < ks; ++r) {
-                    const float4 v = *reinterpret_cast<const float4 *>(recv + (r * RT + i) * (cw + 4) + c4);
+#pragma unroll
+                for (int r = 0; r < 4; ++r) {  // ks is 2 or 4
+                    if (r >= ks) break;
+                    const float4 v = (r == kz ? own : recv)[(r * q4 + ce) * RP + i];
                     acc.x += v.x;
                     acc.y += v.y;
                     acc.z += v.z;
@@ -533,6 +590,8 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
                 }
             }
         }
+        __syncwarp();
+        asm volatile("barrier.cluster.wait.aligned;" ::: "memory");
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -592,19 +651,35 @@ int rows_per_tile(const GroupGemm &p)
     return (blocks + tiles - 1) / tiles;
 }
 
-// Ring depth: as many stages as fit 192 KB, at most kStages and the K chunks.
+// The ring for tiles of rt rows: as many stages as fit `budget` bytes, at most
+// kStages and the K chunks.  A bf16 A stage holds just the tile's rows (rounded
+// to 8), so that short tiles stream their weight with more chunks in flight.
+struct Ring {
+    int stages, a_stride;
+    size_t bytes;
+};
+
 template <int BN, bool AF32>
-int ring_stages(int K, size_t *smem)
+Ring ring_for(int rt, int chunks, size_t budget)
 {
-    const int nk = (K + 63) / 64;
-    const size_t per_stage = (AF32 ? 2 * 128 * 128 : 128 * 128) + BN * 128;  // fp32 A: raw stage, bf16 in place
-    int ns = static_cast<int>((192 * 1024) / per_stage);
+    Ring r;
+    r.a_stride = (rt + 7) / 8 * 8 * 128;
+    const size_t per_stage = (AF32 ? 2 * 128 * 128 : r.a_stride) + BN * 128;  // fp32 A: raw stage, bf16 in place
+    int ns = static_cast<int>(budget / per_stage);
     if (ns > kStages) ns = kStages;
-    if (ns > nk) ns = nk;
-    if (ns < 1) ns = 1;
-    *smem = 1024 + static_cast<size_t>(ns) * per_stage;
-    return ns;
+    if (ns > chunks) ns = chunks;
+    r.stages = ns < 1 ? 1 : ns;
+    r.bytes = r.stages * per_stage;
+    // the last stage's MMA reads a full 128-row window from its base
+    const size_t window = static_cast<size_t>(r.stages - 1) * r.a_stride + 128 * 128;
+    if (!AF32 && r.bytes < window) r.bytes = window;
+    return r;
 }
+
+// Shared memory of a CTA that has an SM for itself, behind the alignment of the
+// ring; 640 rows of the projection (40 KB a chunk) 14.8 us with a ring of four
+// chunks, 13.6 with the five that fit.
+constexpr size_t kRingBytes = 224 * 1024;
 
 template <int BN, bool NMAJ, bool AF32>
 cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope = nullptr)
@@ -638,68 +713,37 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     const int mtiles = (p.M + rt - 1) / rt;
     // Split K over a cluster when the tiles are short (<= 64 rows: a small
     // batch), K is deep (>= 8 chunks) and the tiles alone would leave most SMs
-    // idle: up to 4 ways, at least two chunks each, with a ring of at most 4
-    // stages so that two CTAs share an SM and the split grid runs in one wave.
+    // idle: up to 4 ways, at least two chunks each, with a ring that lets two
+    // CTAs share an SM, so that the split grid runs in one wave.
     const int64_t tiles = static_cast<int64_t>(mtiles) * ntiles * p.G;
     int ks = 1;
     if (rt <= 64 && nk >= 8)
         while (ks < 4 && tiles * ks * 2 <= (AF32 ? 152 : 2 * 152) && nk >= 4 * ks) ks *= 2;  // fp32 A: one CTA per SM
     // Full 128-row tiles that would fill fewer than half the SMs (a mid-size
     // batch against a wide weight): split K as well, one CTA per SM, at least
-    // eight chunks per share, the partials (128 rows x BN / ks columns from
-    // each rank) pushed into the ring.  (Not for an fp32 A: there the
-    // reduction cost as much as the split saved.)
+    // eight chunks per share.  (Not for an fp32 A: there the reduction cost as
+    // much as the split saved.)
     const bool wide_split = rt > 64 && !AF32 && nk >= 16 && tiles * 2 <= 152;
     if (wide_split)
         while (ks < 4 && tiles * ks * 2 <= 152 && nk >= 8 * ks) ks *= 2;
-    size_t smem = 0;
+    // Split K: the partial's staging lies in the ring, what the cluster sends
+    // behind it (at most 66 KB each).  A short tile's ring leaves room for a
+    // second CTA.
+    const size_t part = ks > 1 ? static_cast<size_t>(BN) * recv_rows(rt) * 4 : 0;
+    const size_t room = ks > 1 && rt <= 64 && !AF32 ? 111 * 1024 : kRingBytes;
+    size_t budget = room - part;
+    // an fp32-A grid just past one CTA per SM (W_UV of a large batch):
+    // two stages, so that two CTAs share an SM and the grid runs in one wave
+    if (AF32 && ks == 1 && tiles > 152 && tiles <= 2 * 152) budget = 2 * (2 * 128 * 128 + BN * 128);
+    const Ring ring = ring_for<BN, AF32>(rt, (nk + ks - 1) / ks, budget);
     GroupGemm q = p;
-    q.a_stride = 128 * 128;
-    if (!AF32 && rt <= 64) {
-        // short bf16 A tiles: stages of RT rows (rounded to 8), so that the ring
-        // holds many more weight chunks -- with a split, all of a CTA's chunks
-        // at two CTAs per SM -- and the weights stream with more bytes in flight
-        q.a_stride = (rt + 7) / 8 * 8 * 128;
-        const int nkl = (nk + ks - 1) / ks;
-        const size_t per_stage = static_cast<size_t>(q.a_stride) + BN * 128;
-        const size_t budget = ks > 1 ? 110 * 1024 : 192 * 1024;
-        int ns = static_cast<int>(budget / per_stage);
-        ns = ns > kStages ? kStages : ns;
-        ns = ns > nkl ? nkl : ns;
-        q.stages = ns < 1 ? 1 : ns;
-        // the last stage's MMA reads a full 128-row window from its base
-        const size_t ring = static_cast<size_t>(q.stages) * per_stage;
-        const size_t window = static_cast<size_t>(q.stages - 1) * q.a_stride + 128 * 128;
-        smem = 1024 + (ring > window ? ring : window);
-    } else {
-        q.stages = ring_stages<BN, AF32>((nk + ks - 1) / ks * 64, &smem);
-        const size_t per_stage = (AF32 ? 2 * 128 * 128 : 128 * 128) + BN * 128;
-        if (ks > 1 && !wide_split && q.stages > 4) {
-            q.stages = 4;
-            smem = 1024 + 4 * per_stage;
-        }
-        // an fp32-A grid just past one CTA per SM (W_UV of a large batch):
-        // two stages, so that two CTAs share an SM and the grid runs in one wave
-        if (AF32 && ks == 1 && tiles > 152 && tiles <= 2 * 152 && q.stages > 2) {
-            q.stages = 2;
-            smem = 1024 + 2 * per_stage;
-        }
-    }
+    q.stages = ring.stages;
+    q.a_stride = ring.a_stride;
     q.rblk = rblk;
     q.ksplit = ks;
-    q.recv_off = 0;
-    if (ks > 1) {
-        // the partials received from the cluster: behind the ring where two such
-        // CTAs (of short tiles) or one (of full tiles) still fit an SM, so that a
-        // CTA pushes as soon as its own MMAs are done; else in the ring
-        const size_t recv = static_cast<size_t>(ks) * rt * (BN / ks + 4) * 4;
-        if (smem + recv <= (rt <= 64 ? 112u : 224u) * 1024) {
-            q.recv_off = static_cast<int>(smem - 1024);
-            smem += recv;
-        } else if (smem < 1024 + recv) {
-            smem = 1024 + recv;
-        }
-    }
+    q.recv_off = static_cast<int>(ring.bytes > part ? ring.bytes : part);
+    size_t smem = 1024 + (ks > 1 ? q.recv_off + part : ring.bytes);
+    if (smem < 1024 + kDrainBytes) smem = 1024 + kDrainBytes;  // the results' staging
     e = cudaFuncSetAttribute(gemm_tc_kernel<BN, NMAJ, AF32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
     if (e != cudaSuccess) return e;
@@ -758,10 +802,13 @@ cudaError_t launch_proj(const mla_dims &d, const CacheView &c, int batch, int n_
     }
     const int tiles = pe.tiles_lat + 1 + (nq + BN - 1) / BN;
     p.N = tiles * BN;
-    size_t smem = 0;
-    p.stages = ring_stages<BN, false>(p.K, &smem);
+    const Ring ring = ring_for<BN, false>(rblk, (p.K + 63) / 64, kRingBytes);
+    size_t smem = 1024 + ring.bytes;
+    p.stages = ring.stages;
+    p.a_stride = ring.a_stride;
     p.rblk = rblk;
     p.ksplit = 1;
+    if (smem < 1024 + kDrainBytes) smem = 1024 + kDrainBytes;  // the results' staging
     e = cudaFuncSetAttribute(gemm_tc_kernel<BN, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
     if (e != cudaSuccess) return e;

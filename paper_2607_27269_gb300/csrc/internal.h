@@ -114,7 +114,7 @@ struct GroupGemm {
     int early_weights = 0;
     int stages, rblk, ksplit;  // set by the launcher
     int a_stride;              // bytes between A ring stages (set by the launcher)
-    int recv_off;              // split K: where the cluster's partials arrive, bytes from the ring's start (0: in the ring)
+    int recv_off;              // split K: where the cluster's partials arrive, bytes from the ring's start
 };
 cudaError_t launch_group_gemm(const GroupGemm &p, cudaStream_t st);
 // The absorption GEMM (N-major W_UK, bf16 A) that also writes the rotated
