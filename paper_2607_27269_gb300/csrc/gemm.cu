@@ -651,6 +651,42 @@ int rows_per_tile(const GroupGemm &p)
     return (blocks + tiles - 1) / tiles;
 }
 
+// CTAs that share a tile's K range.  Split K over a cluster when the tiles are
+// short (<= 64 rows: a small batch), K is deep (>= 8 chunks) and the tiles alone
+// would leave most SMs idle: up to 4 ways, at least two chunks each, with a ring
+// that lets two CTAs share an SM, so that the split grid runs in one wave (an
+// fp32 A: one CTA per SM).  Tiles of more rows that would fill fewer than half
+// the SMs (a mid-size batch against a wide weight): split K as well, one CTA per
+// SM, at least eight chunks per share.  (Not for an fp32 A: there the reduction
+// cost as much as the split saved.)
+int split_of(bool f32, int rt, int64_t tiles, int nk)
+{
+    int ks = 1;
+    if (rt <= 64 && nk >= 8)
+        while (ks < 4 && tiles * ks * 2 <= (f32 ? 152 : 2 * 152) && nk >= 4 * ks) ks *= 2;
+    if (rt > 64 && !f32 && nk >= 16)
+        while (ks < 4 && tiles * ks * 2 <= 152 && nk >= 8 * ks) ks *= 2;
+    return ks;
+}
+
+// What column tiles of bn cost (bf16 A), in KB through a CTA's shared memory:
+// its chunks of both operands, four times its partial if K is split (staged,
+// sent, received, summed) and 150 for the exchange's own latency, times the
+// waves of CTAs.  W_UV + W_O of 32 heads, 2048 columns, with 128 against 64
+// columns: 64 rows 12.6 and 11.2 us, 128 rows 13.9 and 12.6, 160 rows 13.3 and
+// 13.7, 320 rows 17.3 and 14.9, 512 rows 20.9 and 17.9, 640 rows (two waves of
+// 64) 21.7 and more.
+int64_t tile_cost(const GroupGemm &p, int bn)
+{
+    const int rt = rows_per_tile(p) * p.hpg, nk = (p.K + 63) / 64;
+    const int64_t tiles = static_cast<int64_t>((p.M + rt - 1) / rt) * ((p.N + bn - 1) / bn) * p.G;
+    const int ks = split_of(false, rt, tiles, nk);
+    const int64_t slots = ks > 1 && rt <= 64 ? 2 * 152 : 152;
+    const int64_t in = static_cast<int64_t>((nk + ks - 1) / ks) * (rt + bn) * 128;
+    const int64_t exchange = ks > 1 ? 4 * 4 * static_cast<int64_t>(rt) * bn + 150 * 1024 : 0;
+    return (tiles * ks + slots - 1) / slots * (in + exchange);
+}
+
 // The ring for tiles of rt rows: as many stages as fit `budget` bytes, at most
 // kStages and the K chunks.  A bf16 A stage holds just the tile's rows (rounded
 // to 8), so that short tiles stream their weight with more chunks in flight.
@@ -711,21 +747,8 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     }
     const int rt = rblk * p.hpg;
     const int mtiles = (p.M + rt - 1) / rt;
-    // Split K over a cluster when the tiles are short (<= 64 rows: a small
-    // batch), K is deep (>= 8 chunks) and the tiles alone would leave most SMs
-    // idle: up to 4 ways, at least two chunks each, with a ring that lets two
-    // CTAs share an SM, so that the split grid runs in one wave.
     const int64_t tiles = static_cast<int64_t>(mtiles) * ntiles * p.G;
-    int ks = 1;
-    if (rt <= 64 && nk >= 8)
-        while (ks < 4 && tiles * ks * 2 <= (AF32 ? 152 : 2 * 152) && nk >= 4 * ks) ks *= 2;  // fp32 A: one CTA per SM
-    // Full 128-row tiles that would fill fewer than half the SMs (a mid-size
-    // batch against a wide weight): split K as well, one CTA per SM, at least
-    // eight chunks per share.  (Not for an fp32 A: there the reduction cost as
-    // much as the split saved.)
-    const bool wide_split = rt > 64 && !AF32 && nk >= 16 && tiles * 2 <= 152;
-    if (wide_split)
-        while (ks < 4 && tiles * ks * 2 <= 152 && nk >= 8 * ks) ks *= 2;
+    const int ks = split_of(AF32, rt, tiles, nk);
     // Split K: the partial's staging lies in the ring, what the cluster sends
     // behind it (at most 66 KB each).  A short tile's ring leaves room for a
     // second CTA.
@@ -842,8 +865,8 @@ cudaError_t launch_group_gemm(const GroupGemm &p, cudaStream_t st)
 {
     if (p.M <= 0 || p.N <= 0 || p.G <= 0) return cudaSuccess;
     // column tile: 64 for narrow outputs and for few rows (more CTAs stream the
-    // weight), else 128
-    const bool narrow = p.N <= 64 || p.M <= 32;
+    // weight), else 128 -- or, of a bf16 A, what costs a CTA less
+    const bool narrow = p.N <= 64 || p.M <= 32 || (!p.a_f32 && tile_cost(p, 64) < tile_cost(p, 128));
     if (p.a_f32) {
         if (p.b_nmajor) return narrow ? launch_tc<64, true, true>(p, st) : launch_tc<128, true, true>(p, st);
         return narrow ? launch_tc<64, false, true>(p, st) : launch_tc<128, false, true>(p, st);

@@ -29,6 +29,8 @@ pytestmark = pytest.mark.gpu
     (160, 32, 8, 512, 64, 1030),  # split; rows of C at odd multiples of four bytes
     (160, 4, 2, 128, 64, 1030),   # the same rows unsplit (K of four chunks)
     (13, 14, 2, 256, 64, 898),    # short tiles, split, rows of C at odd multiples of four bytes
+    (200, 32, 8, 512, 64, 2048),  # two tiles of 100 rows, 128 columns wide, split
+    (384, 32, 8, 512, 64, 2044),  # three tiles, 64 columns wide, unsplit
     (300, 8, 4, 256, 128, 516),   # unsplit, rows of C eight-byte aligned
     (700, 16, 4, 192, 40, 1024),  # 40-wide heads, three chunks of rank
 ])
