@@ -226,7 +226,14 @@ constexpr int kStages = 16;  // most ring stages; fewer when K is short or share
 // Rows of one column group of a split-K partial as received: 1 mod 8, so that
 // lanes on different column groups of a row read different banks.
 __host__ __device__ constexpr int recv_rows(int rt) { return (rt + 7) / 8 * 8 + 1; }
-constexpr int kGemmThreads = 192;  // warp 0 TMA, warp 1 MMA, warps 2..5 convert / epilogue
+// warp 0 TMA, warp 1 MMA, warps 2..5 epilogue; of an fp32 A, warps 2..5 convert
+// too, and in a launch of kConvThreads warps 6..9: two sets of four warps take
+// turns with the ring's stages, so that one set's latency (wait, read, write,
+// proxy fence: 850 cycles a chunk) hides behind the other's.  W_UV + W_O of 32
+// heads: 32 rows 10.4 -> 9.9 us, 160 rows 13.2 -> 12.8.  Where K is split (two
+// chunks a CTA: one row 7.9 -> 8.2) or two CTAs share an SM (640 rows 21.7 ->
+// 21.8), one set remains.
+constexpr int kGemmThreads = 192, kConvThreads = 320;
 
 struct __align__(8) GemmBars {
     uint64_t full[kStages], raw_full[kStages], conv_done[kStages], empty[kStages], done, recv;
@@ -235,7 +242,7 @@ struct __align__(8) GemmBars {
 // BN: columns per CTA.  NMAJ: the weight is N-major.  AF32: A is fp32.
 // PROJ: the projection (K-major weights map_b, map_b2, map_b3 by column region).
 template <int BN, bool NMAJ, bool AF32, bool PROJ>
-__global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_constant__ GroupGemm p,
+__global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_kernel(const __grid_constant__ GroupGemm p,
                                                                const __grid_constant__ CUtensorMap map_a,
                                                                const __grid_constant__ CUtensorMap map_b,
                                                                const __grid_constant__ CUtensorMap map_b2,
@@ -269,6 +276,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
     unsigned char *sb = sa + NS * AS;                    // NS x B tile
     unsigned char *sr = sb + NS * kBBytes;               // NS x raw fp32 A, then its bf16 tile (AF32)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const bool epi = warp >= 2 && warp < 6;              // an epilogue warp
     const int R = p.rblk, RT = R * p.hpg;                // row blocks and rows per tile (<= 128)
     const int mt = blockIdx.x / ks, n0 = blockIdx.y * BN, g = blockIdx.z;
     const int m0 = mt * RT;
@@ -404,15 +412,24 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
             // ---- fp32 -> bf16: thread r converts tile row r (two 128-byte
             // swizzled fp32 rows), all of it read before the first write: in
             // turns, each write held back the next read, 900 cycles a chunk
-            const int r = tid - 64;
+            const int r = (tid - 64) & 127;
+            // A stage belongs to one set, which so waits for each of its phases in
+            // turn: a wait by parity must not miss one.
+            const int set = warp < 6 ? 0 : 1, sets = static_cast<int>(blockDim.x - 64) / 128;
             for (int cc = 0, s = 0, par = 0; cc < nkl; ++cc) {
-                if (!mbar_wait_warp(smem_u32(&bars.raw_full[s]), par, lim)) {
+                const int cs = s, cp = par;
+                if (++s == NS) {
+                    s = 0;
+                    par ^= 1;
+                }
+                if (sets == 2 && (cs & 1) != set) continue;
+                if (!mbar_wait_warp(smem_u32(&bars.raw_full[cs]), cp, lim)) {
                     if (lane == 0) bail();
                     break;
                 }
-                const uint4 *src0 = reinterpret_cast<const uint4 *>(sr + s * kRawBytes + r * 128);
-                const uint4 *src1 = reinterpret_cast<const uint4 *>(sr + s * kRawBytes + 128 * 128 + r * 128);
-                uint4 *dst = reinterpret_cast<uint4 *>(sr + s * kRawBytes + r * 128);  // over src0, in place
+                const uint4 *src0 = reinterpret_cast<const uint4 *>(sr + cs * kRawBytes + r * 128);
+                const uint4 *src1 = reinterpret_cast<const uint4 *>(sr + cs * kRawBytes + 128 * 128 + r * 128);
+                uint4 *dst = reinterpret_cast<uint4 *>(sr + cs * kRawBytes + r * 128);  // over src0, in place
                 float4 x[16];
 #pragma unroll
                 for (int j = 0; j < 16; ++j)
@@ -429,14 +446,10 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
                 }
                 tc::fence_proxy_async_smem();
                 __syncwarp();
-                if (lane == 0) tc::mbar_arrive(smem_u32(&bars.conv_done[s]));
-                if (++s == NS) {
-                    s = 0;
-                    par ^= 1;
-                }
+                if (lane == 0) tc::mbar_arrive(smem_u32(&bars.conv_done[cs]));
             }
         }
-        if (!PROJ && pe.rope_src) {
+        if (!PROJ && !AF32 && pe.rope_src) {
             // ---- the absorption's positional query, while the MMAs run.  The
             // tile's rows are whole (b, i) blocks of hpg heads (row m of group g
             // is head g hpg + m % hpg of token m / hpg), which share one
@@ -477,9 +490,9 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
             }
         }
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31
-        const bool ok = mbar_wait_warp(smem_u32(&bars.done), 0, lim);
+        const bool ok = epi && mbar_wait_warp(smem_u32(&bars.done), 0, lim);
         if (!ok) {
-            if (lane == 0) bail();
+            if (epi && lane == 0) bail();
         } else if (!fail) {
             tc::fence_after_sync();
             const int q = warp & 3;
@@ -523,7 +536,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
         // 2700 cycles where the copies take 1900.
         const int cw = BN / ks, RP = recv_rows(RT);
         asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA has started
-        if (warp >= 2 && ep_ok && !fail) {
+        if (ep_ok && !fail) {
             tc::fence_after_sync();
             const int q = warp & 3, i = q * 32 + lane;
             const uint32_t t_lane = tmem + (static_cast<uint32_t>(q * 32) << 16);
@@ -547,7 +560,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_tc_kernel(const __grid_cons
         }
         const uint32_t slab = static_cast<uint32_t>(cw * RP * 4);
         bool got = false;
-        if (warp >= 2) {
+        if (epi) {
             asm volatile("bar.sync 1, 128;" ::: "memory");
             if (warp == 2 && lane == 0 && ep_ok && !fail) {
                 for (int d = 1; d < ks; ++d) {
@@ -770,9 +783,10 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     e = cudaFuncSetAttribute(gemm_tc_kernel<BN, NMAJ, AF32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
     if (e != cudaSuccess) return e;
+    const int threads = AF32 && ks == 1 && q.stages > 2 ? kConvThreads : kGemmThreads;
     dim3 grid(mtiles * ks, ntiles, p.G);
     ProjEpi none{};
-    return launch_dependent(gemm_tc_kernel<BN, NMAJ, AF32, false>, grid, dim3(kGemmThreads), smem, st, ks, q, ma, mb,
+    return launch_dependent(gemm_tc_kernel<BN, NMAJ, AF32, false>, grid, dim3(threads), smem, st, ks, q, ma, mb,
                             mb, mb, rope ? *rope : none);
 }
 
