@@ -507,7 +507,6 @@ cudaError_t launch_absorb(const mla_dims &d, int batch, int q_len, const void *q
     p.a_f32 = 0;
     p.lda = d.d_nope;
     p.B = w_uk;
-    p.b_nmajor = 1;
     p.C = q_abs;
     p.ldc = d.rank + d.d_rope;
     p.status = status;

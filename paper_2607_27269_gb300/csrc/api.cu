@@ -565,7 +565,6 @@ mla_status mla_gqa_project(const mla_gqa_dims *dims, int32_t batch, int32_t n_ne
         p.a_f32 = 0;
         p.lda = hidden;
         p.B = w[k];
-        p.b_nmajor = 0;
         p.C = outs[k];
         p.ldc = cols[k];
         p.status = status;
@@ -597,7 +596,6 @@ mla_status mla_gqa_out_proj(const mla_gqa_dims *dims, int32_t batch, int32_t q_l
     p.a_f32 = 1;
     p.lda = p.K;
     p.B = w_o;
-    p.b_nmajor = 0;
     p.C = out;
     p.ldc = hidden;
     p.status = status;

@@ -231,9 +231,9 @@ __host__ __device__ constexpr int recv_rows(int rt) { return (rt + 7) / 8 * 8 + 
 // turns with the ring's stages, so that one set's latency (wait, read, write,
 // proxy fence: 850 cycles a chunk) hides behind the other's.  W_UV + W_O of 32
 // heads: 32 rows 10.4 -> 9.9 us, 160 rows 13.2 -> 12.8.  Where K is split (two
-// chunks a CTA: one row 7.9 -> 8.2) or two CTAs share an SM (640 rows 21.7 ->
-// 21.8), one set remains.
+// chunks a CTA: one row 7.9 -> 8.2) or two CTAs share an SM, one set remains.
 constexpr int kGemmThreads = 192, kConvThreads = 320;
+constexpr int kShortRows = 96;
 
 struct __align__(8) GemmBars {
     uint64_t full[kStages], raw_full[kStages], conv_done[kStages], empty[kStages], done, recv;
@@ -241,7 +241,10 @@ struct __align__(8) GemmBars {
 
 // BN: columns per CTA.  NMAJ: the weight is N-major.  AF32: A is fp32.
 // PROJ: the projection (K-major weights map_b, map_b2, map_b3 by column region).
-template <int BN, bool NMAJ, bool AF32, bool PROJ>
+// SHORT: an fp32 A in tiles of at most kShortRows rows, whose stages hold just
+// those (W_UV + W_O of 14 heads, one row 7.1 -> 6.6 us, 64 rows 8.0 -> 7.5);
+// with taller tiles the fixed stage is 1 to 2 percent faster.
+template <int BN, bool NMAJ, bool AF32, bool PROJ, bool SHORT>
 __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_kernel(const __grid_constant__ GroupGemm p,
                                                                const __grid_constant__ CUtensorMap map_a,
                                                                const __grid_constant__ CUtensorMap map_b,
@@ -250,7 +253,6 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
                                                                const __grid_constant__ ProjEpi pe)
 {
     static_assert(!PROJ || (!NMAJ && !AF32), "the projection reads bf16 h and K-major weights");
-    constexpr int kRawBytes = AF32 ? 2 * 128 * 128 : 0;  // two 32-column fp32 boxes
     constexpr uint32_t kTmem = BN <= 32 ? 32 : BN <= 64 ? 64 : BN <= 128 ? 128 : 256;  // accumulator columns
     constexpr int kBBytes = BN * 128;      // BN x 64 K (K-major) or 64 K x BN (N-major)
     extern __shared__ __align__(1024) unsigned char smem_raw[];
@@ -272,6 +274,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
     // bf16 row over the first half of its raw fp32 row, which it has read
     // before, so a stage's bf16 tile is the first 16 KB of its raw stage.
     const int AS = AF32 ? 0 : p.a_stride;
+    const int raw_box = SHORT ? p.a_stride : 128 * 128, raw_bytes = 2 * raw_box;  // fp32 A: two 32-column boxes
     unsigned char *sa = smem;                            // NS x A tile (bf16 A)
     unsigned char *sb = sa + NS * AS;                    // NS x B tile
     unsigned char *sr = sb + NS * kBBytes;               // NS x raw fp32 A, then its bf16 tile (AF32)
@@ -351,10 +354,10 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
         };
         auto load_a = [&](int c, int s) {
             if (AF32) {
-                const uint32_t rb = smem_u32(&bars.raw_full[s]), rdst = smem_u32(sr + s * kRawBytes);
+                const uint32_t rb = smem_u32(&bars.raw_full[s]), rdst = smem_u32(sr + s * raw_bytes);
                 tc::mbar_arrive_expect_tx_elect(rb, 2 * a_bytes);
                 tc::tma_load_4d_elect(rdst, &map_a, 64 * c, 0, g, mt * R, rb);
-                tc::tma_load_4d_elect(rdst + 128 * 128, &map_a, 64 * c + 32, 0, g, mt * R, rb);
+                tc::tma_load_4d_elect(rdst + raw_box, &map_a, 64 * c + 32, 0, g, mt * R, rb);
             } else {
                 tc::tma_load_4d_elect(smem_u32(sa + s * AS), &map_a, 64 * c, 0, g, mt * R, smem_u32(&bars.full[s]));
             }
@@ -397,7 +400,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
             if (!ok) break;
             tc::fence_after_sync();
             // four steps of 16 along K: 32 bytes of a K-major operand, 16 rows of an N-major one
-            tc::mma4_bf16_commit_elect(tmem, with_addr(da, smem_u32(AF32 ? sr + s * kRawBytes : sa + s * AS)),
+            tc::mma4_bf16_commit_elect(tmem, with_addr(da, smem_u32(AF32 ? sr + s * raw_bytes : sa + s * AS)),
                                        with_addr(db, smem_u32(sb + s * kBBytes)), idesc, cc != 0, 2, NMAJ ? 16 * 128 / 16 : 2,
                                        smem_u32(&bars.empty[s]));
             if (++s == NS) {
@@ -427,22 +430,24 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
                     if (lane == 0) bail();
                     break;
                 }
-                const uint4 *src0 = reinterpret_cast<const uint4 *>(sr + cs * kRawBytes + r * 128);
-                const uint4 *src1 = reinterpret_cast<const uint4 *>(sr + cs * kRawBytes + 128 * 128 + r * 128);
-                uint4 *dst = reinterpret_cast<uint4 *>(sr + cs * kRawBytes + r * 128);  // over src0, in place
-                float4 x[16];
+                if (!SHORT || r < RT) {
+                    const uint4 *src0 = reinterpret_cast<const uint4 *>(sr + cs * raw_bytes + r * 128);
+                    const uint4 *src1 = reinterpret_cast<const uint4 *>(sr + cs * raw_bytes + raw_box + r * 128);
+                    uint4 *dst = reinterpret_cast<uint4 *>(sr + cs * raw_bytes + r * 128);  // over src0, in place
+                    float4 x[16];
 #pragma unroll
-                for (int j = 0; j < 16; ++j)
-                    x[j] = *reinterpret_cast<const float4 *>(&(j < 8 ? src0 : src1)[(j & 7) ^ (r & 7)]);
+                    for (int j = 0; j < 16; ++j)
+                        x[j] = *reinterpret_cast<const float4 *>(&(j < 8 ? src0 : src1)[(j & 7) ^ (r & 7)]);
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    // bf16 16-byte chunk j = fp32 chunks 2j, 2j + 1
-                    const float4 a = x[2 * j], b = x[2 * j + 1];
-                    const __nv_bfloat162 b0 = __floats2bfloat162_rn(a.x, a.y), b1 = __floats2bfloat162_rn(a.z, a.w);
-                    const __nv_bfloat162 b2 = __floats2bfloat162_rn(b.x, b.y), b3 = __floats2bfloat162_rn(b.z, b.w);
-                    dst[j ^ (r & 7)] =
-                        make_uint4(*reinterpret_cast<const uint32_t *>(&b0), *reinterpret_cast<const uint32_t *>(&b1),
-                                   *reinterpret_cast<const uint32_t *>(&b2), *reinterpret_cast<const uint32_t *>(&b3));
+                    for (int j = 0; j < 8; ++j) {
+                        // bf16 16-byte chunk j = fp32 chunks 2j, 2j + 1
+                        const float4 a = x[2 * j], b = x[2 * j + 1];
+                        const __nv_bfloat162 b0 = __floats2bfloat162_rn(a.x, a.y), b1 = __floats2bfloat162_rn(a.z, a.w);
+                        const __nv_bfloat162 b2 = __floats2bfloat162_rn(b.x, b.y), b3 = __floats2bfloat162_rn(b.z, b.w);
+                        dst[j ^ (r & 7)] =
+                            make_uint4(*reinterpret_cast<const uint32_t *>(&b0), *reinterpret_cast<const uint32_t *>(&b1),
+                                       *reinterpret_cast<const uint32_t *>(&b2), *reinterpret_cast<const uint32_t *>(&b3));
+                    }
                 }
                 tc::fence_proxy_async_smem();
                 __syncwarp();
@@ -712,16 +717,17 @@ template <int BN, bool AF32>
 Ring ring_for(int rt, int chunks, size_t budget)
 {
     Ring r;
-    r.a_stride = (rt + 7) / 8 * 8 * 128;
-    const size_t per_stage = (AF32 ? 2 * 128 * 128 : r.a_stride) + BN * 128;  // fp32 A: raw stage, bf16 in place
+    r.a_stride = AF32 && rt > kShortRows ? 128 * 128 : (rt + 7) / 8 * 8 * 128;
+    const size_t a_bytes = AF32 ? 2 * r.a_stride : r.a_stride;  // fp32 A: raw stage, bf16 in place
+    const size_t per_stage = a_bytes + BN * 128;
     int ns = static_cast<int>(budget / per_stage);
     if (ns > kStages) ns = kStages;
     if (ns > chunks) ns = chunks;
     r.stages = ns < 1 ? 1 : ns;
     r.bytes = r.stages * per_stage;
     // the last stage's MMA reads a full 128-row window from its base
-    const size_t window = static_cast<size_t>(r.stages - 1) * r.a_stride + 128 * 128;
-    if (!AF32 && r.bytes < window) r.bytes = window;
+    const size_t window = (AF32 ? static_cast<size_t>(r.stages) * BN * 128 : 0) + (r.stages - 1) * a_bytes + 128 * 128;
+    if (r.bytes < window) r.bytes = window;
     return r;
 }
 
@@ -745,6 +751,15 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     // re-reading its (small) weight tile from L2
     if (nk < 8)
         while (tiles_for(rblk) < 64 && rblk > 1 && rblk * p.hpg > 16) rblk = (rblk + 1) / 2;
+    // fp32 A, more tiles than SMs (W_UV of a large batch): two CTAs share an SM,
+    // in tiles as short as still leave one wave.  640 rows of 32 heads, 12.2 us
+    // with 160 tiles of 128 rows and a ring of two chunks, 10.6 with 304 of 68
+    // and four.
+    const bool pairs = AF32 && tiles_for(rblk) > 152;
+    if (pairs) {
+        const int64_t n = 2 * 152 / (static_cast<int64_t>(ntiles) * p.G), blocks = p.M / p.hpg;
+        if (n * rblk >= blocks) rblk = static_cast<int>((blocks + n - 1) / n);
+    }
     CUtensorMap ma, mb;
     if (!encode_a(p, rblk, AF32, &ma)) return cudaErrorInvalidValue;
     if (NMAJ) {  // [G K rows][N columns], 64 x 64 boxes
@@ -766,11 +781,8 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     // behind it (at most 66 KB each).  A short tile's ring leaves room for a
     // second CTA.
     const size_t part = ks > 1 ? static_cast<size_t>(BN) * recv_rows(rt) * 4 : 0;
-    const size_t room = ks > 1 && rt <= 64 && !AF32 ? 111 * 1024 : kRingBytes;
+    const size_t room = pairs || (ks > 1 && rt <= 64 && !AF32) ? 111 * 1024 : kRingBytes;
     size_t budget = room - part;
-    // an fp32-A grid just past one CTA per SM (W_UV of a large batch):
-    // two stages, so that two CTAs share an SM and the grid runs in one wave
-    if (AF32 && ks == 1 && tiles > 152 && tiles <= 2 * 152) budget = 2 * (2 * 128 * 128 + BN * 128);
     const Ring ring = ring_for<BN, AF32>(rt, (nk + ks - 1) / ks, budget);
     GroupGemm q = p;
     q.stages = ring.stages;
@@ -780,13 +792,14 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     q.recv_off = static_cast<int>(ring.bytes > part ? ring.bytes : part);
     size_t smem = 1024 + (ks > 1 ? q.recv_off + part : ring.bytes);
     if (smem < 1024 + kDrainBytes) smem = 1024 + kDrainBytes;  // the results' staging
-    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, NMAJ, AF32, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smem));
+    const auto kernel = AF32 && rt <= kShortRows ? gemm_tc_kernel<BN, NMAJ, AF32, false, AF32>
+                                                 : gemm_tc_kernel<BN, NMAJ, AF32, false, false>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    const int threads = AF32 && ks == 1 && q.stages > 2 ? kConvThreads : kGemmThreads;
+    const int threads = AF32 && ks == 1 && !pairs ? kConvThreads : kGemmThreads;
     dim3 grid(mtiles * ks, ntiles, p.G);
     ProjEpi none{};
-    return launch_dependent(gemm_tc_kernel<BN, NMAJ, AF32, false>, grid, dim3(threads), smem, st, ks, q, ma, mb,
+    return launch_dependent(kernel, grid, dim3(threads), smem, st, ks, q, ma, mb,
                             mb, mb, rope ? *rope : none);
 }
 
@@ -846,11 +859,11 @@ cudaError_t launch_proj(const mla_dims &d, const CacheView &c, int batch, int n_
     p.rblk = rblk;
     p.ksplit = 1;
     if (smem < 1024 + kDrainBytes) smem = 1024 + kDrainBytes;  // the results' staging
-    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, false, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, false, false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     dim3 grid((p.M + rblk - 1) / rblk, tiles, 1);
-    return launch_dependent(gemm_tc_kernel<BN, false, false, true>, grid, dim3(kGemmThreads), smem, st, 1, p, ma, m0,
+    return launch_dependent(gemm_tc_kernel<BN, false, false, true, false>, grid, dim3(kGemmThreads), smem, st, 1, p, ma, m0,
                             m1, m2, pe);
 }
 
@@ -881,11 +894,7 @@ cudaError_t launch_group_gemm(const GroupGemm &p, cudaStream_t st)
     // column tile: 64 for narrow outputs and for few rows (more CTAs stream the
     // weight), else 128 -- or, of a bf16 A, what costs a CTA less
     const bool narrow = p.N <= 64 || p.M <= 32 || (!p.a_f32 && tile_cost(p, 64) < tile_cost(p, 128));
-    if (p.a_f32) {
-        if (p.b_nmajor) return narrow ? launch_tc<64, true, true>(p, st) : launch_tc<128, true, true>(p, st);
-        return narrow ? launch_tc<64, false, true>(p, st) : launch_tc<128, false, true>(p, st);
-    }
-    if (p.b_nmajor) return narrow ? launch_tc<64, true, false>(p, st) : launch_tc<128, true, false>(p, st);
+    if (p.a_f32) return narrow ? launch_tc<64, false, true>(p, st) : launch_tc<128, false, true>(p, st);
     return narrow ? launch_tc<64, false, false>(p, st) : launch_tc<128, false, false>(p, st);
 }
 

@@ -93,8 +93,8 @@ cudaError_t launch_out_proj(const mla_dims &d, int batch, int q_len, const float
 // Grouped GEMM of the projections: for each group g < G and row m < M,
 // C[phys(g, m), n] = sum_k A[phys(g, m), k] B_g(n, k) (bf16 result), with
 // phys(g, m) = (m / hpg) * blk + g * hpg + m % hpg.  A is fp32 or bf16 with
-// row stride lda; B_g(n, k) = B[g N K + n K + k] (K-major) or B[g K N + k N + n]
-// (N-major), bf16.  K and N are multiples of 8; A, B and C 16-byte aligned;
+// row stride lda; B_g(n, k) = B[g N K + n K + k] (K-major), of the absorption
+// B[g K N + k N + n] (N-major), bf16.  K and N are multiples of 8; A, B and C 16-byte aligned;
 // hpg <= 128 divides M.
 struct GroupGemm {
     int M, N, K, G;
@@ -103,7 +103,6 @@ struct GroupGemm {
     int a_f32;
     int64_t lda;
     const void *B;
-    int b_nmajor;
     void *C;
     int64_t ldc;
     unsigned *status;

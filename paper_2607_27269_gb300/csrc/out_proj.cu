@@ -22,7 +22,6 @@ cudaError_t launch_out_proj(const mla_dims &d, int batch, int q_len, const float
     p.a_f32 = 1;
     p.lda = d.rank;
     p.B = w_uv;  // [G][d_v][rank]: K-major
-    p.b_nmajor = 0;
     p.C = o;
     p.ldc = d.d_v;
     p.status = status;
@@ -40,7 +39,6 @@ cudaError_t launch_out_proj(const mla_dims &d, int batch, int q_len, const float
     q.a_f32 = 0;
     q.lda = H * d.d_v;
     q.B = w_o;  // [hidden][H d_v]: K-major
-    q.b_nmajor = 0;
     q.C = out;
     q.ldc = d.hidden;
     q.status = status;

@@ -33,6 +33,7 @@ pytestmark = pytest.mark.gpu
     (384, 32, 8, 512, 64, 2044),  # three tiles, 64 columns wide, unsplit
     (300, 8, 4, 256, 128, 516),   # unsplit, rows of C eight-byte aligned
     (700, 16, 4, 192, 40, 1024),  # 40-wide heads, three chunks of rank
+    (640, 32, 8, 512, 64, 264),   # more tiles of o_lat than SMs: 68 rows each, two CTAs an SM
     (96, 16, 4, 512, 128, 512),   # 128-wide heads, a ring of four stages under eight chunks
 ])
 def test_out_proj_tiles(rows, heads, groups, rank, d_v, hidden):
