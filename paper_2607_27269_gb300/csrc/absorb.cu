@@ -92,11 +92,6 @@ __device__ __forceinline__ void tma_store_5d(const CUtensorMap *map, uint32_t sr
                  : "memory");
 }
 
-__device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
-// every committed store has finished reading shared memory / has completed
-__device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-__device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
-
 __device__ __forceinline__ void named_bar_sync(int id, int threads)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
@@ -326,7 +321,7 @@ __global__ void __launch_bounds__(kAbThreads) absorb_kernel(const __grid_constan
             tc::fence_after_sync();
             int g, mt, nh;
             item_of(j, &g, &mt, &nh);
-            if (issuer) bulk_wait_read0();  // the previous item's store has left the staging buffer
+            if (issuer) tc::bulk_wait_read0();  // the previous item's store has left the staging buffer
             named_bar_sync(1, kAbEpiThreads);
             const uint32_t t_buf = t_lane + static_cast<uint32_t>(buf * a.ni);
 #pragma unroll 1
@@ -352,10 +347,10 @@ __global__ void __launch_bounds__(kAbThreads) absorb_kernel(const __grid_constan
             named_bar_sync(1, kAbEpiThreads);
             if (issuer && ok) {
                 tma_store_5d(&map_c, smem_u32(stage), 0, 0, g, mt * a.R, nh * nblk);
-                bulk_commit();
+                tc::bulk_commit();
             }
         }
-        if (issuer) bulk_wait0();
+        if (issuer) tc::bulk_wait0();
     }
 
     tc::fence_before_sync();

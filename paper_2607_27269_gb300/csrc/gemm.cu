@@ -54,6 +54,18 @@ struct ProjEpi {
     int q_len;
 };
 
+// eight fp32 bit patterns -> eight bf16 (round to nearest even)
+__device__ __forceinline__ uint4 pack8_bf16(const uint32_t *v)
+{
+    uint32_t w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
+        w[e] = *reinterpret_cast<const uint32_t *>(&b);
+    }
+    return make_uint4(w[0], w[1], w[2], w[3]);
+}
+
 // The bf16 results of a warp's 32 tile rows x BN columns, from TMEM to memory:
 // 64 columns at a time go through a staging block (32 rows of 144 bytes: both
 // sides free of bank conflicts), so that eight lanes store 128 contiguous bytes
@@ -88,16 +100,8 @@ __device__ __forceinline__ void drain_tile(uint32_t t_lane, unsigned char *stage
         tc::wait_ld();
         __syncwarp();  // the block before has been read
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-            uint32_t w[4];
-#pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int c = 8 * (k & 1) + 2 * e;
-                const __nv_bfloat162 b = __floats2bfloat162_rn(__uint_as_float(v[k >> 1][c]), __uint_as_float(v[k >> 1][c + 1]));
-                w[e] = *reinterpret_cast<const uint32_t *>(&b);
-            }
-            *reinterpret_cast<uint4 *>(stage + lane * kDrainRow + 16 * k) = make_uint4(w[0], w[1], w[2], w[3]);
-        }
+        for (int k = 0; k < 8; ++k)
+            *reinterpret_cast<uint4 *>(stage + lane * kDrainRow + 16 * k) = pack8_bf16(&v[k >> 1][8 * (k & 1)]);
         __syncwarp();
         const auto row = store(j + 8 * (lane & 7));
 #pragma unroll
@@ -105,6 +109,41 @@ __device__ __forceinline__ void drain_tile(uint32_t t_lane, unsigned char *stage
             const int r = 4 * rr + (lane >> 3);
             row(r, *reinterpret_cast<const uint4 *>(stage + r * kDrainRow + 16 * (lane & 7)));
         }
+    }
+}
+
+// The same by TMA stores: the tile's RT rows x 64 columns at a time, staged in
+// the 128-byte swizzle as the box that store(j) sends (called by one thread).
+// Plain stores leave an SM at 30 bytes a clock, TMA stores at 88 (192 KB from
+// each of 152 SMs: 6700 and 2200 cycles).  Called by the four epilogue warps,
+// also by one whose accumulator never came (good false): it keeps to the barriers.
+// W_UV + W_O of 14 heads, 64 rows, 7.5 -> 6.9 us, of 32 heads and 640 rows 19.8 ->
+// 18.6; not for the projection, whose queries are boxes too (13.0 -> 13.3 us).
+template <int BN, class Store>
+__device__ __forceinline__ void drain_tile_tma(uint32_t t_lane, unsigned char *stage, int i, int RT, bool good, Store store)
+{
+#pragma unroll 1
+    for (int j = 0; j < BN; j += 64) {
+        unsigned char *row = stage + j * 256 + i * 128;
+        if (good) {
+            uint32_t v[4][16];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) tc::ld_32x32b_x16(t_lane + j + 16 * u, v[u]);
+            tc::wait_ld();
+            if (i < RT) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k)
+                    *reinterpret_cast<uint4 *>(row + ((k ^ (i & 7)) << 4)) = pack8_bf16(&v[k >> 1][8 * (k & 1)]);
+            }
+            tc::fence_proxy_async_smem();
+        }
+        asm volatile("bar.sync 1, 128;" ::: "memory");
+        if (threadIdx.x == 64 && good) store(j, smem_u32(stage + j * 256));
+        __syncwarp();
+    }
+    if (threadIdx.x == 64) {
+        tc::bulk_commit();
+        tc::bulk_wait0();
     }
 }
 
@@ -239,17 +278,28 @@ struct __align__(8) GemmBars {
     uint64_t full[kStages], raw_full[kStages], conv_done[kStages], empty[kStages], done, recv;
 };
 
+// A, the weight and C; of the projection, the weights of its three column regions.
+template <bool PROJ>
+struct GemmMaps {
+    CUtensorMap a, b, c;
+};
+template <>
+struct GemmMaps<true> {
+    CUtensorMap a, b, b2, b3;
+};
+
 // BN: columns per CTA.  NMAJ: the weight is N-major.  AF32: A is fp32.
-// PROJ: the projection (K-major weights map_b, map_b2, map_b3 by column region).
+// PROJ: the projection (K-major weights b, b2, b3 by column region).
 // SHORT: an fp32 A in tiles of at most kShortRows rows, whose stages hold just
 // those (W_UV + W_O of 14 heads, one row 7.1 -> 6.6 us, 64 rows 8.0 -> 7.5);
 // with taller tiles the fixed stage is 1 to 2 percent faster.
-template <int BN, bool NMAJ, bool AF32, bool PROJ, bool SHORT>
-__global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_kernel(const __grid_constant__ GroupGemm p,
-                                                               const __grid_constant__ CUtensorMap map_a,
-                                                               const __grid_constant__ CUtensorMap map_b,
-                                                               const __grid_constant__ CUtensorMap map_b2,
-                                                               const __grid_constant__ CUtensorMap map_b3,
+// SPLIT: K split over a cluster; a kernel holds one of the two ways out.
+// (Two CTAs an SM stated, or the compiler takes 64 registers and spills in the
+// split kernels: 24 heads, 64 rows 12.6 us instead of 11.7.  The projection is
+// one CTA an SM and was slower with either bound: 160 rows 9.7 -> 10.2.)
+template <int BN, bool NMAJ, bool AF32, bool PROJ, bool SHORT, bool SPLIT>
+__global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 : 2) gemm_tc_kernel(const __grid_constant__ GroupGemm p,
+                                                               const __grid_constant__ GemmMaps<PROJ> maps,
                                                                const __grid_constant__ ProjEpi pe)
 {
     static_assert(!PROJ || (!NMAJ && !AF32), "the projection reads bf16 h and K-major weights");
@@ -262,7 +312,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
     unsigned char *smem = reinterpret_cast<unsigned char *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                                             ~static_cast<uintptr_t>(1023));
     const int nk = (p.K + 63) / 64;
-    const int ks = PROJ ? 1 : p.ksplit;                  // CTAs of the cluster sharing the K range
+    const int ks = SPLIT ? p.ksplit : 1;                // CTAs of the cluster sharing the K range
     const int kz = blockIdx.x % ks;                      // this CTA's share: chunks [c_begin, c_end)
     const int c_begin = kz * nk / ks, nkl = (kz + 1) * nk / ks - c_begin;
     const int NS = p.stages;                             // ring stages (<= kStages)
@@ -297,7 +347,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
         mbar_init(&bars.recv, 1);
         fail = 0;
         tc::fence_barrier_init();
-        if (!PROJ && ks > 1)  // the slabs of the other CTAs
+        if (SPLIT)  // the slabs of the other CTAs
             tc::mbar_arrive_expect_tx(smem_u32(&bars.recv), static_cast<uint32_t>((ks - 1) * (BN / ks) * recv_rows(RT) * 4));
     }
     if (warp == 1) {
@@ -309,7 +359,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
     tc::fence_after_sync();
     // a peer's shared memory is written only once its CTA has started: arrive
     // now, wait before the first such write
-    if (!PROJ && ks > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+    if (SPLIT) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
     // the activations come from the previous launch; with early_weights the
     // producer sends for the first weight tiles before it waits
     const bool early = !PROJ && p.early_weights && warp == 0;
@@ -329,17 +379,17 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
         // issues: with a lone lane and a division per chunk this loop took
         // 0.45 us a chunk and was the kernel's pace -- W_O of 640 rows 15 us
         // for 32 chunks, the projection of 640 rows 18.5)
-        const CUtensorMap *mb = &map_b;
+        const CUtensorMap *mb = &maps.b;
         int brow = g * p.N + n0;
         uint32_t bbytes = kBBytes;
-        if (PROJ) {
+        if constexpr (PROJ) {
             const int ty = blockIdx.y, region = ty < pe.tiles_lat ? 0 : ty == pe.tiles_lat ? 1 : 2;
-            mb = region == 0 ? &map_b : region == 1 ? &map_b2 : &map_b3;
+            mb = region == 0 ? &maps.b : region == 1 ? &maps.b2 : &maps.b3;
             brow = region == 0 ? n0 : region == 1 ? 0 : (ty - pe.tiles_lat - 1) * BN;
             bbytes = pe.box_bytes[region];
         }
         tc::prefetch_tensormap(mb);
-        tc::prefetch_tensormap(&map_a);
+        tc::prefetch_tensormap(&maps.a);
         auto load_b = [&](int c, int s) {
             const uint32_t fb = smem_u32(&bars.full[s]), dst = smem_u32(sb + s * kBBytes);
             tc::mbar_arrive_expect_tx_elect(fb, bbytes + (AF32 ? 0u : a_bytes));
@@ -347,7 +397,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
                 // rows = K of group g, columns = N: one 64 x 64 box per 64 columns
 #pragma unroll
                 for (int j = 0; j < BN / 64; ++j)
-                    tc::tma_load_2d_elect(dst + j * 64 * 128, &map_b, n0 + 64 * j, g * p.K + 64 * c, fb);
+                    tc::tma_load_2d_elect(dst + j * 64 * 128, &maps.b, n0 + 64 * j, g * p.K + 64 * c, fb);
             } else {
                 tc::tma_load_2d_elect(dst, mb, 64 * c, brow, fb);
             }
@@ -356,10 +406,10 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
             if (AF32) {
                 const uint32_t rb = smem_u32(&bars.raw_full[s]), rdst = smem_u32(sr + s * raw_bytes);
                 tc::mbar_arrive_expect_tx_elect(rb, 2 * a_bytes);
-                tc::tma_load_4d_elect(rdst, &map_a, 64 * c, 0, g, mt * R, rb);
-                tc::tma_load_4d_elect(rdst + raw_box, &map_a, 64 * c + 32, 0, g, mt * R, rb);
+                tc::tma_load_4d_elect(rdst, &maps.a, 64 * c, 0, g, mt * R, rb);
+                tc::tma_load_4d_elect(rdst + raw_box, &maps.a, 64 * c + 32, 0, g, mt * R, rb);
             } else {
-                tc::tma_load_4d_elect(smem_u32(sa + s * AS), &map_a, 64 * c, 0, g, mt * R, smem_u32(&bars.full[s]));
+                tc::tma_load_4d_elect(smem_u32(sa + s * AS), &maps.a, 64 * c, 0, g, mt * R, smem_u32(&bars.full[s]));
             }
         };
         const int head = nkl < NS ? nkl : NS;  // the ring's first round
@@ -496,20 +546,27 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
         }
         // ---- epilogue: warp w reads TMEM lanes 32 (w % 4) .. + 31
         const bool ok = epi && mbar_wait_warp(smem_u32(&bars.done), 0, lim);
-        if (!ok) {
-            if (epi && lane == 0) bail();
-        } else if (!fail) {
-            tc::fence_after_sync();
-            const int q = warp & 3;
-            const int i = q * 32 + lane;  // tile row
-            const int me = m0 + i;
-            const uint32_t t_lane = tmem + (static_cast<uint32_t>(q * 32) << 16);
+        if (epi && !ok && lane == 0) bail();
+        const bool good = ok && !fail;
+        const int q = warp & 3;
+        const int i = q * 32 + lane;  // tile row
+        const int me = m0 + i;
+        const uint32_t t_lane = tmem + (static_cast<uint32_t>(q * 32) << 16);
+        tc::fence_after_sync();
+        if constexpr (SPLIT) {
+            ep_ok = good;  // the partial leaves below
+        } else if (!PROJ && p.tma_out) {
+            if constexpr (!PROJ) {
+                if (epi)
+                    drain_tile_tma<BN>(t_lane, smem, i, RT, good, [&](int j, uint32_t src) {
+                        if (n0 + j < p.N) tc::tma_store_4d(&maps.c, src, n0 + j, 0, g, mt * R);
+                    });
+            }
+        } else if (good) {
             unsigned char *stage = smem + q * kDrainWarp;  // in the ring: its tiles have been read
             if (PROJ) {
                 const int rows = min(RT, p.M - m0) - q * 32;
                 proj_epilogue<BN>(p, pe, t_lane, stage, lane, me, rows);
-            } else if (ks > 1) {
-                ep_ok = true;  // the partial is pushed once the whole cluster is past its MMAs
             } else {
                 const bool vec = p.ldc % 8 == 0;  // 16-byte stores
                 uint16_t *crow = i < RT && me < p.M ? static_cast<uint16_t *>(p.C) + phys_row(p, g, me) * p.ldc : nullptr;
@@ -531,14 +588,14 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
             }
         }
     }
-    if (!PROJ && ks > 1) {
+    if constexpr (SPLIT) {
         // (1) the CTA's partial into its ring (its own MMAs are done), a slab
         // [four columns][row] for every owner: CTA o owns columns [o cw, (o + 1)
         // cw); (2) one bulk copy a peer takes its slab there, behind the peer's
-        // ring, and completes on the peer's barrier; (3) each owner sums its slice in rank
-        // order (four columns per step) and stores the bf16 result.  Remote
-        // stores of the same 30 KB, 512 bytes a warp, and a cluster barrier took
-        // 2700 cycles where the copies take 1900.
+        // ring, and completes on the peer's barrier; (3) each owner sums its
+        // slice in rank order (four columns per step) and stores the bf16
+        // result.  Remote stores of the same 30 KB, 512 bytes a warp, and a
+        // cluster barrier took 2700 cycles where the copies take 1900.
         const int cw = BN / ks, RP = recv_rows(RT);
         asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA has started
         if (ep_ok && !fail) {
@@ -546,18 +603,18 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads) gemm_tc_ke
             const int q = warp & 3, i = q * 32 + lane;
             const uint32_t t_lane = tmem + (static_cast<uint32_t>(q * 32) << 16);
 #pragma unroll 1
-            for (int j = 0; j < BN; j += 64) {
-                uint32_t v[4][16];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) tc::ld_32x32b_x16(t_lane + j + 16 * u, v[u]);
+            for (int j = 0; j < BN; j += 32) {
+                uint32_t v[2][16];
+                tc::ld_32x32b_x16(t_lane + j, v[0]);
+                tc::ld_32x32b_x16(t_lane + j + 16, v[1]);
                 tc::wait_ld();
                 if (i < RT) {  // (the slabs of the owners follow one another: column c at group c / 4)
-                    float4 *dst = reinterpret_cast<float4 *>(smem) + j / 4 * RP + i;
+                    uint4 *dst = reinterpret_cast<uint4 *>(smem) + j / 4 * RP + i;
 #pragma unroll
-                    for (int e = 0; e < 16; ++e)
-                        dst[e * RP] = make_float4(__uint_as_float(v[e / 4][4 * (e % 4)]), __uint_as_float(v[e / 4][4 * (e % 4) + 1]),
-                                                  __uint_as_float(v[e / 4][4 * (e % 4) + 2]),
-                                                  __uint_as_float(v[e / 4][4 * (e % 4) + 3]));
+                    for (int e = 0; e < 8; ++e) {
+                        const uint32_t *x = &v[e / 4][4 * (e % 4)];
+                        dst[e * RP] = make_uint4(x[0], x[1], x[2], x[3]);
+                    }
                 }
                 __syncwarp();
             }
@@ -645,6 +702,21 @@ bool encode_a(const GroupGemm &p, int rblk, bool f32, CUtensorMap *ma)
     return g_encode_gemm(ma, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4,
                          const_cast<void *>(p.A), dims, strides, box, es4, CU_TENSOR_MAP_INTERLEAVE_NONE,
                          CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                         CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+// The results: C (column, head in group, group, row block) in boxes of 64 columns
+// x a tile's rows; only rows of whole 16 bytes.
+bool encode_c(const GroupGemm &p, int rblk, CUtensorMap *mc)
+{
+    if (p.ldc % 8) return false;
+    cuuint64_t dims[4] = {static_cast<cuuint64_t>(p.N), static_cast<cuuint64_t>(p.hpg), static_cast<cuuint64_t>(p.G),
+                          static_cast<cuuint64_t>(p.M / p.hpg)};
+    cuuint64_t strides[3] = {static_cast<cuuint64_t>(p.ldc) * 2, static_cast<cuuint64_t>(p.hpg) * p.ldc * 2,
+                             static_cast<cuuint64_t>(p.blk) * p.ldc * 2};
+    cuuint32_t box[4] = {64u, static_cast<cuuint32_t>(p.hpg), 1u, static_cast<cuuint32_t>(rblk)}, es4[4] = {1, 1, 1, 1};
+    return g_encode_gemm(mc, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, p.C, dims, strides, box, es4,
+                         CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                          CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -791,16 +863,22 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     q.ksplit = ks;
     q.recv_off = static_cast<int>(ring.bytes > part ? ring.bytes : part);
     size_t smem = 1024 + (ks > 1 ? q.recv_off + part : ring.bytes);
-    if (smem < 1024 + kDrainBytes) smem = 1024 + kDrainBytes;  // the results' staging
-    const auto kernel = AF32 && rt <= kShortRows ? gemm_tc_kernel<BN, NMAJ, AF32, false, AF32>
-                                                 : gemm_tc_kernel<BN, NMAJ, AF32, false, false>;
+    CUtensorMap mc = mb;
+    q.tma_out = encode_c(p, rblk, &mc);
+    const size_t stage = q.tma_out ? BN * 256 : kDrainBytes;  // the results' staging
+    if (smem < 1024 + stage) smem = 1024 + stage;
+    const bool is_short = AF32 && rt <= kShortRows;
+    const auto kernel = ks > 1 ? (is_short ? gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, true>
+                                           : gemm_tc_kernel<BN, NMAJ, AF32, false, false, true>)
+                               : (is_short ? gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, false>
+                                           : gemm_tc_kernel<BN, NMAJ, AF32, false, false, false>);
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     const int threads = AF32 && ks == 1 && !pairs ? kConvThreads : kGemmThreads;
     dim3 grid(mtiles * ks, ntiles, p.G);
     ProjEpi none{};
-    return launch_dependent(kernel, grid, dim3(threads), smem, st, ks, q, ma, mb,
-                            mb, mb, rope ? *rope : none);
+    return launch_dependent(kernel, grid, dim3(threads), smem, st, ks, q,
+                            GemmMaps<false>{ma, mb, mc}, rope ? *rope : none);
 }
 
 // The projection: h [M = batch n_new, hidden] against W^DKV (rank rows), W^KR
@@ -859,12 +937,12 @@ cudaError_t launch_proj(const mla_dims &d, const CacheView &c, int batch, int n_
     p.rblk = rblk;
     p.ksplit = 1;
     if (smem < 1024 + kDrainBytes) smem = 1024 + kDrainBytes;  // the results' staging
-    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, false, false, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, false, false, true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     dim3 grid((p.M + rblk - 1) / rblk, tiles, 1);
-    return launch_dependent(gemm_tc_kernel<BN, false, false, true, false>, grid, dim3(kGemmThreads), smem, st, 1, p, ma, m0,
-                            m1, m2, pe);
+    return launch_dependent(gemm_tc_kernel<BN, false, false, true, false, false>, grid, dim3(kGemmThreads), smem, st, 1, p,
+                            GemmMaps<true>{ma, m0, m1, m2}, pe);
 }
 
 }  // namespace

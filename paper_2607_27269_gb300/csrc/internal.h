@@ -112,6 +112,7 @@ struct GroupGemm {
     // behind a caller's kernel that lets its dependents launch early.
     int early_weights = 0;
     int stages, rblk, ksplit;  // set by the launcher
+    int tma_out;               // the results leave by TMA stores (set by the launcher)
     int a_stride;              // bytes between A ring stages (set by the launcher)
     int recv_off;              // split K: where the cluster's partials arrive, bytes from the ring's start
 };
