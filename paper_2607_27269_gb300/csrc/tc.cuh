@@ -68,17 +68,6 @@ __device__ __forceinline__ void fence_after_sync()
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 }
 
-// D[tmem] (+)= A[smem desc] * B[smem desc]^T, issued by one thread.
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
-                                         uint32_t accumulate)
-{
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
-        "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 // Warp-collective forms: the whole warp executes them converged and one
 // elected lane issues.  A lone lane running the issue loop pays a large
 // per-iteration cost for every branch; a converged warp does not.
@@ -144,13 +133,6 @@ __device__ __forceinline__ void commit_elect(uint32_t mbar)
         : "memory");
 }
 
-__device__ __forceinline__ void mbar_arrive_elect(uint32_t mbar)
-{
-    asm volatile(
-        "{\n .reg .pred e;\n elect.sync _|e, 0xffffffff;\n @e mbarrier.arrive.shared::cta.b64 _, [%0];\n}\n" ::"r"(mbar)
-        : "memory");
-}
-
 // Arrive once on the mbarrier when every MMA this thread issued so far has
 // completed (and its smem operands may be overwritten).
 __device__ __forceinline__ void commit(uint32_t mbar)
@@ -163,14 +145,7 @@ __device__ __forceinline__ void wait_ld() { asm volatile("tcgen05.wait::ld.sync.
 __device__ __forceinline__ void wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
 // 32 lanes x 32-bit: thread t of the warp reads lane (taddr.lane + t),
-// columns taddr.col .. +N-1.
-__device__ __forceinline__ void ld_32x32b_x8(uint32_t taddr, uint32_t (&r)[8])
-{
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-                 : "r"(taddr));
-}
-
+// columns taddr.col .. + 15.
 __device__ __forceinline__ void ld_32x32b_x16(uint32_t taddr, uint32_t (&r)[16])
 {
     asm volatile(
@@ -245,26 +220,6 @@ __device__ __forceinline__ void fence_proxy_async_smem()
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1,
-                                            uint32_t mbar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-            dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(mbar)
-        : "memory");
-}
-
-__device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1,
-                                            int32_t c2, uint32_t mbar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
-        "[%5];" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(mbar)
-        : "memory");
-}
-
 // L2 eviction policies for cache-hinted loads.
 __device__ __forceinline__ uint64_t policy_evict_last()
 {
@@ -278,16 +233,6 @@ __device__ __forceinline__ uint64_t policy_evict_first()
     uint64_t p;
     asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));
     return p;
-}
-
-__device__ __forceinline__ void tma_load_2d_hint(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1,
-                                                 uint32_t mbar, uint64_t policy)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, "
-        "%3}], [%4], %5;" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(mbar), "l"(policy)
-        : "memory");
 }
 
 __device__ __forceinline__ void tma_load_3d_hint(uint32_t dst, const CUtensorMap *map, int32_t c0, int32_t c1,
@@ -332,24 +277,6 @@ __device__ __forceinline__ void tma_load_3d_hint_elect(uint32_t dst, const CUten
         : "memory");
 }
 
-// One refill of a ring slot in one election: the bytes to expect on `mbar`, a
-// 3-d box at `dst`, a second one at `dst2` unless `one`, and (if `map_q`) a 2-d box at `dst_q`.
-__device__ __forceinline__ void tma_refill_elect(uint32_t mbar, uint32_t bytes, const CUtensorMap *map, int32_t c0, int32_t c1,
-                                                 uint32_t dst, int32_t blk, uint32_t dst2, int32_t blk2, uint32_t two,
-                                                 uint64_t policy)
-{
-    asm volatile(
-        "{\n .reg .pred e, f, t;\n elect.sync _|e, 0xffffffff;\n setp.ne.b32 t, %9, 0;\n and.pred f, e, t;\n"
-        " @e mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n"
-        " @e cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%5], [%2, {%3, "
-        "%4, %6}], [%0], %10;\n"
-        " @f cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%7], [%2, {%3, "
-        "%4, %8}], [%0], %10;\n}\n" ::"r"(mbar),
-        "r"(bytes), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(dst), "r"(blk), "r"(dst2), "r"(blk2),
-        "r"(two), "l"(policy)
-        : "memory");
-}
-
 // The same with a 2-d box (of another map) as the last load.
 __device__ __forceinline__ void tma_refill_q_elect(uint32_t mbar, uint32_t bytes, const CUtensorMap *map, int32_t c0,
                                                    int32_t c1, uint32_t dst, int32_t blk, uint32_t dst2, int32_t blk2,
@@ -389,20 +316,6 @@ __device__ __forceinline__ void tma_refill_pair_elect(uint32_t mbar, uint32_t by
         "%4, %8}], [%0], %10;\n}\n" ::"r"(mbar),
         "r"(bytes), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(dst), "r"(blk), "r"(dst + half), "r"(blk2),
         "r"(two), "l"(policy), "r"(dst + step), "r"(dst + step + half), "r"(c0 + 64)
-        : "memory");
-}
-
-// Bring a box (or two) into L2.
-__device__ __forceinline__ void prefetch_3d_elect(const CUtensorMap *map, int32_t c0, int32_t c1, int32_t blk, int32_t blk2,
-                                                  uint32_t boxes, uint64_t policy)
-{
-    asm volatile(
-        "{\n .reg .pred e, f, g;\n elect.sync _|e, 0xffffffff;\n setp.gt.and.u32 f, %5, 0, e;\n"
-        " setp.gt.and.u32 g, %5, 1, e;\n"
-        " @f cp.async.bulk.prefetch.tensor.3d.L2.global.L2::cache_hint [%0, {%1, %2, %3}], %6;\n"
-        " @g cp.async.bulk.prefetch.tensor.3d.L2.global.L2::cache_hint [%0, {%1, %2, %4}], %6;\n}\n" ::"l"(
-            reinterpret_cast<uint64_t>(map)),
-        "r"(c0), "r"(c1), "r"(blk), "r"(blk2), "r"(boxes), "l"(policy)
         : "memory");
 }
 
