@@ -270,7 +270,9 @@ mla_status mla_gqa_append(const mla_gqa_dims *dims, const mla_cache *cache, int3
                           const void *k_new, const void *v_new, const int32_t *start_pos, void *stream);
 
 /* Partial-buffer sizes and split count of mla_gqa_decode_attn (as
- * mla_workspace_size, over the batch*G units). */
+ * mla_workspace_size, over the batch*G units; num_splits 0: seven partitions
+ * per SM, shared by the row groups of a unit (32 query rows at head_dim 64, 24
+ * at 128), fewer while a partition would hold under four tiles). */
 mla_status mla_gqa_workspace_size(const mla_gqa_dims *dims, int32_t batch, int32_t q_len, int32_t max_kv_len,
                                   int32_t num_splits, size_t *o_part_bytes, size_t *lse_part_bytes,
                                   int32_t *num_splits_used);
