@@ -275,6 +275,13 @@ __host__ __device__ constexpr int recv_rows(int rt) { return (rt + 7) / 8 * 8 + 
 constexpr int kGemmThreads = 192, kConvThreads = 320;
 constexpr int kShortRows = 96;
 
+// The tile row whose accumulator lane `lane` of TMEM quarter q holds: with M = 64
+// the rows lie in the first 16 lanes of each quarter (the other lanes: none).
+__device__ __forceinline__ int tile_row(bool m64, int q, int lane)
+{
+    return !m64 ? q * 32 + lane : lane < 16 ? q * 16 + lane : 128;
+}
+
 struct __align__(8) GemmBars {
     uint64_t full[kStages], raw_full[kStages], conv_done[kStages], empty[kStages], done, recv;
 };
@@ -298,7 +305,10 @@ struct GemmMaps<true> {
 // (Two CTAs an SM stated, or the compiler takes 64 registers and spills in the
 // split kernels: 24 heads, 64 rows 12.6 us instead of 11.7.  The projection is
 // one CTA an SM and was slower with either bound: 160 rows 9.7 -> 10.2.)
-template <int BN, bool NMAJ, bool AF32, bool PROJ, bool SHORT, bool SPLIT>
+// M64: tiles of at most 64 rows take MMAs of M = 64, which read half the A rows
+// (8 rows of 24 heads, W_UV + W_O: 9.4 -> 8.6 us); a kernel of its own, because
+// the choice at run time cost the tall tiles 2 to 5 percent.
+template <int BN, bool NMAJ, bool AF32, bool PROJ, bool SHORT, bool SPLIT, bool M64>
 __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 : 2) gemm_tc_kernel(const __grid_constant__ GroupGemm p,
                                                                const __grid_constant__ GemmMaps<PROJ> maps,
                                                                const __grid_constant__ ProjEpi pe)
@@ -317,8 +327,8 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 :
     const int kz = blockIdx.x % ks;                      // this CTA's share: chunks [c_begin, c_end)
     const int c_begin = kz * nk / ks, nkl = (kz + 1) * nk / ks - c_begin;
     const int NS = p.stages;                             // ring stages (<= kStages)
-    // A stages sit a_stride apart: the tile's RT rows (rounded to 8).  The M = 128
-    // MMA still reads 128 rows from its stage base: the rows past RT come from
+    // A stages sit a_stride apart: the tile's RT rows (rounded to 8).  The MMA
+    // still reads 64 or 128 rows from its stage base: the rows past RT come from
     // the next stages or the B ring (inside the allocation), land in accumulator
     // rows >= RT and are never stored.
     // An fp32 A has no A stages of its own: each converter thread writes its
@@ -332,6 +342,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 :
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const bool epi = warp >= 2 && warp < 6;              // an epilogue warp
     const int R = p.rblk, RT = R * p.hpg;                // row blocks and rows per tile (<= 128)
+    constexpr bool m64 = M64;
     const int mt = blockIdx.x / ks, n0 = blockIdx.y * BN, g = blockIdx.z;
     const int m0 = mt * RT;
     const uint32_t a_bytes = static_cast<uint32_t>(RT) * 128;  // per 64-column (bf16) or 32-column (fp32) box
@@ -437,7 +448,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 :
         }
     } else if (warp == 1) {
         // ---- MMA issuer (converged warp, one elected lane issues)
-        const uint32_t idesc = tc::idesc_bf16_f32(128, BN, false, NMAJ);
+        const uint32_t idesc = tc::idesc_bf16_f32(m64 ? 64 : 128, BN, false, NMAJ);
         const uint64_t da = tc::smem_desc(0, 16, 1024, tc::kSwizzle128B);
         const uint64_t db = NMAJ ? tc::smem_desc(0, 64 * 128, 1024, tc::kSwizzle128B)
                                  : tc::smem_desc(0, 16, 1024, tc::kSwizzle128B);
@@ -550,8 +561,8 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 :
         if (epi && !ok && lane == 0) bail();
         const bool good = ok && !fail;
         const int q = warp & 3;
-        const int i = q * 32 + lane;  // tile row
-        const int me = m0 + i;
+        const int i = tile_row(m64, q, lane);
+        const int me = m0 + q * (m64 ? 16 : 32) + lane;
         const uint32_t t_lane = tmem + (static_cast<uint32_t>(q * 32) << 16);
         tc::fence_after_sync();
         if constexpr (SPLIT) {
@@ -566,7 +577,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 :
         } else if (good) {
             unsigned char *stage = smem + q * kDrainWarp;  // in the ring: its tiles have been read
             if (PROJ) {
-                const int rows = min(RT, p.M - m0) - q * 32;
+                const int rows = m64 ? min(16, min(RT, p.M - m0) - q * 16) : min(RT, p.M - m0) - q * 32;
                 proj_epilogue<BN>(p, pe, t_lane, stage, lane, me, rows);
             } else {
                 const bool vec = p.ldc % 8 == 0;  // 16-byte stores
@@ -601,7 +612,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 :
         asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA has started
         if (ep_ok && !fail) {
             tc::fence_after_sync();
-            const int q = warp & 3, i = q * 32 + lane;
+            const int q = warp & 3, i = tile_row(m64, q, lane);
             const uint32_t t_lane = tmem + (static_cast<uint32_t>(q * 32) << 16);
 #pragma unroll 1
             for (int j = 0; j < BN; j += 32) {
@@ -809,6 +820,14 @@ Ring ring_for(int rt, int chunks, size_t budget)
 // chunks, 13.6 with the five that fit.
 constexpr size_t kRingBytes = 224 * 1024;
 
+template <int BN, bool NMAJ, bool AF32, bool SPLIT>
+auto gemm_kernel(int rt)
+{
+    if (rt <= 64) return gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, true>;
+    if (AF32 && rt <= kShortRows) return gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, false>;
+    return gemm_tc_kernel<BN, NMAJ, AF32, false, false, SPLIT, false>;
+}
+
 template <int BN, bool NMAJ, bool AF32>
 cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope = nullptr)
 {
@@ -868,11 +887,7 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     q.tma_out = encode_c(p, rblk, &mc);
     const size_t stage = q.tma_out ? BN * 256 : kDrainBytes;  // the results' staging
     if (smem < 1024 + stage) smem = 1024 + stage;
-    const bool is_short = AF32 && rt <= kShortRows;
-    const auto kernel = ks > 1 ? (is_short ? gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, true>
-                                           : gemm_tc_kernel<BN, NMAJ, AF32, false, false, true>)
-                               : (is_short ? gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, false>
-                                           : gemm_tc_kernel<BN, NMAJ, AF32, false, false, false>);
+    const auto kernel = ks > 1 ? gemm_kernel<BN, NMAJ, AF32, true>(rt) : gemm_kernel<BN, NMAJ, AF32, false>(rt);
     e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     const int threads = AF32 && ks == 1 && !pairs ? kConvThreads : kGemmThreads;
@@ -938,11 +953,13 @@ cudaError_t launch_proj(const mla_dims &d, const CacheView &c, int batch, int n_
     p.rblk = rblk;
     p.ksplit = 1;
     if (smem < 1024 + kDrainBytes) smem = 1024 + kDrainBytes;  // the results' staging
-    e = cudaFuncSetAttribute(gemm_tc_kernel<BN, false, false, true, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(smem));
+    constexpr bool kShort = BN == 64;  // (few rows take 64 columns)
+    const auto kernel = kShort && rblk <= 64 ? gemm_tc_kernel<BN, false, false, true, false, false, kShort>
+                                             : gemm_tc_kernel<BN, false, false, true, false, false, false>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     dim3 grid((p.M + rblk - 1) / rblk, tiles, 1);
-    return launch_dependent(gemm_tc_kernel<BN, false, false, true, false, false>, grid, dim3(kGemmThreads), smem, st, 1, p,
+    return launch_dependent(kernel, grid, dim3(kGemmThreads), smem, st, 1, p,
                             GemmMaps<true>{ma, m0, m1, m2}, pe);
 }
 

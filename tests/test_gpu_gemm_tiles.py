@@ -28,6 +28,8 @@ pytestmark = pytest.mark.gpu
     (129, 32, 8, 512, 64, 2056),  # two tiles of 65 rows, split over a cluster, eight columns in the last tile
     (160, 32, 8, 512, 64, 1030),  # split; rows of C at odd multiples of four bytes
     (160, 4, 2, 128, 64, 1030),   # the same rows unsplit (K of four chunks)
+    (64, 4, 2, 128, 64, 1024),    # the tallest tile of 64-row products, unsplit
+    (17, 4, 2, 128, 64, 1030),    # the same products, rows of C at odd multiples of four bytes
     (13, 14, 2, 256, 64, 898),    # short tiles, split, rows of C at odd multiples of four bytes
     (200, 32, 8, 512, 64, 2048),  # two tiles of 100 rows, 128 columns wide, split
     (384, 32, 8, 512, 64, 2044),  # three tiles, 64 columns wide, unsplit
