@@ -274,6 +274,7 @@ __host__ __device__ constexpr int recv_rows(int rt) { return (rt + 7) / 8 * 8 + 
 // chunks a CTA: one row 7.9 -> 8.2) or two CTAs share an SM, one set remains.
 constexpr int kGemmThreads = 192, kConvThreads = 320;
 constexpr int kShortRows = 96;
+constexpr int kM64Rows = 64;  // the tallest tile that MMAs of M = 64 take
 
 // The tile row whose accumulator lane `lane` of TMEM quarter q holds: with M = 64
 // the rows lie in the first 16 lanes of each quarter (the other lanes: none).
@@ -792,13 +793,17 @@ int64_t tile_cost(const GroupGemm &p, int bn)
 // The ring for tiles of rt rows: as many stages as fit `budget` bytes, at most
 // kStages and the K chunks.  A bf16 A stage holds just the tile's rows (rounded
 // to 8), so that short tiles stream their weight with more chunks in flight.
+// An MMA reads mma_rows (64 or 128) rows from its stage's base, and the last
+// stage's rows past the tile may lie past the ring (an fp32 A's stages are its
+// end): the allocation covers them, and they count against the budget.  (They
+// once did not: 20 rows of 24 heads of 128 against W_O asked for 232704 bytes.)
 struct Ring {
     int stages, a_stride;
     size_t bytes;
 };
 
 template <int BN, bool AF32>
-Ring ring_for(int rt, int chunks, size_t budget)
+Ring ring_for(int rt, int mma_rows, int chunks, size_t budget)
 {
     Ring r;
     r.a_stride = AF32 && rt > kShortRows ? 128 * 128 : (rt + 7) / 8 * 8 * 128;
@@ -807,11 +812,14 @@ Ring ring_for(int rt, int chunks, size_t budget)
     int ns = static_cast<int>(budget / per_stage);
     if (ns > kStages) ns = kStages;
     if (ns > chunks) ns = chunks;
-    r.stages = ns < 1 ? 1 : ns;
-    r.bytes = r.stages * per_stage;
-    // the last stage's MMA reads a full 128-row window from its base
-    const size_t window = (AF32 ? static_cast<size_t>(r.stages) * BN * 128 : 0) + (r.stages - 1) * a_bytes + 128 * 128;
-    if (r.bytes < window) r.bytes = window;
+    if (ns < 1) ns = 1;
+    auto bytes = [&](int n) {
+        const size_t window = (AF32 ? static_cast<size_t>(n) * BN * 128 : 0) + (n - 1) * a_bytes + mma_rows * 128;
+        return n * per_stage > window ? n * per_stage : window;
+    };
+    while (ns > 1 && bytes(ns) > budget) --ns;
+    r.stages = ns;
+    r.bytes = bytes(ns);
     return r;
 }
 
@@ -823,7 +831,7 @@ constexpr size_t kRingBytes = 224 * 1024;
 template <int BN, bool NMAJ, bool AF32, bool SPLIT>
 auto gemm_kernel(int rt)
 {
-    if (rt <= 64) return gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, true>;
+    if (rt <= kM64Rows) return gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, true>;
     if (AF32 && rt <= kShortRows) return gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, false>;
     return gemm_tc_kernel<BN, NMAJ, AF32, false, false, SPLIT, false>;
 }
@@ -875,7 +883,7 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     const size_t part = ks > 1 ? static_cast<size_t>(BN) * recv_rows(rt) * 4 : 0;
     const size_t room = pairs || (ks > 1 && rt <= 64 && !AF32) ? 111 * 1024 : kRingBytes;
     size_t budget = room - part;
-    const Ring ring = ring_for<BN, AF32>(rt, (nk + ks - 1) / ks, budget);
+    const Ring ring = ring_for<BN, AF32>(rt, rt <= kM64Rows ? 64 : 128, (nk + ks - 1) / ks, budget);
     GroupGemm q = p;
     q.stages = ring.stages;
     q.a_stride = ring.a_stride;
@@ -946,7 +954,7 @@ cudaError_t launch_proj(const mla_dims &d, const CacheView &c, int batch, int n_
     }
     const int tiles = pe.tiles_lat + 1 + (nq + BN - 1) / BN;
     p.N = tiles * BN;
-    const Ring ring = ring_for<BN, false>(rblk, (p.K + 63) / 64, kRingBytes);
+    const Ring ring = ring_for<BN, false>(rblk, 128, (p.K + 63) / 64, kRingBytes);
     size_t smem = 1024 + ring.bytes;
     p.stages = ring.stages;
     p.a_stride = ring.a_stride;

@@ -16,7 +16,7 @@ import torch
 
 from paper_2607_27269_gb300 import abi
 from paper_2607_27269_gb300 import workloads as wl
-from tests.helpers import bf16_to_f64, bits
+from tests.helpers import bf16_to_f64, bits, oracle_step, rel_errors
 from tests.test_gpu_project import assert_one_rounding, check_projection, run_projection
 
 pytestmark = pytest.mark.gpu
@@ -37,6 +37,9 @@ pytestmark = pytest.mark.gpu
     (700, 16, 4, 192, 40, 1024),  # 40-wide heads, three chunks of rank
     (640, 32, 8, 512, 64, 264),   # more tiles of o_lat than SMs: 68 rows each, two CTAs an SM
     (96, 16, 4, 512, 128, 512),   # 128-wide heads, a ring of four stages under eight chunks
+    (41, 80, 80, 512, 128, 512),  # one head a group, 128 columns: the last stage's rows read past the ring
+    (48, 80, 80, 512, 128, 264),  # the tallest such tile
+    (45, 40, 40, 512, 256, 264),  # two column tiles a group
 ])
 def test_out_proj_tiles(rows, heads, groups, rank, d_v, hidden):
     g = torch.Generator().manual_seed(rows + hidden)
@@ -59,6 +62,37 @@ def test_out_proj_tiles(rows, heads, groups, rank, d_v, hidden):
     got = bits(out.cpu())
     assert_one_rounding(got[:rows, 0], a @ u.T, np.abs(a) @ np.abs(u).T, "out")
     assert (out[rows:] == 7.0).all()
+
+
+@pytest.mark.parametrize("rows", [1, 8, 17, 20, 24, 25, 32, 33, 65])
+@pytest.mark.parametrize("hidden,heads", [(3072, 24), (4096, 32), (5120, 40)])
+def test_gqa_out_proj_tiles(rows, hidden, heads):
+    """An fp32 activation as wide as the output against a few dozen rows: rings
+    of many short stages, K split and not; 17 to 32 rows leave the last stage's
+    products reading past the ring."""
+    g = torch.Generator().manual_seed(rows + hidden)
+    width = heads * 128
+    o = torch.randn(rows, 1, heads, 128, generator=g)
+    w_o = (torch.randn(hidden, width, generator=g) * width ** -0.5).bfloat16()
+    out = torch.full((rows + 1, 1, hidden), 7.0, dtype=torch.bfloat16, device="cuda")  # one guard row
+    abi.gqa_out_proj(abi.GqaDims(heads, 8, 128, 128 ** -0.5), o.cuda(), w_o.cuda(), out[:rows])
+    assert abi.check_status() == abi.MLA_OK
+    a, u = bf16_to_f64(bits(o.bfloat16())).reshape(rows, width), bf16_to_f64(bits(w_o))  # the GEMM reads o as bf16
+    assert_one_rounding(bits(out.cpu())[:rows, 0], a @ u.T, np.abs(a) @ np.abs(u).T, "out")
+    assert (out[rows:] == 7.0).all()
+
+
+@pytest.mark.parametrize("rows", [41, 48])
+def test_decode_step_many_single_head_groups(rows):
+    """The whole step where W_UV runs one head a group in tiles of 41 to 48 rows."""
+    s = wl.Shape("groups80", rows, 80, 80, 64, 32, 128, 512, 0, 1, 70, 200)
+    w = wl.make(s, seed=45)
+    dw = abi.to_device(w)
+    step = abi.DecodeStep(dw.dims, dw.cache, rows, 1, dw.max_kv_len)
+    step(dw.q_nope, dw.q_pe, dw.kv_len, dw.w_uk, dw.w_uv, None, c_new=dw.c_new, kr_new=dw.kr_new, start_pos=dw.start_pos)
+    assert abi.check_status() == abi.MLA_OK
+    mx, mean = rel_errors(bf16_to_f64(bits(step.o.cpu())), oracle_step(w)["o"])
+    assert mx <= 2e-2 and mean <= 5e-3, (mx, mean)  # the bars of the parity tests
 
 
 @pytest.mark.parametrize("name,batch,n_new,rank,heads,with_q", [
