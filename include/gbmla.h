@@ -272,7 +272,10 @@ mla_status mla_gqa_append(const mla_gqa_dims *dims, const mla_cache *cache, int3
 /* Partial-buffer sizes and split count of mla_gqa_decode_attn (as
  * mla_workspace_size, over the batch*G units; num_splits 0: seven partitions
  * per SM, shared by the row groups of a unit (32 query rows at head_dim 64, 24
- * at 128), fewer while a partition would hold under four tiles). */
+ * at 128), at most one per tile; when that leaves at most four tiles per
+ * partition, the fewest partitions that keep the same most tiles per
+ * partition).  Buffers of these sizes also serve every call with the same
+ * num_splits whose batch, q_len and max_kv_len are no larger. */
 mla_status mla_gqa_workspace_size(const mla_gqa_dims *dims, int32_t batch, int32_t q_len, int32_t max_kv_len,
                                   int32_t num_splits, size_t *o_part_bytes, size_t *lse_part_bytes,
                                   int32_t *num_splits_used);

@@ -434,17 +434,23 @@ mla_status gqa_as_mla(const mla_gqa_dims *g, mla_dims *d)
     return MLA_OK;
 }
 
+// The most partitions num_splits 0 picks: as many (warps) as the SMs hold at a
+// time, each shared by the row groups, and no more than there are tiles.
+int64_t gqa_most_splits(const mla_gqa_dims *g, int batch, int q_len, int max_kv_len, int sms)
+{
+    const int64_t s = static_cast<int64_t>(sms) * kGqaPartsPerSm /
+                      gqa_row_groups(q_len * (g->num_heads / g->num_kv_groups), g->head_dim);
+    const int64_t tiles = static_cast<int64_t>(batch) * g->num_kv_groups * ((max_kv_len + MLA_SPLIT_TILE - 1) / MLA_SPLIT_TILE);
+    return s < 1 || tiles < 1 ? 1 : s < tiles ? s : tiles;
+}
+
 int gqa_splits(const mla_gqa_dims *g, int batch, int q_len, int max_kv_len, int requested, int sms)
 {
     if (requested > 0) return requested;
-    // as many partitions (warps) as the SMs hold at a time, each shared by the row groups
-    int64_t s = static_cast<int64_t>(sms) * kGqaPartsPerSm /
-                gqa_row_groups(q_len * (g->num_heads / g->num_kv_groups), g->head_dim);
+    int64_t s = gqa_most_splits(g, batch, q_len, max_kv_len, sms);
     const int64_t tiles = static_cast<int64_t>(batch) * g->num_kv_groups * ((max_kv_len + MLA_SPLIT_TILE - 1) / MLA_SPLIT_TILE);
-    if (s > tiles) s = tiles;
-    if (s < 1) s = 1;
     const int64_t per = (tiles + s - 1) / s;  // short partitions: the fewest with the same most tiles each
-    if (per <= 4) s = (tiles + per - 1) / per;
+    if (per >= 1 && per <= 4) s = (tiles + per - 1) / per;
     return static_cast<int>(s);
 }
 }  // namespace
@@ -479,11 +485,19 @@ mla_status mla_gqa_workspace_size(const mla_gqa_dims *dims, int32_t batch, int32
     int sms = 0;
     if ((s = device_info(nullptr, &sms)) != MLA_OK) return s;
     const int S = gqa_splits(dims, batch, q_len, max_kv_len, num_splits, sms);
+    // The partition count may rise where an argument falls (fewer queries are
+    // fewer row groups, fewer tiles may not pair up): the sizes are the largest
+    // of all calls with no larger arguments.
     const size_t units = static_cast<size_t>(batch) * dims->num_kv_groups;
-    const size_t slots = units > 0 ? units + S - 1 : 0;
-    const size_t rows = static_cast<size_t>(q_len) * (dims->num_heads / dims->num_kv_groups);
-    if (o_part_bytes) *o_part_bytes = slots * rows * dims->head_dim * sizeof(float);
-    if (lse_part_bytes) *lse_part_bytes = slots * rows * sizeof(float);
+    const int hpg = dims->num_heads / dims->num_kv_groups;
+    size_t slot_rows = 0;
+    for (int q = 1; q <= q_len && units > 0; ++q) {
+        const size_t most = num_splits > 0 ? num_splits : gqa_most_splits(dims, batch, q, max_kv_len, sms);
+        const size_t n = (units + most - 1) * q * hpg;
+        if (n > slot_rows) slot_rows = n;
+    }
+    if (o_part_bytes) *o_part_bytes = slot_rows * dims->head_dim * sizeof(float);
+    if (lse_part_bytes) *lse_part_bytes = slot_rows * sizeof(float);
     if (num_splits_used) *num_splits_used = S;
     return MLA_OK;
 }

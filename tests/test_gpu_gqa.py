@@ -128,3 +128,46 @@ def test_gqa_row_counts_and_stage_tails(hpg, q_len, d, paged, style):
     _, ref = oracle_run(gw)
     assert_close(step.o.cpu().numpy(), ref["o"], "o")
     assert_close(step.lse.cpu().numpy(), ref["lse"], "lse")
+
+
+@pytest.mark.parametrize("heads,groups,d", [(64, 8, 64), (32, 8, 64), (40, 8, 128), (14, 2, 64)])
+@pytest.mark.parametrize("splits", [0, 5])
+def test_gqa_workspace_covers_smaller_calls(heads, groups, d, splits):
+    """Buffers sized once for the longest chunk, batch and cache hold every
+    smaller call's partials (units + S - 1 slots of q_len * H/G rows), although
+    its partition count may be the larger one."""
+    dims = abi.GqaDims(heads, groups, d, d ** -0.5)
+    for batch, q_len, kv in [(8, 5, 2048), (8, 16, 2200), (3, 16, 900), (61, 7, 4096)]:
+        if q_len * heads // groups > 128:
+            continue
+        o_bytes, lse_bytes, _ = abi.gqa_workspace_size(dims, batch, q_len, kv, splits)
+        for b in range(1, batch + 1, 1 + batch // 8):
+            for q in range(1, q_len + 1):
+                for t in range(q, kv + 1, 1 + kv // 50):
+                    s = abi.gqa_workspace_size(dims, b, q, t, splits)[2]
+                    rows = (b * groups + s - 1) * q * (heads // groups)
+                    assert rows * d * 4 <= o_bytes and rows * 4 <= lse_bytes, (b, q, t, s)
+
+
+def test_gqa_shorter_chunk_in_the_longest_chunks_buffers():
+    """8 heads a group, 64 units of up to 2048 tokens: four queries are one row
+    group and take more partitions than five, and twice as many slots.  With
+    num_splits 0 in buffers sized for five queries nothing past them is written
+    and the results are those of buffers of their own."""
+    B, G, d, cap = 8, 8, 64, 2048
+    g = torch.Generator(device="cuda").manual_seed(64)
+    k, v = (torch.randn(B * G, cap, d, generator=g, device="cuda").bfloat16() for _ in range(2))
+    q = torch.randn(B, 4, 8 * G, d, generator=g, device="cuda").bfloat16()
+    kv = torch.tensor([cap - 97 * b for b in range(B)], dtype=torch.int32, device="cuda")
+    dims, cache = abi.GqaDims(8 * G, G, d, d ** -0.5), abi.Cache(v, k, cap)
+    own = abi.GqaStep(dims, cache, B, 4, cap)
+    want = own(q, kv).clone()
+    o_bytes, lse_bytes, _ = abi.gqa_workspace_size(dims, B, 5, cap)
+    step = abi.GqaStep(dims, cache, B, 4, cap)
+    step.num_splits = 0
+    step.o_part = torch.full((o_bytes // 4 + (1 << 22),), 7.0, device="cuda")    # sized for five queries, and a guard
+    step.lse_part = torch.full((lse_bytes // 4 + (1 << 16),), 7.0, device="cuda")
+    step(q, kv)
+    assert abi.check_status() == abi.MLA_OK
+    assert torch.equal(step.o, want) and torch.equal(step.lse, own.lse)
+    assert (step.o_part[o_bytes // 4:] == 7.0).all() and (step.lse_part[lse_bytes // 4:] == 7.0).all()
