@@ -187,6 +187,13 @@ __global__ void __launch_bounds__(32 * kWarps, 1)
     // dependents only on completion); the queries and the partial buffers
     // belong to the previous launches: a warp waits before it reads queries
     griddep_launch_dependents();
+    // a length that cannot be served holds no tiles, here and in the combine
+    if (blockIdx.x == 0 && blockIdx.y == 0) {
+        for (int b = tid; b < a.batch; b += 32 * kWarps) {
+            const int kv = a.kv_len[b];
+            if (kv < a.q_len || kv > a.max_kv) record_status(a.status, kStatusBounds);
+        }
+    }
     // (the block-wide sums also order the barriers' set-up before their use)
     const int64_t T = block_tile_sum(a.kv_len, a.batch, a.q_len, a.max_kv, red64) * a.groups;
     const int part = warp * gridDim.x + blockIdx.x;  // spread over the SMs first

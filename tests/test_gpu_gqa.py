@@ -171,3 +171,24 @@ def test_gqa_shorter_chunk_in_the_longest_chunks_buffers():
     assert abi.check_status() == abi.MLA_OK
     assert torch.equal(step.o, want) and torch.equal(step.lse, own.lse)
     assert (step.o_part[o_bytes // 4:] == 7.0).all() and (step.lse_part[lse_bytes // 4:] == 7.0).all()
+
+
+@pytest.mark.parametrize("lens", [(200, 301, 150), (200, 2, 150), (301, 2, -5), (0, 0, 0)])
+def test_gqa_lengths_that_cannot_be_served_are_recorded(lens):
+    """A length above the stated maximum or below q_len: recorded, the unit
+    left out, the other units right; nothing but such lengths too."""
+    q_len, most = 3, 300
+    shape = wl.Shape("lens", len(lens), 8, 2, 64, 64, 64, 128, 0, q_len, most, most)
+    gw = wl.gqa(wl.make(shape, seed=65), seed=65)
+    dims, cache, step = devices(gw)
+    abi.gqa_append(dims, cache, gw.k_new.cuda(), gw.v_new.cuda(), gw.start_pos.cuda())
+    good = torch.tensor([n if q_len <= n <= most else q_len for n in lens], dtype=torch.int32, device="cuda")
+    step(gw.q.cuda(), good)
+    assert abi.check_status() == abi.MLA_OK
+    want = step.o.clone()
+    step(gw.q.cuda(), torch.tensor(lens, dtype=torch.int32, device="cuda"))
+    assert abi.check_status() == abi.MLA_ERR_DEVICE_BOUNDS
+    for b, n in enumerate(lens):
+        if q_len <= n <= most:
+            # another partition of the tiles: other roundings of the weights, as in the bars above
+            assert_close(step.o[b].cpu().numpy(), want[b].cpu().numpy(), f"o[{b}]")
