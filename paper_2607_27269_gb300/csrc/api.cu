@@ -21,20 +21,26 @@ unsigned *g_status_ptr[kMaxDevices];
 int g_sm_count[kMaxDevices];
 
 // Device address of this device's status word and its SM count, looked up
-// once per device with that device current.
+// once per device with that device current.  Each host thread looks the address
+// up once for itself: that gives a thread which has made no CUDA call yet its
+// context, without which no tensor map can be encoded (its first call would
+// fail as an invalid argument).
 mla_status device_info(unsigned **status, int *sms)
 {
+    thread_local uint64_t seen = 0;  // devices this thread has been here for
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return MLA_ERR_CUDA;
-    std::lock_guard<std::mutex> lock(g_mutex);
-    if (!g_status_ptr[dev]) {
+    if (!((seen >> dev) & 1u)) {
         void *p = nullptr;
         if (cudaGetSymbolAddress(&p, g_status_word) != cudaSuccess) return MLA_ERR_CUDA;
         int n = 0;
         if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return MLA_ERR_CUDA;
+        std::lock_guard<std::mutex> lock(g_mutex);
         g_status_ptr[dev] = static_cast<unsigned *>(p);
         g_sm_count[dev] = n;
+        seen |= uint64_t{1} << dev;
     }
+    std::lock_guard<std::mutex> lock(g_mutex);
     if (status) *status = g_status_ptr[dev];
     if (sms) *sms = g_sm_count[dev];
     return MLA_OK;
