@@ -471,11 +471,9 @@ cudaError_t launch_absorb_persistent(const mla_dims &d, int batch, int q_len, co
             return cudaErrorInvalidValue;
     }
     // ring stages (A 16 KB + B 32 KB each) and the output staging (ni / 64 blocks of 16 KB)
-    const size_t smem = 1024 + static_cast<size_t>(kAbStages) * (128 * 128 + kAbMaxN * 128) +
-                        static_cast<size_t>(a.ni / 64) * (128 * 128);
-    if ((e = cudaFuncSetAttribute(absorb_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(smem))) != cudaSuccess)
-        return e;
+    constexpr size_t kRing = 1024 + static_cast<size_t>(kAbStages) * (128 * 128 + kAbMaxN * 128);
+    const size_t smem = kRing + static_cast<size_t>(a.ni / 64) * (128 * 128);
+    if ((e = allow_smem<absorb_kernel>(kRing + kAbMaxN / 64 * (128 * 128))) != cudaSuccess) return e;
     const int grid = a.items < sms ? a.items : sms;
     return launch_dependent(absorb_kernel, dim3(grid), dim3(kAbThreads), smem, st, 1, a, ma, mb, mc);
 }

@@ -204,9 +204,9 @@ __global__ void __launch_bounds__(kThreads) attn_simt_kernel(AttnArgs a)
 cudaError_t launch_attn_simt(const AttnArgs &a, cudaStream_t st)
 {
     const int K = a.rank + a.d_rope;
-    const size_t smem = sizeof(float) * kRows * (K + 1) + sizeof(uint16_t) * kTok * (K + 2);
-    cudaError_t e = cudaFuncSetAttribute(attn_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
+    auto bytes = [](int k) { return sizeof(float) * kRows * (k + 1) + sizeof(uint16_t) * kTok * (k + 2); };
+    const size_t smem = bytes(K);
+    cudaError_t e = allow_smem<attn_simt_kernel>(bytes(512 + 64));  // the widest rank and d_rope
     if (e != cudaSuccess) return e;
     const int rows = a.q_len * a.num_heads;
     dim3 grid(a.num_splits, (rows + kRows - 1) / kRows);

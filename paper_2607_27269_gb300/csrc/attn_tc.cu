@@ -1201,9 +1201,8 @@ cudaError_t launch_cfg(const AttnArgs &a, int groups, cudaStream_t st)
     if (qk_slots < 2) return cudaErrorInvalidConfiguration;
     const size_t smem = static_cast<size_t>(fixed) + static_cast<size_t>(qk_slots) * slot_a +
                         static_cast<size_t>(pv_slots) * kChunkBytes + p_bytes;
-    if ((e = cudaFuncSetAttribute(attn_tc_kernel<N, SQ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(smem))) != cudaSuccess)
-        return e;
+    // (smem is whole KB, and so is the static part: its alignment is the dynamic part's)
+    if ((e = allow_smem<attn_tc_kernel<N, SQ>>((optin - static_bytes) & ~1023)) != cudaSuccess) return e;
     TcArgs t;
     t.batch = a.batch;
     t.q_len = a.q_len;

@@ -3,6 +3,8 @@
 
 #include <math.h>
 
+#include <atomic>
+#include <mutex>
 #include <utility>
 
 #include <cuda_bf16.h>
@@ -95,6 +97,29 @@ __device__ __forceinline__ void griddep_wait() { asm volatile("griddepcontrol.wa
 __device__ __forceinline__ void griddep_launch_dependents()
 {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Lets launches of Kernel ask for up to `most` bytes of dynamic shared memory.
+// The limit is one value per kernel and device, shared by all host threads, and
+// a launch that asks for more fails, as does one while the limit is being set.
+// So it is set once per device, before the first launch there, to what the
+// kernel's largest shape needs, whatever the launch at hand needs.
+template <auto Kernel>
+cudaError_t allow_smem(size_t most)
+{
+    constexpr int kDevices = 64;
+    static std::mutex m;
+    static std::atomic<bool> done[kDevices];
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev < 0 || dev >= kDevices) return cudaErrorInvalidDevice;
+    if (done[dev].load(std::memory_order_acquire)) return cudaSuccess;
+    std::lock_guard<std::mutex> lock(m);
+    if (done[dev].load(std::memory_order_relaxed)) return cudaSuccess;
+    e = cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most));
+    if (e == cudaSuccess) done[dev].store(true, std::memory_order_release);
+    return e;
 }
 
 // Launch `kernel` on `st` as a programmatic dependent of the stream's

@@ -828,12 +828,21 @@ Ring ring_for(int rt, int mma_rows, int chunks, size_t budget)
 // chunks, 13.6 with the five that fit.
 constexpr size_t kRingBytes = 224 * 1024;
 
-template <int BN, bool NMAJ, bool AF32, bool SPLIT>
-auto gemm_kernel(int rt)
+using GemmKernel = void (*)(GroupGemm, GemmMaps<false>, ProjEpi);
+
+template <auto Kernel, class K>
+cudaError_t take_kernel(K *kernel)
 {
-    if (rt <= kM64Rows) return gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, true>;
-    if (AF32 && rt <= kShortRows) return gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, false>;
-    return gemm_tc_kernel<BN, NMAJ, AF32, false, false, SPLIT, false>;
+    *kernel = Kernel;
+    return allow_smem<Kernel>(1024 + kRingBytes);
+}
+
+template <int BN, bool NMAJ, bool AF32, bool SPLIT>
+cudaError_t gemm_kernel(int rt, GemmKernel *kernel)
+{
+    if (rt <= kM64Rows) return take_kernel<gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, true>>(kernel);
+    if (AF32 && rt <= kShortRows) return take_kernel<gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, false>>(kernel);
+    return take_kernel<gemm_tc_kernel<BN, NMAJ, AF32, false, false, SPLIT, false>>(kernel);
 }
 
 template <int BN, bool NMAJ, bool AF32>
@@ -895,8 +904,8 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     q.tma_out = encode_c(p, rblk, &mc);
     const size_t stage = q.tma_out ? BN * 256 : kDrainBytes;  // the results' staging
     if (smem < 1024 + stage) smem = 1024 + stage;
-    const auto kernel = ks > 1 ? gemm_kernel<BN, NMAJ, AF32, true>(rt) : gemm_kernel<BN, NMAJ, AF32, false>(rt);
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    GemmKernel kernel;
+    e = ks > 1 ? gemm_kernel<BN, NMAJ, AF32, true>(rt, &kernel) : gemm_kernel<BN, NMAJ, AF32, false>(rt, &kernel);
     if (e != cudaSuccess) return e;
     const int threads = AF32 && ks == 1 && !pairs ? kConvThreads : kGemmThreads;
     dim3 grid(mtiles * ks, ntiles, p.G);
@@ -962,9 +971,9 @@ cudaError_t launch_proj(const mla_dims &d, const CacheView &c, int batch, int n_
     p.ksplit = 1;
     if (smem < 1024 + kDrainBytes) smem = 1024 + kDrainBytes;  // the results' staging
     constexpr bool kShort = BN == 64;  // (few rows take 64 columns)
-    const auto kernel = kShort && rblk <= 64 ? gemm_tc_kernel<BN, false, false, true, false, false, kShort>
-                                             : gemm_tc_kernel<BN, false, false, true, false, false, false>;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    void (*kernel)(GroupGemm, GemmMaps<true>, ProjEpi);
+    e = kShort && rblk <= 64 ? take_kernel<gemm_tc_kernel<BN, false, false, true, false, false, kShort>>(&kernel)
+                             : take_kernel<gemm_tc_kernel<BN, false, false, true, false, false, false>>(&kernel);
     if (e != cudaSuccess) return e;
     dim3 grid((p.M + rblk - 1) / rblk, tiles, 1);
     return launch_dependent(kernel, grid, dim3(kGemmThreads), smem, st, 1, p,

@@ -524,9 +524,7 @@ cudaError_t launch_dn(const GqaLaunch &g, int row_groups, cudaStream_t st)
     a.status = g.status;
     a.turns = rope_turns(D, g.rope_base);
     constexpr size_t smem = 1024 + static_cast<size_t>(kWarps) * kStages * kStageBytes;
-    if ((e = cudaFuncSetAttribute(gqa_attn_kernel<D, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  static_cast<int>(smem))) != cudaSuccess)
-        return e;
+    if ((e = allow_smem<gqa_attn_kernel<D, N>>(smem)) != cudaSuccess) return e;
     // the partitions over the SMs' blocks first, then over each block's warps
     const int per_group = (g.sms + row_groups - 1) / row_groups;
     int grid = g.num_splits < per_group ? g.num_splits : per_group;

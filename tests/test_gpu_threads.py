@@ -1,4 +1,7 @@
-"""Calls from host threads other than the main one."""
+"""Host threads that call the library at the same time, each on its own stream
+and with shapes of its own: a launch must not depend on what another thread
+sets for its launch of the same kernel (the shared memory a kernel may ask for
+is one value per kernel, not per launch)."""
 from __future__ import annotations
 
 import threading
@@ -108,3 +111,46 @@ def test_a_threads_first_call(make):
     assert abi.check_status() == abi.MLA_OK
     torch.cuda.synchronize()
     assert torch.equal(out, want)
+
+
+@pytest.mark.parametrize("small,large", [
+    (lambda: _out_proj(1, 64, 8, 1), lambda: _out_proj(64, 512, 32, 2)),
+    (lambda: _project(1, 64, 3), lambda: _project(64, 2048, 4)),
+    (lambda: _absorb(1, 128, 5), lambda: _absorb(2048, 512, 6)),
+], ids=["out_proj", "project", "absorb"])
+def test_threads_with_different_shapes(small, large, monkeypatch):
+    calls = [make() for _ in range(4) for make in (small, large)]
+    streams = [torch.cuda.Stream() for _ in calls]
+    raw = []  # each call's library function and arguments: a loop over them leaves the threads little time in Python
+
+    class Recorder:
+        def __getattr__(self, name):
+            return lambda *args: raw.append((getattr(library, name), args)) or abi.MLA_OK
+
+    library = abi.lib()
+    with monkeypatch.context() as m:
+        m.setattr(abi, "lib", Recorder)
+        for (call, _), stream in zip(calls, streams):
+            with torch.cuda.stream(stream):
+                call()
+    for fn, args in raw:
+        assert fn(*args) == abi.MLA_OK
+    torch.cuda.synchronize()
+    want = [out.clone() for _, out in calls]
+    bad = []
+    start = threading.Barrier(len(calls))
+
+    def work(fn, args):
+        start.wait()
+        bad.extend(code for code in (fn(*args) for _ in range(4000)) if code != abi.MLA_OK)
+
+    threads = [threading.Thread(target=work, args=r) for r in raw]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not bad, (len(bad), abi.status_name(bad[0]))
+    assert abi.check_status() == abi.MLA_OK
+    for (_, out), ref in zip(calls, want):
+        assert torch.equal(out, ref)
