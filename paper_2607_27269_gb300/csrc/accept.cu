@@ -485,7 +485,9 @@ cudaError_t launch_typed(int rows, int vocab, const void *draft, const void *tar
     constexpr double kAlone = 28e3, kPerSm = 33e3, kRowCost = 2.0;  // bytes per us, bytes per us, us
     double best = 0;
     int C = 0, n_cl = 0;
+    const int forced = tuning().accept_cluster;  // testing aid: 1 .. 8 CTAs a cluster
     for (int c = 1; c <= kMaxCluster; ++c) {
+        if (forced >= 1 && forced <= kMaxCluster && c != forced) continue;
         const int n = row_clusters<T>(c);
         if (n <= 0) continue;
         const int live = rows < n ? rows : n;

@@ -132,9 +132,9 @@ def test_acceptance_full_rows_sampled(name):
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("rows,vocab", [(2, 1), (3, 8), (2, 2049), (5, 4099), (700, 515), (61, 9001), (1200, 37)])
 def test_acceptance_masked_logits_and_cluster_sizes(rows, vocab, dtype):
-    """Rows and vocabularies that take clusters of one to eight CTAs, slices
-    with no vector at all, groups that end inside and several rows per cluster;
-    logits masked with -inf and with the type's lowest value (whole vectors of
+    """Few and many rows, clusters of one, two, seven and eight CTAs (the sizes
+    these shapes are given), slices with no vector at all, groups that end
+    inside and several rows per cluster; logits masked with -inf and with the type's lowest value (whole vectors of
     them, a thread's first ones included) weigh nothing.  Error: the sums are
     trees of fp32 exponentials, as above."""
     g = torch.Generator().manual_seed(57)
@@ -151,3 +151,26 @@ def test_acceptance_masked_logits_and_cluster_sizes(rows, vocab, dtype):
         d[rows - 1, : vocab // 2] += 60.0  # the base is raised late, and by much
         t[rows - 1, vocab // 2:] += 60.0
         check(d, t)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("cluster", range(1, 9))
+def test_acceptance_every_cluster_size(cluster, dtype, tuning):
+    """Each cluster size, also those that no shape above is given: three rows
+    and more a cluster (both sets of exchange slots are used again; up to 456
+    clusters run at a time), slices of unequal length, a tail past the last
+    whole vector, fewer vectors than CTAs, equal maxima in different slices (the
+    first wins), rows whose maximum every CTA but one has not seen."""
+    tuning(GBMLA_ACCEPT_CLUSTER=cluster)
+    g = torch.Generator().manual_seed(58)
+    rows, n = 3 * 456 + 5, 16 // torch.empty((), dtype=dtype).element_size()
+    for vocab in (3 * n + 1, 8 * n, 1003, 4099):
+        d = (torch.randn(rows, vocab, generator=g) * 2).to(dtype)
+        t = (torch.randn(rows, vocab, generator=g) * 2).to(dtype)
+        at = torch.randint(0, vocab, (rows, 2), generator=g)
+        r = torch.arange(rows)
+        d[r, at[:, 0]] = d[r, at[:, 1]] = 12.0
+        t[r[::2], at[::2, 1]] = 12.0
+        t[r[1::2], at[1::2, 0]] = 12.0
+        ref = check(d, t)
+        assert 0 < ref["greedy"].mean() < 1
