@@ -125,7 +125,7 @@ int resolve_splits(const mla_dims *d, int batch, int q_len, int max_kv_len, int 
     // attention + combine from 22.3 to 16.9 us).  Longer ones keep one per SM:
     // with ragged lengths the bound is loose and the idle SMs would cost more.
     const int64_t per = (max_tiles + s - 1) / s;
-    if (per <= 4) s = (max_tiles + per - 1) / per;
+    if (per >= 1 && per <= 4) s = (max_tiles + per - 1) / per;  // (0: an empty batch)
     return static_cast<int>(s);
 }
 

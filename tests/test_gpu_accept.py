@@ -132,7 +132,7 @@ def test_acceptance_full_rows_sampled(name):
 @pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
 @pytest.mark.parametrize("rows,vocab", [(2, 1), (3, 8), (2, 2049), (5, 4099), (700, 515), (61, 9001), (1200, 37)])
 def test_acceptance_masked_logits_and_cluster_sizes(rows, vocab, dtype):
-    """Few and many rows, clusters of one, two, seven and eight CTAs (the sizes
+    """Few and many rows, clusters of one, seven and eight CTAs (the sizes
     these shapes are given), slices with no vector at all, groups that end
     inside and several rows per cluster; logits masked with -inf and with the type's lowest value (whole vectors of
     them, a thread's first ones included) weigh nothing.  Error: the sums are

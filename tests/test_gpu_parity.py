@@ -357,6 +357,12 @@ def test_device_faults_are_reported_not_trapped():
     run_step(dw)
 
 
+def test_workspace_of_an_empty_batch():
+    """No tiles to share out: no bytes, one partition (not the quotient of a division by zero)."""
+    assert abi.workspace_size(abi.Dims(8, 2, 64, 64, 64, 128), 0, 1, 100) == (0, 0, 1)
+    assert abi.gqa_workspace_size(abi.GqaDims(8, 2, 64, 0.125), 0, 1, 100) == (0, 0, 1)
+
+
 def test_deterministic():
     w = wl.small("llama3b_long_b8_h24_r512_t16k_32k", seed=20)
     a = run_step(abi.to_device(w)).o_lat.cpu()
