@@ -192,3 +192,24 @@ def test_gqa_lengths_that_cannot_be_served_are_recorded(lens):
         if q_len <= n <= most:
             # another partition of the tiles: other roundings of the weights, as in the bars above
             assert_close(step.o[b].cpu().numpy(), want[b].cpu().numpy(), f"o[{b}]")
+
+
+@pytest.mark.parametrize("at", [5, 40, 70, 127])
+@pytest.mark.parametrize("d", [64, 128])
+def test_gqa_largest_weight_of_the_first_tile_is_exact(d, at):
+    """One token of 128 outweighs each other one 128.5 times, a ratio halfway
+    between two bf16 values.  The exponent base is the maximum of the first
+    tile, wherever in it that lies: the large weight is 1 and the small ones
+    1/128.5, which bf16 holds to 1.6e-5.  (Over a base of 1 the large weight would
+    be 128, and the output 2e-3 off.)  Values +1 and -1: o = (128.5 - 127) /
+    (128.5 + 127), each weight's error halved."""
+    k = torch.zeros(1, 128, d, dtype=torch.bfloat16)
+    v = torch.full((1, 128, d), -1.0, dtype=torch.bfloat16)
+    q = torch.zeros(1, 1, 1, d, dtype=torch.bfloat16)
+    k[0, at, d // 2 - 1] = q[0, 0, 0, d // 2 - 1] = 1.0  # a pair that a base of 1e30 does not turn
+    v[0, at] = 1.0
+    dims = abi.GqaDims(1, 1, d, float(np.log(128.5)), 0, 1e30)
+    step = abi.GqaStep(dims, abi.Cache(v.cuda(), k.cuda(), 128), 1, 1, 128)
+    o = step(q.cuda(), torch.tensor([128], dtype=torch.int32, device="cuda"))
+    assert abi.check_status() == abi.MLA_OK
+    assert (o.double() - 1.5 / 255.5).abs().max().item() <= 2e-5
