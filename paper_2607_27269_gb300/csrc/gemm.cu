@@ -581,21 +581,17 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 :
                 const int rows = m64 ? min(16, min(RT, p.M - m0) - q * 16) : min(RT, p.M - m0) - q * 32;
                 proj_epilogue<BN>(p, pe, t_lane, stage, lane, me, rows);
             } else {
-                const bool vec = p.ldc % 8 == 0;  // 16-byte stores
+                // rows of C that are not whole 16 bytes: element by element
                 uint16_t *crow = i < RT && me < p.M ? static_cast<uint16_t *>(p.C) + phys_row(p, g, me) * p.ldc : nullptr;
                 drain_tile<BN>(t_lane, stage, lane, [&](int col) {
-                    const int n = n0 + col;
-                    const bool full = vec && n + 8 <= p.N;
-                    const int left = full ? 0 : p.N - n;  // columns to store one by one
+                    const int n = n0 + col, left = p.N - n;
                     return [=](int r, const uint4 &v) {
                         uint16_t *row = shfl_ptr(crow, r);
-                        store16_if(row && full, row + n, v);
-                        if (row && left > 0) {
-                            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                        if (!row) return;
+                        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                            for (int e = 0; e < 8; ++e)
-                                if (e < left) row[n + e] = static_cast<uint16_t>(w[e / 2] >> (16 * (e % 2)));
-                        }
+                        for (int e = 0; e < 8; ++e)
+                            if (e < left) row[n + e] = static_cast<uint16_t>(w[e / 2] >> (16 * (e % 2)));
                     };
                 });
             }
@@ -651,7 +647,7 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 :
         // a CTA leaves once every copy from its shared memory has landed
         asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
         if (got && !fail) {
-            const int q4 = cw / 4;  // 4, 8, 16 or 32: the 128 threads keep their columns and step 128 / q4 rows
+            const int q4 = cw / 4;  // 4, 8 or 16: the 128 threads keep their columns and step 128 / q4 rows
             const float4 *own = reinterpret_cast<const float4 *>(smem), *recv = reinterpret_cast<const float4 *>(smem + p.recv_off);
             const int ce = (tid - 64) % q4, n = n0 + kz * cw + 4 * ce;
 #pragma unroll 2
@@ -837,12 +833,23 @@ cudaError_t take_kernel(K *kernel)
     return allow_smem<Kernel>(1024 + kRingBytes);
 }
 
-template <int BN, bool NMAJ, bool AF32, bool SPLIT>
-cudaError_t gemm_kernel(int rt, GemmKernel *kernel)
+// The kernel for tiles of rt rows.  split_of() splits neither the absorption
+// (NMAJ: at most four K chunks) nor an fp32 A in tiles past 64 rows.
+template <int BN, bool NMAJ, bool AF32>
+cudaError_t gemm_kernel(int rt, bool split, GemmKernel *kernel)
 {
-    if (rt <= kM64Rows) return take_kernel<gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, true>>(kernel);
-    if (AF32 && rt <= kShortRows) return take_kernel<gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, SPLIT, false>>(kernel);
-    return take_kernel<gemm_tc_kernel<BN, NMAJ, AF32, false, false, SPLIT, false>>(kernel);
+    const bool m64 = rt <= kM64Rows;
+    if (split) {
+        if constexpr (!NMAJ) {
+            if (m64) return take_kernel<gemm_tc_kernel<BN, false, AF32, false, AF32, true, true>>(kernel);
+            if constexpr (!AF32) return take_kernel<gemm_tc_kernel<BN, false, false, false, false, true, false>>(kernel);
+        }
+        return cudaErrorInvalidConfiguration;
+    }
+    if (m64) return take_kernel<gemm_tc_kernel<BN, NMAJ, AF32, false, AF32, false, true>>(kernel);
+    if constexpr (AF32)
+        if (rt <= kShortRows) return take_kernel<gemm_tc_kernel<BN, NMAJ, AF32, false, true, false, false>>(kernel);
+    return take_kernel<gemm_tc_kernel<BN, NMAJ, AF32, false, false, false, false>>(kernel);
 }
 
 template <int BN, bool NMAJ, bool AF32>
@@ -905,8 +912,7 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     const size_t stage = q.tma_out ? BN * 256 : kDrainBytes;  // the results' staging
     if (smem < 1024 + stage) smem = 1024 + stage;
     GemmKernel kernel;
-    e = ks > 1 ? gemm_kernel<BN, NMAJ, AF32, true>(rt, &kernel) : gemm_kernel<BN, NMAJ, AF32, false>(rt, &kernel);
-    if (e != cudaSuccess) return e;
+    if ((e = gemm_kernel<BN, NMAJ, AF32>(rt, ks > 1, &kernel)) != cudaSuccess) return e;
     const int threads = AF32 && ks == 1 && !pairs ? kConvThreads : kGemmThreads;
     dim3 grid(mtiles * ks, ntiles, p.G);
     ProjEpi none{};

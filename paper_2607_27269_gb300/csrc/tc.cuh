@@ -133,14 +133,6 @@ __device__ __forceinline__ void commit_elect(uint32_t mbar)
         : "memory");
 }
 
-// Arrive once on the mbarrier when every MMA this thread issued so far has
-// completed (and its smem operands may be overwritten).
-__device__ __forceinline__ void commit(uint32_t mbar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
-                 : "memory");
-}
-
 __device__ __forceinline__ void wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
