@@ -698,6 +698,14 @@ cudaError_t get_encoder()
     return cudaSuccess;
 }
 
+int sm_count()
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms > 0 ? sms : 1;
+}
+
 // A: (K, head in group, group, row block) with the row mapping's strides.
 bool encode_a(const GroupGemm &p, int rblk, bool f32, CUtensorMap *ma)
 {
@@ -758,13 +766,13 @@ int rows_per_tile(const GroupGemm &p)
 // the SMs (a mid-size batch against a wide weight): split K as well, one CTA per
 // SM, at least eight chunks per share.  (Not for an fp32 A: there the reduction
 // cost as much as the split saved.)
-int split_of(bool f32, int rt, int64_t tiles, int nk)
+int split_of(bool f32, int rt, int64_t tiles, int nk, int sms)
 {
     int ks = 1;
     if (rt <= 64 && nk >= 8)
-        while (ks < 4 && tiles * ks * 2 <= (f32 ? 152 : 2 * 152) && nk >= 4 * ks) ks *= 2;
+        while (ks < 4 && tiles * ks * 2 <= (f32 ? sms : 2 * sms) && nk >= 4 * ks) ks *= 2;
     if (rt > 64 && !f32 && nk >= 16)
-        while (ks < 4 && tiles * ks * 2 <= 152 && nk >= 8 * ks) ks *= 2;
+        while (ks < 4 && tiles * ks * 2 <= sms && nk >= 8 * ks) ks *= 2;
     return ks;
 }
 
@@ -775,12 +783,12 @@ int split_of(bool f32, int rt, int64_t tiles, int nk)
 // columns: 64 rows 12.6 and 11.2 us, 128 rows 13.9 and 12.6, 160 rows 13.3 and
 // 13.7, 320 rows 17.3 and 14.9, 512 rows 20.9 and 17.9, 640 rows (two waves of
 // 64) 21.7 and more.
-int64_t tile_cost(const GroupGemm &p, int bn)
+int64_t tile_cost(const GroupGemm &p, int bn, int sms)
 {
     const int rt = rows_per_tile(p) * p.hpg, nk = (p.K + 63) / 64;
     const int64_t tiles = static_cast<int64_t>((p.M + rt - 1) / rt) * ((p.N + bn - 1) / bn) * p.G;
-    const int ks = split_of(false, rt, tiles, nk);
-    const int64_t slots = ks > 1 && rt <= 64 ? 2 * 152 : 152;
+    const int ks = split_of(false, rt, tiles, nk, sms);
+    const int64_t slots = ks > 1 && rt <= 64 ? 2 * sms : sms;
     const int64_t in = static_cast<int64_t>((nk + ks - 1) / ks) * (rt + bn) * 128;
     const int64_t exchange = ks > 1 ? 4 * 4 * static_cast<int64_t>(rt) * bn + 150 * 1024 : 0;
     return (tiles * ks + slots - 1) / slots * (in + exchange);
@@ -853,7 +861,7 @@ cudaError_t gemm_kernel(int rt, bool split, GemmKernel *kernel)
 }
 
 template <int BN, bool NMAJ, bool AF32>
-cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope = nullptr)
+cudaError_t launch_tc(const GroupGemm &p, int sms, cudaStream_t st, const ProjEpi *rope = nullptr)
 {
     cudaError_t e = get_encoder();
     if (e != cudaSuccess) return e;
@@ -871,9 +879,9 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     // in tiles as short as still leave one wave.  640 rows of 32 heads, 12.2 us
     // with 160 tiles of 128 rows and a ring of two chunks, 10.6 with 304 of 68
     // and four.
-    const bool pairs = AF32 && tiles_for(rblk) > 152;
+    const bool pairs = AF32 && tiles_for(rblk) > sms;
     if (pairs) {
-        const int64_t n = 2 * 152 / (static_cast<int64_t>(ntiles) * p.G), blocks = p.M / p.hpg;
+        const int64_t n = 2 * sms / (static_cast<int64_t>(ntiles) * p.G), blocks = p.M / p.hpg;
         if (n * rblk >= blocks) rblk = static_cast<int>((blocks + n - 1) / n);
     }
     CUtensorMap ma, mb;
@@ -892,7 +900,7 @@ cudaError_t launch_tc(const GroupGemm &p, cudaStream_t st, const ProjEpi *rope =
     const int rt = rblk * p.hpg;
     const int mtiles = (p.M + rt - 1) / rt;
     const int64_t tiles = static_cast<int64_t>(mtiles) * ntiles * p.G;
-    const int ks = split_of(AF32, rt, tiles, nk);
+    const int ks = split_of(AF32, rt, tiles, nk, sms);
     // Split K: the partial's staging lies in the ring, what the cluster sends
     // behind it (at most 66 KB each).  A short tile's ring leaves room for a
     // second CTA.
@@ -1004,7 +1012,8 @@ cudaError_t launch_absorb_gemm(const GroupGemm &p, const mla_dims &d, const void
     r.style = d.rope_style;
     r.turns = rope_turns(d.d_rope, d.rope_base);
     const bool narrow = p.N <= 64 || p.M <= 32;
-    return narrow ? launch_tc<64, true, false>(p, st, &r) : launch_tc<128, true, false>(p, st, &r);
+    const int sms = sm_count();
+    return narrow ? launch_tc<64, true, false>(p, sms, st, &r) : launch_tc<128, true, false>(p, sms, st, &r);
 }
 
 cudaError_t launch_group_gemm(const GroupGemm &p, cudaStream_t st)
@@ -1012,9 +1021,10 @@ cudaError_t launch_group_gemm(const GroupGemm &p, cudaStream_t st)
     if (p.M <= 0 || p.N <= 0 || p.G <= 0) return cudaSuccess;
     // column tile: 64 for narrow outputs and for few rows (more CTAs stream the
     // weight), else 128 -- or, of a bf16 A, what costs a CTA less
-    const bool narrow = p.N <= 64 || p.M <= 32 || (!p.a_f32 && tile_cost(p, 64) < tile_cost(p, 128));
-    if (p.a_f32) return narrow ? launch_tc<64, false, true>(p, st) : launch_tc<128, false, true>(p, st);
-    return narrow ? launch_tc<64, false, false>(p, st) : launch_tc<128, false, false>(p, st);
+    const int sms = sm_count();
+    const bool narrow = p.N <= 64 || p.M <= 32 || (!p.a_f32 && tile_cost(p, 64, sms) < tile_cost(p, 128, sms));
+    if (p.a_f32) return narrow ? launch_tc<64, false, true>(p, sms, st) : launch_tc<128, false, true>(p, sms, st);
+    return narrow ? launch_tc<64, false, false>(p, sms, st) : launch_tc<128, false, false>(p, sms, st);
 }
 
 cudaError_t launch_project(const mla_dims &d, const CacheView &c, int batch, int n_new, const void *h,
@@ -1028,10 +1038,7 @@ cudaError_t launch_project(const mla_dims &d, const CacheView &c, int batch, int
     // bytes per column; of equal ones the narrowest.  640 rows of the
     // Llama-3.2-1B shape (4672 columns): 64, 128, 192 and 256 columns take 3 x
     // 24, 2 x 32, 1 x 40 and 1 x 48 KB; 160 rows 1 x 24 with 64 columns.
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (sms <= 0) sms = 1;
+    const int sms = sm_count();
     const int nq = w_q ? d.num_heads * (d.d_nope + d.d_rope) : 0;
     const int64_t mt = (static_cast<int64_t>(batch) * n_new + 127) / 128;
     int bn = 64;
