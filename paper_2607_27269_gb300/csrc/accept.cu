@@ -156,7 +156,8 @@ __device__ __forceinline__ float warp_reduce(float v, Op op)
 
 constexpr int kRowThreads = 256;
 constexpr int kRowCtas = 3;        // per SM
-constexpr int kRowUnroll = 2;      // vectors per tensor in a group
+constexpr int kRowUnroll = 2;      // vectors per tensor and thread in a group
+constexpr int kGroup = kRowThreads * kRowUnroll;  // vectors per tensor in a group
 constexpr int kMaxCluster = 8;
 constexpr float kLowest = -2e38f;  // stands in for a maximum of -inf (or the type's lowest) as the exponents' base
 constexpr float kRaise = 16.f;     // a base is raised once a logit passes it by this much
@@ -276,7 +277,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtas) accept_row_kernel(int r
                                                                 int32_t *greedy, int C)
 {
     static_assert(kMaxCluster * kRowThreads / 32 <= 64, "a warp merges the cluster's statistics two per lane");
-    constexpr int VN = Vec<T>::n, kWarps = kRowThreads / 32, U = kRowUnroll, kGroup = kRowThreads * U;
+    constexpr int VN = Vec<T>::n, kWarps = kRowThreads / 32, U = kRowUnroll;
     __shared__ Stat s_stat[2][2][kMaxCluster * kWarps];  // [row parity][draft, target][rank, warp]
     __shared__ float s_part[2][kMaxCluster * kWarps];    // rank 0's copy is read
     __shared__ Stat s_final[2];                 // warp 0 of rank 0: the row's statistics until its results are written
@@ -476,28 +477,40 @@ template <typename T>
 cudaError_t launch_typed(int rows, int vocab, const void *draft, const void *target, int64_t stride, float *alpha,
                         int32_t *argmax_d, int32_t *argmax_t, int32_t *greedy, cudaStream_t st)
 {
-    // The cluster size with the least time by a model of what was measured: a
-    // wave of rows takes each CTA its share of a row, at 28 GB/s alone and a
-    // third of 33 GB/s with three CTAs on its SM, and 2 us of latency; of equal
-    // ones the largest.  (640 rows of 128256 bf16 with C = 1, 2, 3, 4, 6, 8:
-    // 98.7, 78.3, 101.2, 78.7, 93.8, 102.3 us; 160 rows 33.2, 25.3, 32.1, 28.3,
-    // 30.7, 31.5; 40 rows of 151936 fp32 46.9, 26.8, 20.5, 18.2, 17.2, 15.3.)
-    constexpr double kAlone = 28e3, kPerSm = 33e3, kRowCost = 2.0;  // bytes per us, bytes per us, us
+    // The cluster size with the least time by a model fitted to 440 shapes (2 to
+    // 1200 rows of 1000 to 262144 logits, both types) in each of the eight sizes;
+    // its choice takes 0.6 % longer than the best of them on average.  A wave of
+    // rows costs its latency (more in clusters, and with more CTAs an SM), the
+    // pairs of groups a CTA folds (whole ones: padding costs like logits), and what
+    // its rows, both passes of them between L2 and memory, take past the L2's
+    // size.  In more than two waves clusters of 3 and 5 run 10 to 25 % behind the
+    // model: they fill the SMs unevenly.  (A model of bytes alone took 7 CTAs a
+    // row for 480 rows of 32000, 34 us against 20 with one, and two for 640 rows of
+    // 128256 fp32, 164 us against 135 with six.)
+    const bool f32 = sizeof(T) == 4;
+    const double group = f32 ? 0.47 : 1.14, shared = f32 ? 0.02 : 0.18;
+    const int sms = row_clusters<T>(1) / kRowCtas > 0 ? row_clusters<T>(1) / kRowCtas : 1;
     double best = 0;
     int C = 0, n_cl = 0;
     const int forced = tuning().accept_cluster;  // testing aid: 1 .. 8 CTAs a cluster
     for (int c = 1; c <= kMaxCluster; ++c) {
-        if (forced >= 1 && forced <= kMaxCluster && c != forced) continue;
+        const bool force = forced >= 1 && forced <= kMaxCluster;
+        if (force && c != forced) continue;
         const int n = row_clusters<T>(c);
         if (n <= 0) continue;
-        const int live = rows < n ? rows : n;
-        const double load = live * c / static_cast<double>(row_clusters<T>(1)) * kRowCtas;  // CTAs per SM
-        const double rate = load * kAlone > kPerSm ? kPerSm / load : kAlone;
-        const double us = ((rows + n - 1) / n) * (2.0 * vocab * sizeof(T) / (c * rate) + kRowCost);
-        if (C == 0 || us < best * 1.001) {
+        if (!force && (c == 3 || c == 5) && rows > 2 * n) continue;
+        const int share = (vocab / Vec<T>::n + c - 1) / c, pairs = (share + 2 * kGroup - 1) / (2 * kGroup);
+        auto wave = [&](int live) {
+            const double load = static_cast<double>(live) * c / sms, mb = 2e-6 * live * vocab * sizeof(T);
+            const double most = load > 2 ? 3 : load > 1 ? 2 : 1;  // CTAs on an SM
+            return (c == 1 ? 0.95 : 1.54) + (load > 1 ? 0.18 + 0.62 * (load < 2 ? load - 1 : 1) : 0) +
+                   pairs * (group > most * shared ? group : most * shared) + 0.088 * mb * (mb < 230 ? mb / 230 : 1);
+        };
+        const double us = rows / n * wave(n) + (rows % n ? wave(rows % n) : 0);
+        if (C == 0 || us < best) {
             best = us;
             C = c;
-            n_cl = live;
+            n_cl = rows < n ? rows : n;
         }
     }
     if (C == 0) return cudaErrorInvalidConfiguration;

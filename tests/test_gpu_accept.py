@@ -174,3 +174,33 @@ def test_acceptance_every_cluster_size(cluster, dtype, tuning):
         t[r[1::2], at[1::2, 0]] = 12.0
         ref = check(d, t)
         assert 0 < ref["greedy"].mean() < 1
+
+
+@pytest.mark.parametrize("rows,vocab,dtype", [(512, 32000, torch.bfloat16), (560, 50257, torch.float32),
+                                              (640, 128256, torch.float32)])
+def test_acceptance_cluster_choice(rows, vocab, dtype, tuning):
+    """The size that the launcher picks is near the fastest of the eight where
+    they differ most (waves that the rows do not fill; rows past the L2's size).
+    The model is within a few percent; the bar leaves room for other load on the
+    GPU, and the worst sizes take two to three times the best one's time."""
+    target = torch.randn(rows, (vocab + 7) // 8 * 8, device="cuda")
+    draft = (target + torch.randn_like(target)).to(dtype)[:, :vocab]
+    target = target.to(dtype)[:, :vocab]
+    out = [torch.empty(rows, dtype=t, device="cuda") for t in (torch.float32,) + 3 * (torch.int32,)]
+
+    def us(size):
+        tuning(GBMLA_ACCEPT_CLUSTER=size)
+        times = []
+        for _ in range(5):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            torch.cuda.synchronize()
+            a.record()
+            for _ in range(20):
+                abi.acceptance_stats(draft, target, *out)
+            b.record()
+            b.synchronize()
+            times.append(a.elapsed_time(b) * 50)
+        return min(times)
+
+    picked, each = us(0), [us(size) for size in range(1, 9)]
+    assert picked <= 1.25 * min(each), (picked, each)
