@@ -445,8 +445,7 @@ mla_status gqa_as_mla(const mla_gqa_dims *g, mla_dims *d)
 // time, each shared by the row groups, and no more than there are tiles.
 int64_t gqa_most_splits(const mla_gqa_dims *g, int batch, int q_len, int max_kv_len, int sms)
 {
-    const int64_t s = static_cast<int64_t>(sms) * kGqaPartsPerSm /
-                      gqa_row_groups(q_len * (g->num_heads / g->num_kv_groups), g->head_dim);
+    const int64_t s = sms / gqa_row_groups(q_len * (g->num_heads / g->num_kv_groups), g->head_dim) * kGqaPartsPerSm;
     const int64_t tiles = static_cast<int64_t>(batch) * g->num_kv_groups * ((max_kv_len + MLA_SPLIT_TILE - 1) / MLA_SPLIT_TILE);
     return s < 1 || tiles < 1 ? 1 : s < tiles ? s : tiles;
 }

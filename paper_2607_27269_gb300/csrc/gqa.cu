@@ -533,8 +533,11 @@ cudaError_t launch_dn(const GqaLaunch &g, int row_groups, cudaStream_t st)
     a.turns = rope_turns(D, g.rope_base);
     constexpr size_t smem = 1024 + static_cast<size_t>(kWarps) * kStages * kStageBytes;
     if ((e = allow_smem<gqa_attn_kernel<D, N>>(smem)) != cudaSuccess) return e;
-    // the partitions over the SMs' blocks first, then over each block's warps
-    const int per_group = (g.sms + row_groups - 1) / row_groups;
+    // the partitions over the SMs' blocks first, then over each block's warps.
+    // All row groups' blocks run at a time, one an SM: with a block more than there
+    // are SMs (3 groups of 51 on 152) it waits for a whole block to end, 28 rows
+    // in 3 groups 19.4 us instead of 13.4.
+    const int per_group = g.sms > row_groups ? g.sms / row_groups : 1;
     int grid = g.num_splits < per_group ? g.num_splits : per_group;
     if (g.num_splits > grid * kWarps) grid = (g.num_splits + kWarps - 1) / kWarps;
     return launch_dependent(gqa_attn_kernel<D, N>, dim3(grid, row_groups, 1), dim3(32 * kWarps), smem, st, 1, a, mk,
