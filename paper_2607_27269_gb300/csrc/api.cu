@@ -153,6 +153,7 @@ void read_tuning()
     const char *tq = getenv("GBMLA_TC_QUERY");
     t.tc_query = !tq ? 0 : strcmp(tq, "resident") == 0 ? 1 : strcmp(tq, "streamed") == 0 ? 2 : 0;
     t.accept_cluster = env_int("GBMLA_ACCEPT_CLUSTER");
+    t.gqa_rows = env_int("GBMLA_GQA_ROWS") & ~7;
     std::lock_guard<std::mutex> lock(g_mutex);
     g_tuning = t;
 }

@@ -574,7 +574,22 @@ cudaError_t launch_gqa_attn(const GqaLaunch &g, cudaStream_t st)
     if (g.batch <= 0) return cudaSuccess;
     const int rows = g.q_len * g.hpg;
     if (rows > 128) return cudaErrorInvalidConfiguration;
-    const int groups = gqa_row_groups(rows, g.head_dim);
+    // Rows a warp: as few as leave all row groups' partitions a warp of the SMs at
+    // a time (they read the cache again, from L2).  Few partitions otherwise
+    // leave the SMs to a handful of long chains: 28 rows of one sequence of 2000
+    // tokens 13.8 us in one group, 7.9 in four of 8 rows; 56 rows of eight of 1000
+    // 15.4 in two, 10.3 in seven; 32 rows in 512 partitions 17.7, 14.9 in two of 16.
+    const int fewest = gqa_row_groups(rows, g.head_dim);
+    int groups = fewest;
+    const int forced = tuning().gqa_rows;  // testing aid: most rows a warp
+    for (int most = forced > 0 ? forced : 8; most <= 24; most += 8) {
+        const int more = (rows + most - 1) / most;
+        if (more <= fewest) break;
+        if (forced > 0 || g.num_splits <= g.sms / more * kWarps) {
+            groups = more;
+            break;
+        }
+    }
     const int n = ((rows + groups - 1) / groups + 7) / 8 * 8;
     if (g.head_dim == 64) return launch_d<64>(g, groups, n, st);
     if (g.head_dim == 128) return launch_d<128>(g, groups, n, st);

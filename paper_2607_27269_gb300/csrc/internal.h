@@ -65,7 +65,7 @@ cudaError_t launch_attn_simt(const AttnArgs &a, cudaStream_t st);
 // 80-row tensor-core CTA in shared memory or streams them with the cache
 // chunks.  0 means "not set".  They change tiling only.
 struct Tuning {
-    int attn_simt, tc_max_rows, tc_max_slots, tc_pv_slots, absorb_path, tc_query, accept_cluster;
+    int attn_simt, tc_max_rows, tc_max_slots, tc_pv_slots, absorb_path, tc_query, accept_cluster, gqa_rows;
 };
 const Tuning &tuning();
 void reload_tuning();

@@ -108,9 +108,24 @@ def test_gqa_split_counts_and_paged(splits):
     (6, 4, 128, True, 0), (5, 5, 128, False, 0), (8, 4, 64, True, 1), (11, 3, 64, False, 0), (8, 6, 128, False, 1),
     (7, 8, 64, True, 0), (8, 16, 64, False, 0), (8, 16, 128, True, 0)])
 def test_gqa_row_counts_and_stage_tails(hpg, q_len, d, paged, style):
-    """Query rows from 1 to 128 (every width of the kernel's row blocks, one
-    to six row groups) against units that end around every load stage and tile
+    """Query rows from 1 to 128 (one to thirteen row groups of 8 or 16 rows, as
+    so few tiles take) against units that end around every load stage and tile
     boundary; rows past a unit's end hold NaN and must not reach an output."""
+    check_row_counts_and_stage_tails(hpg, q_len, d, paged, style)
+
+
+@pytest.mark.parametrize("width", [8, 16, 24, 32])
+@pytest.mark.parametrize("hpg,q_len,d,paged,style", [
+    (3, 3, 64, True, 0), (5, 5, 64, False, 1), (6, 4, 128, True, 0), (5, 5, 128, False, 0), (8, 4, 64, True, 1),
+    (8, 6, 128, False, 1), (7, 8, 64, True, 0), (8, 16, 64, False, 0), (8, 16, 128, True, 0)])
+def test_gqa_row_widths(hpg, q_len, d, paged, style, width, tuning):
+    """The same with warps of up to 8, 16, 24 and 32 rows (24 at most at width
+    128), which batches of many tiles take."""
+    tuning(GBMLA_GQA_ROWS=width)
+    check_row_counts_and_stage_tails(hpg, q_len, d, paged, style)
+
+
+def check_row_counts_and_stage_tails(hpg, q_len, d, paged, style):
     lens = [1, 31, 32, 33, 63, 64, 65, 96, 127, 128, 129, 192, 300]
     G, B = 2, len(lens)
     shape = wl.Shape("rows", B, hpg * G, G, d, 64, d, 128, 0, q_len, 300, 300, paged=paged, rope_style=style)
