@@ -477,34 +477,35 @@ template <typename T>
 cudaError_t launch_typed(int rows, int vocab, const void *draft, const void *target, int64_t stride, float *alpha,
                         int32_t *argmax_d, int32_t *argmax_t, int32_t *greedy, cudaStream_t st)
 {
-    // The cluster size with the least time by a model fitted to 440 shapes (2 to
-    // 1200 rows of 1000 to 262144 logits, both types) in each of the eight sizes;
-    // its choice takes 0.6 % longer than the best of them on average.  A wave of
-    // rows costs its latency (more in clusters, and with more CTAs an SM), the
-    // pairs of groups a CTA folds (whole ones: padding costs like logits), and what
-    // its rows, both passes of them between L2 and memory, take past the L2's
-    // size.  In more than two waves clusters of 3 and 5 run 10 to 25 % behind the
-    // model: they fill the SMs unevenly.  (A model of bytes alone took 7 CTAs a
-    // row for 480 rows of 32000, 34 us against 20 with one, and two for 640 rows of
+    // The cluster size with the least time by a model fitted to 950 measurements
+    // (2 to 1200 rows of 1000 to 262144 logits, both types, from L2 and from
+    // memory) of each of the eight sizes; its choice takes 1 % longer than the best
+    // of them on average, 25 % at most.  A wave of rows costs its latency (more in
+    // clusters, and with more CTAs an SM), the pairs of groups a CTA folds (mostly
+    // whole ones: padding costs like logits), and what its rows, past the L2's
+    // size, take to come from memory twice.  Of clusters of 3 and 5 a few less run
+    // at a time than the device says (142 of 148, 82 of 87); those left over would
+    // begin when the others have ended.  (A model of bytes alone took 7 CTAs a row
+    // for 480 rows of 32000 bf16, 34 us against 20 with one, and two for 640 rows of
     // 128256 fp32, 164 us against 135 with six.)
     const bool f32 = sizeof(T) == 4;
-    const double group = f32 ? 0.47 : 1.14, shared = f32 ? 0.02 : 0.18;
+    const double group = f32 ? 0.685 : 1.14, shared = f32 ? 0.016 : 0.282;  // a pair; a pair times the CTAs on the SM
     const int sms = row_clusters<T>(1) / kRowCtas > 0 ? row_clusters<T>(1) / kRowCtas : 1;
     double best = 0;
     int C = 0, n_cl = 0;
     const int forced = tuning().accept_cluster;  // testing aid: 1 .. 8 CTAs a cluster
     for (int c = 1; c <= kMaxCluster; ++c) {
-        const bool force = forced >= 1 && forced <= kMaxCluster;
-        if (force && c != forced) continue;
-        const int n = row_clusters<T>(c);
+        if (forced >= 1 && forced <= kMaxCluster && c != forced) continue;
+        int n = row_clusters<T>(c);
         if (n <= 0) continue;
-        if (!force && (c == 3 || c == 5) && rows > 2 * n) continue;
-        const int share = (vocab / Vec<T>::n + c - 1) / c, pairs = (share + 2 * kGroup - 1) / (2 * kGroup);
+        if (c == 3 || c == 5) n -= n / 16;
+        const int nvec = vocab / Vec<T>::n, share = (nvec + c - 1) / c;
+        const double pairs = 0.91 * ((share + 2 * kGroup - 1) / (2 * kGroup)) + 0.09 * nvec / (2.0 * kGroup * c);
         auto wave = [&](int live) {
             const double load = static_cast<double>(live) * c / sms, mb = 2e-6 * live * vocab * sizeof(T);
             const double most = load > 2 ? 3 : load > 1 ? 2 : 1;  // CTAs on an SM
-            return (c == 1 ? 0.95 : 1.54) + (load > 1 ? 0.18 + 0.62 * (load < 2 ? load - 1 : 1) : 0) +
-                   pairs * (group > most * shared ? group : most * shared) + 0.088 * mb * (mb < 230 ? mb / 230 : 1);
+            return (c == 1 ? 0.234 : 0.925) + (load > 1 ? 0.368 + 0.868 * (load < 2 ? load - 1 : 1) : 0) +
+                   pairs * (group > most * shared ? group : most * shared) + 0.108 * mb * (mb < 313 ? mb / 313 : 1);
         };
         const double us = rows / n * wave(n) + (rows % n ? wave(rows % n) : 0);
         if (C == 0 || us < best) {
