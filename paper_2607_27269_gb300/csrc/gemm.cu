@@ -89,6 +89,14 @@ __device__ __forceinline__ void store16_if(bool ok, uint16_t *dst, const uint4 &
                  : "memory");
 }
 
+// the same with 8 bytes
+__device__ __forceinline__ void store8_if(bool ok, uint16_t *dst, uint32_t x, uint32_t y)
+{
+    asm volatile("{.reg .pred p; setp.ne.u32 p, %0, 0; @p st.global.v2.b32 [%1], {%2, %3};}" ::"r"(static_cast<uint32_t>(ok)),
+                 "l"(dst), "r"(x), "r"(y)
+                 : "memory");
+}
+
 template <int BN, class Store>
 __device__ __forceinline__ void drain_tile(uint32_t t_lane, unsigned char *stage, int lane, Store store)
 {
@@ -581,17 +589,24 @@ __global__ void __launch_bounds__(AF32 ? kConvThreads : kGemmThreads, PROJ ? 0 :
                 const int rows = m64 ? min(16, min(RT, p.M - m0) - q * 16) : min(RT, p.M - m0) - q * 32;
                 proj_epilogue<BN>(p, pe, t_lane, stage, lane, me, rows);
             } else {
-                // rows of C that are not whole 16 bytes: element by element
+                // rows of C that are not whole 16 bytes: 8 bytes a store where they
+                // are whole 8, else (and at the last columns) element by element
+                const bool eight = p.ldc % 4 == 0;
                 uint16_t *crow = i < RT && me < p.M ? static_cast<uint16_t *>(p.C) + phys_row(p, g, me) * p.ldc : nullptr;
                 drain_tile<BN>(t_lane, stage, lane, [&](int col) {
-                    const int n = n0 + col, left = p.N - n;
+                    const int n = n0 + col;
+                    const bool full = eight && n + 8 <= p.N;
+                    const int left = full ? 0 : p.N - n;  // columns to store one by one
                     return [=](int r, const uint4 &v) {
                         uint16_t *row = shfl_ptr(crow, r);
-                        if (!row) return;
-                        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                        store8_if(row && full, row + n, v.x, v.y);
+                        store8_if(row && full, row + n + 4, v.z, v.w);
+                        if (row && left > 0) {
+                            const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
-                        for (int e = 0; e < 8; ++e)
-                            if (e < left) row[n + e] = static_cast<uint16_t>(w[e / 2] >> (16 * (e % 2)));
+                            for (int e = 0; e < 8; ++e)
+                                if (e < left) row[n + e] = static_cast<uint16_t>(w[e / 2] >> (16 * (e % 2)));
+                        }
                     };
                 });
             }
