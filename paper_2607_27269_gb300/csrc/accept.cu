@@ -5,21 +5,23 @@
 //
 // A context's two rows go to one cluster of C CTAs (1 .. 8), which takes two
 // passes over them: maxima, sums of exponentials and argmaxes (from HBM, the
-// lines marked evict-last), then the overlap (from L2).  Exponentials are base
-// 2 with log2(e) folded into one FMA, and pass 2 folds the normaliser into the
-// exponent, p = 2^(x log2 e - c) with c = m log2 e + log2 Z, so that
-// min(p_D, p_T) = 2^min(., .) costs one exponential per token, not two.
+// lines marked evict-last), then the overlap (from L2, as far as it holds the
+// rows between their passes: 228 rows of 128256 bf16 are 117 MB, and 1.2 times
+// the logits come from memory).  Exponentials are base 2 with log2(e) folded into
+// one FMA, and pass 2 folds the normaliser into the exponent, p = 2^(x log2 e - c)
+// with c = m log2 e + log2 Z, so that min(p_D, p_T) = 2^min(., .) costs one
+// exponential per token, not two.
 //
 // Bound: HBM (both rows once), then issue slots (about 16 per token pair over
 // both passes); between the two passes of a row stand reductions and a cluster
 // barrier, some 2 us that only other CTAs' work can hide.  So three CTAs of
-// 256 threads share an SM, and C is chosen so that the rows fill the GPU in
-// whole waves.  640 rows of 128256 bf16: 109.2 us with one CTA of 512 threads
-// per row (304 at a time: a third wave of 32 rows, and the lines of 304 rows
-// past the L2's 129 MB), 78.4 us so; 40 rows of 151936 fp32: 35.4 us with the
-// slices resident in shared memory (320 CTAs of 152 KB, three waves), 15.3 us
-// so; 2 rows of 128256 bf16: 8.4 -> 6.0 us.  The sums and orders are fixed: the
-// bits do not depend on timing.
+// 256 threads share an SM, and C is chosen by a model of what that costs.  640
+// rows of 128256 bf16: 109.2 us with one CTA of 512 threads per row (304 at a
+// time: a third wave of 32 rows, and the lines of 304 rows past the L2's 129
+// MB), 78.7 us so; 40 rows of 151936 fp32: 35.4 us with the slices resident in
+// shared memory (320 CTAs of 152 KB, three waves), 14.9 us so; 2 rows of 128256
+// bf16: 8.9 -> 6.3 us.  The sums and orders are fixed: the bits do not depend on
+// timing.
 #include <math.h>
 
 #include <atomic>

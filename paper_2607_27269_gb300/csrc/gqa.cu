@@ -20,7 +20,8 @@
 // A column's running maximum, sum and accumulators sit in the same lanes, so
 // a rescale (a new maximum in a segment's first tile, later only a score that
 // passes the base by 2^8) needs no exchange.
-// More than 32 rows run as row groups (grid y) that each read the cache.
+// More rows than a warp holds (32, or 24 of width 128) run as row groups (grid y)
+// that each read the cache, as do fewer where the partitions leave warps idle.
 //
 // The first form of this kernel (one CTA per partition, tcgen05 with M = 128
 // query rows of which 20 are real, one softmax warp) took 727 us on the
@@ -535,7 +536,7 @@ cudaError_t launch_dn(const GqaLaunch &g, int row_groups, cudaStream_t st)
     if ((e = allow_smem<gqa_attn_kernel<D, N>>(smem)) != cudaSuccess) return e;
     // the partitions over the SMs' blocks first, then over each block's warps.
     // All row groups' blocks run at a time, one an SM: with a block more than there
-    // are SMs (3 groups of 51 on 152) it waits for a whole block to end, 28 rows
+    // are SMs (3 groups of 51 on 152) it waits for a whole block to end, 56 rows
     // in 3 groups 19.4 us instead of 13.4.
     const int per_group = g.sms > row_groups ? g.sms / row_groups : 1;
     int grid = g.num_splits < per_group ? g.num_splits : per_group;
@@ -577,7 +578,7 @@ cudaError_t launch_gqa_attn(const GqaLaunch &g, cudaStream_t st)
     // Rows a warp: as few as leave all row groups' partitions a warp of the SMs at
     // a time (they read the cache again, from L2).  Few partitions otherwise
     // leave the SMs to a handful of long chains: 28 rows of one sequence of 2000
-    // tokens 13.8 us in one group, 7.9 in four of 8 rows; 56 rows of eight of 1000
+    // tokens 13.8 us in one group, 8.0 in four of 8 rows; 56 rows of eight of 1000
     // 15.4 in two, 10.3 in seven; 32 rows in 512 partitions 17.7, 14.9 in two of 16.
     const int fewest = gqa_row_groups(rows, g.head_dim);
     int groups = fewest;
