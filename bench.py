@@ -733,12 +733,12 @@ def measure_projection(args, w, dws, stream, dev, l2, peaks):
 # DRAM bytes (read + write) per attention launch from one ncu capture of the
 # kernel source with this sha256 prefix (profiles/attn_tc_<workload>.md); a
 # kernel that has changed since reports null.
-TRAFFIC_SOURCE = "afb784248dad3ea5"
+TRAFFIC_SOURCE = "c5a92824da0b4d2f"
 TRAFFIC = {
-    "qwen05b_b16_h14_r256_t2048": 21207552,
-    "llama3b_long_b8_h24_r512_t16k_32k": 208548352,
-    "llama1b_paged_b128_h32_r512_t128_8192": 688454400,
-    "llama1b_chunk5_b32_h32_r512_t4096": 162208256,
+    "qwen05b_b16_h14_r256_t2048": 21208576,
+    "llama3b_long_b8_h24_r512_t16k_32k": 210178560,
+    "llama1b_paged_b128_h32_r512_t128_8192": 688888576,
+    "llama1b_chunk5_b32_h32_r512_t4096": 161851648,
 }
 
 
