@@ -289,7 +289,10 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtas) accept_row_kernel(int r
     const int share = (nvec + C - 1) / C;
     const int v_lo = min(nvec, rank * share), v_hi = min(nvec, v_lo + share);
     const int mine = v_hi - v_lo;  // the slice's vectors
-    const int pairs = (mine + 2 * kGroup - 1) / (2 * kGroup);  // of groups: two buffers take turns
+    // pairs of groups (two buffers take turns), or one group alone, which stays in
+    // its buffer for pass 2 (1000 bf16 logits: 256 rows 5.3 -> 4.4 us)
+    const bool one = mine > 0 && mine <= kGroup;
+    const int pairs = one ? 0 : (mine + 2 * kGroup - 1) / (2 * kGroup);
     const int tail = rank == C - 1 ? nvec * VN + tid : vocab;  // the row's last, partial vector: a logit per thread
     const uint64_t keep = tc::policy_evict_last(), drop = tc::policy_evict_first();
     const uint32_t none = sizeof(T) == 2 ? 0xff80ff80u : 0xff800000u;  // -inf
@@ -348,7 +351,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtas) accept_row_kernel(int r
     const T *d = draft + row * stride, *t = target + row * stride;
     Group ga, gb;
     auto vec = [&](const T *x) { return reinterpret_cast<const uint4 *>(x) + v_lo + tid; };
-    if (pairs > 0) load(vec(d), vec(t), 0, keep, ga);
+    if (mine > 0) load(vec(d), vec(t), 0, keep, ga);
     int par = 0;
     for (;; par ^= 1) {
         // ---- pass 1: maxima, sums, argmaxes
@@ -370,6 +373,7 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtas) accept_row_kernel(int r
             }
         };
         const uint4 *vd = vec(d), *vt = vec(t);
+        if (one) fold(ga, 0);
 #pragma unroll 1
         for (int k = 0; k < pairs; ++k) {
             load(vd, vt, 2 * k + 1, keep, gb);
@@ -423,6 +427,10 @@ __global__ void __launch_bounds__(kRowThreads, kRowCtas) accept_row_kernel(int r
 #pragma unroll
             for (int u = 0; u < U; ++u) acc += vec_pmin(g.d[u], g.t[u], cd, ct, T{});
         };
+        if (one) {
+            overlap(ga);
+            if (next < rows) load(vec(dn), vec(tn), 0, keep, ga);
+        }
 #pragma unroll 1
         for (int k = 0; k < pairs; ++k) {
             load(vd, vt, 2 * k + 1, drop, gb);

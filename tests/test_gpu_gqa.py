@@ -108,8 +108,8 @@ def test_gqa_split_counts_and_paged(splits):
     (6, 4, 128, True, 0), (5, 5, 128, False, 0), (8, 4, 64, True, 1), (11, 3, 64, False, 0), (8, 6, 128, False, 1),
     (7, 8, 64, True, 0), (8, 16, 64, False, 0), (8, 16, 128, True, 0)])
 def test_gqa_row_counts_and_stage_tails(hpg, q_len, d, paged, style):
-    """Query rows from 1 to 128 (one to thirteen row groups of 8 or 16 rows, as
-    so few tiles take) against units that end around every load stage and tile
+    """Query rows from 1 to 128 (one to eight row groups of 8 or 16 rows, as so
+    few tiles take) against units that end around every load stage and tile
     boundary; rows past a unit's end hold NaN and must not reach an output."""
     check_row_counts_and_stage_tails(hpg, q_len, d, paged, style)
 
