@@ -161,7 +161,11 @@ constexpr int kRowCtas = 3;        // per SM
 constexpr int kRowUnroll = 2;      // vectors per tensor and thread in a group
 constexpr int kGroup = kRowThreads * kRowUnroll;  // vectors per tensor in a group
 constexpr int kMaxCluster = 8;
-constexpr float kLowest = -2e38f;  // stands in for a maximum of -inf (or the type's lowest) as the exponents' base
+// The lowest base of the exponents: logits below it (-inf, the type's lowest, -1e30
+// and the like) are masks and weigh nothing.  A base b has x log2 e + c, c =
+// -b log2 e rounded, off by up to |b| 2^-24 at x = b: 2^86 here, which vanishes when
+// a real logit raises the base; 2^(1e22) = inf with a base of -1e30, and then NaN.
+constexpr float kLowest = -2e9f;
 constexpr float kRaise = 16.f;     // a base is raised once a logit passes it by this much
 
 // Running statistics of one thread: the exact maximum and the first vector

@@ -204,3 +204,18 @@ def test_acceptance_cluster_choice(rows, vocab, dtype, tuning):
 
     picked, each = us(0), [us(size) for size in range(1, 9)]
     assert picked <= 1.25 * min(each), (picked, each)
+
+
+@pytest.mark.parametrize("dtype", [torch.bfloat16, torch.float32])
+@pytest.mark.parametrize("mask", [-1e4, -65504.0, -1e9, -1e10, -1e20, -1e30, -1e38])
+@pytest.mark.parametrize("rows,vocab", [(15, 73), (11, 536), (40, 4096), (9, 50257)])
+def test_acceptance_finite_masks(rows, vocab, mask, dtype):
+    """Masks by a large negative number: most of a row, whole vectors and threads'
+    whole shares of it, weigh nothing, as -inf does."""
+    g = torch.Generator().manual_seed(59)
+    d = (torch.randn(rows, vocab, generator=g) * 2).to(dtype)
+    t = (torch.randn(rows, vocab, generator=g) * 2).to(dtype)
+    for share in (0.3, 0.9, 0.999):
+        out = torch.rand(rows, vocab, generator=g) < share
+        out[:, vocab // 2] = False
+        check(d.masked_fill(out, mask), t.masked_fill(out, mask))
